@@ -55,6 +55,7 @@ struct MrgParams {
   int64_t total_chunks;
   int64_t head_units;         // virtual units before `out` in the first chunk
   uint64_t stride_lo, stride_hi;  // word stride between streams
+  uint32_t m1, m2;            // the moduli, as operands the compiler does not know
   uint32_t x[6];              // state at the call's word offset
   uint32_t x1[6];             // state at the first unit of chunk 1 of stream 0
   int32_t chunk_levels;       // entries of chunk_tab (0: generic jump)
@@ -63,45 +64,72 @@ struct MrgParams {
   uint32_t stream_tab[kJumpLevels][2][9];  // A^(stride 2^k)
 };
 
-// p mod m for the products of one step (p < 2^54), folding 2^32 = c (mod m)
-// with as few 32x32 -> 64-bit products as the ranges allow (they take twice
-// the multiplier's time of a 32-bit product): m1: the high word times c1 fits
-// 32 bits, so one 32-bit product, an add whose carry out is worth c1, and a
-// conditional subtraction; m2: one wide fold (the high word times c2 needs
-// 37 bits), then the same 32-bit step.
-__device__ __forceinline__ uint32_t red_m1(uint64_t p) {
-  const uint32_t lo = (uint32_t)p;
-  const uint32_t u0 = lo + (uint32_t)(p >> 32) * mrg::C1;  // high word < 2^22: product < 2^30
-  const uint32_t u = u0 + (u0 < lo ? mrg::C1 : 0u);        // a carry out of 2^32 is worth c1
-  return u >= mrg::M1 ? u - mrg::M1 : u;
-}
-__device__ __forceinline__ uint32_t red_m2(uint64_t p) {
-  const uint64_t t = (uint64_t)(uint32_t)p + (p >> 32) * (uint64_t)mrg::C2;  // < 2^32 + 2^37
-  const uint32_t tl = (uint32_t)t;
-  const uint32_t u0 = tl + (uint32_t)(t >> 32) * mrg::C2;  // t >> 32 < 2^6: product < 2^21
-  const uint32_t u = u0 + (u0 < tl ? mrg::C2 : 0u);
-  return u >= mrg::M2 ? u - mrg::M2 : u;
-}
-
 struct MrgRegs {
   uint32_t a0, a1, a2;  // x1_{n-3}, x1_{n-2}, x1_{n-1}
   uint32_t b0, b1, b2;  // x2_{n-3}, x2_{n-2}, x2_{n-1}
 };
 
+__device__ __forceinline__ uint64_t mul_wide(uint32_t a, uint32_t b) {
+  uint64_t r;
+  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mad_wide(uint32_t a, uint32_t b, uint64_t c) {
+  uint64_t r;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+
+// lo + 2^32 (h - 1) mod m = 2^32 - c, h c < 2^32: with L = lo + h c, the
+// value is congruent to L - c.  Where the 32-bit sum carries, L - 2^32 is
+// that value mod m and below m (h c < m); where it does not, L < 2^32 makes
+// L - c < m.  So one comparison and one conditional subtraction give the
+// canonical residue, where a fold of lo + 2^32 h needs one pair for the carry
+// and one for the residue at or above m.
+template <uint32_t kC>
+__device__ __forceinline__ uint32_t fold_carry(uint32_t lo, uint32_t h) {
+  uint32_t n = lo + h * kC;
+  asm("{ .reg .pred p; setp.ge.u32 p, %0, %1; @p sub.u32 %0, %0, %2; }"
+      : "+r"(n) : "r"(lo), "n"(kC));
+  return n;
+}
+
 // One step of both components; returns z_n = (x1_n - x2_n) mod m1.
-// -a13 x = a13 (m1 - x) (mod m1) keeps the sums non-negative and below 2^54.
-__device__ __forceinline__ uint32_t mrg_next(MrgRegs& s) {
-  const uint64_t p1 = (uint64_t)mrg::A12 * s.a1 + (uint64_t)mrg::A13 * (mrg::M1 - s.a0);
-  const uint64_t p2 = (uint64_t)mrg::A21 * s.b2 + (uint64_t)mrg::A23 * (mrg::M2 - s.b0);
-  const uint32_t n1 = red_m1(p1);
-  const uint32_t n2 = red_m2(p2);
+// -a13 x = a13 (m1 - x) (mod m1) keeps the sums non-negative and below 2^54;
+// m1's sum folds at once (its high word times c1 fits 32 bits), m2's high
+// word times c2 needs 37 bits, so one wide fold goes before.
+//
+// Bound by the FMA-heavy pipe, which takes every product (a wide one about
+// 4.5 cycles per warp) and every add that the compiler issues as an IMAD; it
+// splits the adds evenly between that pipe and the ALU, so fewer instructions
+// of any kind relieve it.  Steps alone, per word and warp: 28.6 instructions
+// and 44.4 cycles with two conditional corrections per component, 22.7 and
+// 38.7 with fold_carry, 20.6 and 35.5 with the moduli read from the kernel's
+// parameters (as immediates the two subtractions cost a further instruction
+// each).  Wide products with a constant or (lo, 1) as the 64-bit addend in
+// place of the two 32-bit adds cost two moves each (23.6 instructions).  In
+// the fills: 10^9 bits 1.250 -> 0.976 ms, 16384 x 16384 FP64 gaussians
+// 2.099 -> 1.986 ms.
+__device__ __forceinline__ uint32_t mrg_next(MrgRegs& s, const MrgParams& p) {
+  const uint64_t p1 = mad_wide(p.m1 - s.a0, mrg::A13, mul_wide(s.a1, mrg::A12));
+  const uint64_t p2 = mad_wide(p.m2 - s.b0, mrg::A23, mul_wide(s.b2, mrg::A21));
+  const uint32_t n1 = fold_carry<mrg::C1>((uint32_t)p1, (uint32_t)(p1 >> 32) + 1u);
+  const uint64_t t = mul_wide((uint32_t)(p2 >> 32), mrg::C2);
+  uint32_t tl, th;  // lo(p2) + t, its high word one up (below 2^6)
+  asm("add.cc.u32 %0, %2, %3; addc.u32 %1, %4, 1;"
+      : "=r"(tl), "=r"(th)
+      : "r"((uint32_t)p2), "r"((uint32_t)t), "r"((uint32_t)(t >> 32)));
+  const uint32_t n2 = fold_carry<mrg::C2>(tl, th);
   s.a0 = s.a1;
   s.a1 = s.a2;
   s.a2 = n1;
   s.b0 = s.b1;
   s.b1 = s.b2;
   s.b2 = n2;
-  return n1 >= n2 ? n1 - n2 : n1 - n2 + mrg::M1;
+  uint32_t z = n1 - n2;  // below 0: + m1, which is - c1 in 32 bits
+  asm("{ .reg .pred p; setp.lt.u32 p, %1, %2; @p sub.u32 %0, %0, %3; }"
+      : "+r"(z) : "r"(n1), "r"(n2), "n"(mrg::C1));
+  return z;
 }
 
 // y = M x mod m with one fold per product: each product p < 2^64 becomes
@@ -164,13 +192,13 @@ __device__ __forceinline__ void jump(MrgRegs& s, uint64_t e_lo, uint64_t e_hi) {
 
 // Generates one unit's words and writes its kWpu output words to o.
 template <int V>
-__device__ __forceinline__ void gen_unit(MrgRegs& st, uint32_t* o, const TransformParams& t,
+__device__ __forceinline__ void gen_unit(MrgRegs& st, uint32_t* o, const MrgParams& p,
                                          bool odd = false) {
   constexpr int kWpu = VInfo<V>::wpu;
   uint32_t w[kWpu];
 #pragma unroll
-  for (int i = 0; i < kWpu; ++i) w[i] = mrg_next(st);
-  unit_outputs<V>(w, o, t, odd);
+  for (int i = 0; i < kWpu; ++i) w[i] = mrg_next(st, p);
+  unit_outputs<V>(w, o, p.t, odd);
 }
 
 // The 16-byte stage chunk from 4 new output words: as they are, or (carry
@@ -199,7 +227,7 @@ __device__ __forceinline__ uint4 shift_in(uint32_t* carry, const uint32_t* o4) {
 // its own carry mode when its start splits a pair (a warp's 32 chunks lie in
 // one stream, so both are warp-uniform).
 template <int V, int kMode>
-__global__ void __launch_bounds__(kThreads) mrg_fill_kernel(const MrgParams p) {
+__global__ void __launch_bounds__(kThreads) mrg_fill_kernel(const __grid_constant__ MrgParams p) {
   constexpr bool kAligned = kMode != 0;
   constexpr bool kPerStream = kMode == 3;
   constexpr int kWpu = VInfo<V>::wpu;
@@ -245,7 +273,7 @@ __global__ void __launch_bounds__(kThreads) mrg_fill_kernel(const MrgParams p) {
       // chunk 1's state is taken at the largest head (p.head_units); a stream
       // with a smaller head starts its chunks that many units later
       if (active && c > 0)
-        for (int64_t k = 0; k < (p.head_units - hu) * kWpu; ++k) mrg_next(st);
+        for (int64_t k = 0; k < (p.head_units - hu) * kWpu; ++k) mrg_next(st, p);
     }
   } else {
     st.a0 = p.x[0]; st.a1 = p.x[1]; st.a2 = p.x[2];
@@ -272,7 +300,7 @@ __global__ void __launch_bounds__(kThreads) mrg_fill_kernel(const MrgParams p) {
     uint32_t o[kWpu];
 #pragma unroll
     for (int i = 0; i < kWpu; ++i) o[i] = 0u;
-    if (active && u_first >= 0 && u_first < p.units) gen_unit<V>(st, o, p.t);
+    if (active && u_first >= 0 && u_first < p.units) gen_unit<V>(st, o, p);
 #pragma unroll
     for (int i = 0; i < kOwpe; ++i) carry[i] = o[kOwpe + i];
   }
@@ -304,7 +332,7 @@ __global__ void __launch_bounds__(kThreads) mrg_fill_kernel(const MrgParams p) {
         for (int ch = 0; ch < 8; ++ch) {
           uint32_t o4[4];
 #pragma unroll
-          for (int u = 0; u < kUpc; ++u) gen_unit<V>(st, o4 + u * kWpu, p.t, (u & 1) != 0);
+          for (int u = 0; u < kUpc; ++u) gen_unit<V>(st, o4 + u * kWpu, p, (u & 1) != 0);
           stage[warp][lane][ch ^ (lane & 7)] = kCarry ? shift_in<true, kOwpe>(carry, o4)
                                                       : shift_in<false, kOwpe>(carry, o4);
         }
@@ -314,7 +342,7 @@ __global__ void __launch_bounds__(kThreads) mrg_fill_kernel(const MrgParams p) {
 #pragma unroll
           for (int u = 0; u < kUpc; ++u) {
             const int64_t unit = ub + ch * kUpc + u;
-            if (unit >= 0 && unit < p.units) gen_unit<V>(st, o4 + u * kWpu, p.t);
+            if (unit >= 0 && unit < p.units) gen_unit<V>(st, o4 + u * kWpu, p);
           }
           stage[warp][lane][ch ^ (lane & 7)] = kCarry ? shift_in<true, kOwpe>(carry, o4)
                                                       : shift_in<false, kOwpe>(carry, o4);
@@ -433,6 +461,8 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
   p.out_words = r.n * (I::es / 4);
   p.stride_lo = r.stride_lo;
   p.stride_hi = r.stride_hi;
+  p.m1 = mrg::M1;
+  p.m2 = mrg::M2;
   for (int i = 0; i < 6; ++i) p.x[i] = r.mrg[i];
 
   const uintptr_t addr = (uintptr_t)r.out;
