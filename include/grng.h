@@ -257,7 +257,7 @@ GRNG_API grng_status grng_generate_host(const grng_distribution* dist, grng_engi
  * (1..16: a cap on the resident CTAs; 17..64: value - 16 waves of resident
  * CTAs); MRG32k3a, the threads per SM of the chunk plan in units of 256 (sets
  * the chunk length); 0 = the built-in choice (Philox: 8 waves of resident
- * CTAs; MRG32k3a: 2048 threads per SM).  Tuning is
+ * CTAs; MRG32k3a: 2048 threads per SM, 3072 for long fills).  Tuning is
  * what the paper expects of kernels written for the hardware (Sec. 8; Sec. 7
  * shows the launch configuration mattering).  Outputs never depend on the
  * geometry.  The table starts from the file named by the environment

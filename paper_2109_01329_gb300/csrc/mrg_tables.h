@@ -65,6 +65,37 @@ constexpr PowTable make_pow_table() {
   return t;
 }
 
+// A^(k 2^(5 d)) for the 26 radix-32 digits d of a 128-bit exponent and
+// k = 0..31 (k = 0 the identity): words 0..8 of a row are A1's power, 12..20
+// A2's, row-major, so that each is a run of 16-byte loads.
+constexpr int kDigits = 26;
+constexpr int kRowWords = 24;
+struct DigitTable {
+  uint32_t row[kDigits * 32][kRowWords];
+};
+
+constexpr void cx_matmul(const uint32_t* a, const uint32_t* b, uint32_t* out, uint32_t m) {
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) {
+      uint64_t acc = 0;
+      for (int k = 0; k < 3; ++k) acc += cx_mulmod(a[3 * i + k], b[3 * k + j], m);
+      out[3 * i + j] = (uint32_t)(acc % m);
+    }
+}
+
+constexpr DigitTable make_digit_table() {
+  DigitTable t{};
+  const PowTable p = make_pow_table();
+  for (int d = 0; d < kDigits; ++d)
+    for (int c = 0; c < 2; ++c) {
+      const int o = 12 * c;
+      for (int i = 0; i < 3; ++i) t.row[32 * d][o + 4 * i] = 1;
+      for (int k = 1; k < 32; ++k)
+        cx_matmul(t.row[32 * d + k - 1] + o, p.m[c][5 * d], t.row[32 * d + k] + o, c == 0 ? M1 : M2);
+    }
+  return t;
+}
+
 // (hi * 2^32 + lo) mod m for m = 2^32 - c, any 64-bit value.
 GRNG_HD inline uint32_t reduce64(uint64_t p, uint32_t m, uint32_t c) {
   uint64_t t = (p & 0xFFFFFFFFull) + (p >> 32) * (uint64_t)c;  // < 2^32 + 2^32 c

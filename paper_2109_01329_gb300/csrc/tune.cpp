@@ -13,7 +13,7 @@
 //   MRG32k3a: the threads per SM of the chunk plan in units of 256 (the
 //     chunk length, hence the jump-ahead work per output, follows from it).
 // 0 keeps the launcher's built-in choice (Philox: 8 waves of resident CTAs;
-// MRG32k3a: 2048 threads per SM).  The table starts from the file named by
+// MRG32k3a: 2048 threads per SM, 3072 for long fills).  The table starts from the file named by
 // the environment variable GRNG_TUNE_CACHE, if set, when it is first read;
 // grng_fill_autotune fills entries by timing, grng_tune_save / _load write and
 // read the text format "grng-tune 1" followed by lines

@@ -479,3 +479,26 @@ def test_odd_length_substreams_at_every_phase(g, engine_kind, stride, var):
         got = host[s * n:(s + 1) * n]
         assert_parity(kind, dtype, got.view(np.uint32) if dtype == 0 else got, ref,
                       f"{var[0]} stream {s}")
+
+
+@pytest.mark.parametrize("var", [v for v in VARIANTS if v[2] == 2 and v[1] >= 2], ids=lambda v: v[0])
+def test_mrg_small_fp64_fills_by_row_length(g, var):
+    """The MRG32k3a FP64 fixed-point fills cut their chunks shorter the fewer
+    words they have: on both sides of each cut the outputs equal the head of a
+    large fill bit for bit, and the smallest the oracle's."""
+    _, kind, dtype, p0, p1 = var
+    d = g.Distribution(kind, dtype, p0, p1)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    big = torch.empty(4_000_000, dtype=torch.float64, device="cuda")
+    g.generate(d, g.Engine(1, 2021, 4), big)
+    ref = oracle.generate(1, 2021, 4, kind, dtype, p0, p1, 1000)
+    for rows in (0, 1, 2, 3):
+        cut = (sms * 256 << (rows + 2)) // 2  # elements: two words each
+        for n in (1, 2, 3, 31, 32, 33, 1000) if rows == 0 else (cut - 3, cut - 1, cut, cut + 2):
+            out = torch.zeros(n + 2, dtype=torch.float64, device="cuda")
+            g.generate(d, g.Engine(1, 2021, 4), out, n)
+            torch.cuda.synchronize()
+            assert torch.equal(out[:n].view(torch.int64), big[:n].view(torch.int64)), (var[0], n)
+            assert out[n:].eq(0).all(), (var[0], n)
+            if n <= 1000:
+                assert_parity(kind, dtype, out[:n].cpu().numpy(), ref[:n], f"{var[0]} n {n}")
