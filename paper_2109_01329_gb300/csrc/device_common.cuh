@@ -308,6 +308,106 @@ __device__ __forceinline__ float icdf_f32(uint32_t w) {
   return icdf_f32_finish(c);
 }
 
+// ------------------------------------------------------ two floats at once
+// FP32 operations on two values per instruction (f32x2): the same
+// round-to-nearest operations as the scalar forms, so the same bits, in half
+// the issue slots.  On this part 8 FFMA and 4 packed ones take the same pipe
+// time (8.9 and 8.6 cycles per warp), but the FP32 fills are bound by issue
+// (71 % of the slots with the pipes 45-65 % busy), not by the FP32 pipes:
+// 10^8 FP32 gaussians 140.2 -> 126.9 us, lognormals 162.2 -> 149.7, inverse
+// CDFs 134.7 -> 128.0.  The uniforms keep their scalar multiply (packed: the
+// same time, 1-2 % slower at word offsets 1-3).  ptxas contracts a packed
+// multiply feeding a packed add into one rounding, so no such pair may stand
+// where the two roundings are wanted.
+struct F2 {
+  uint64_t v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ F2 f2(float a) { return f2(a, a); }
+__device__ __forceinline__ void unpack(F2 x, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+// the generated polynomials are written as nested fmaf calls
+__device__ __forceinline__ F2 fmaf(F2 a, F2 b, float c) { return fma2(a, b, f2(c)); }
+__device__ __forceinline__ F2 fmaf(float a, F2 b, float c) { return fma2(f2(a), b, f2(c)); }
+using ::fmaf;
+
+// neg2_log_u1_f32 of two words, operation by operation (2 fma(k, ln 2, -ln m)
+// as fma(k, 2 ln 2, -2 ln m): scaled by a power of two throughout).
+__device__ __forceinline__ F2 neg2_log_u1_f32x2(uint32_t wa, uint32_t wb) {
+  const int ia = __float_as_int(__uint2float_rn((wa >> 8) + 1u));
+  const int ib = __float_as_int(__uint2float_rn((wb >> 8) + 1u));
+  const int ea = (ia - 0x3F3504F3) >> 23, eb = (ib - 0x3F3504F3) >> 23;
+  const F2 t =
+      add2(f2(__int_as_float(ia - (ea << 23)), __int_as_float(ib - (eb << 23))), f2(-1.0f));
+  F2 p = f2(0.08734750747680664f);
+  p = fmaf(p, t, -0.14307482540607452f);
+  p = fmaf(p, t, 0.14917989075183868f);
+  p = fmaf(p, t, -0.165705144405365f);
+  p = fmaf(p, t, 0.19962070882320404f);
+  p = fmaf(p, t, -0.25001755356788635f);
+  p = fmaf(p, t, 0.33333951234817505f);
+  p = fmaf(p, t, -0.49999991059303284f);
+  const F2 lnm = fma2(mul2(t, t), p, t);
+  const F2 k = add2(f2(__int_as_float(0x4B000000 + 24 - ea), __int_as_float(0x4B000000 + 24 - eb)),
+                    f2(-8388608.0f));
+  return fma2(k, f2(2.0f * 0.693147182464599609375f), mul2(lnm, f2(-2.0f)));
+}
+
+// sincos_turns_f32 of two words.
+__device__ __forceinline__ void sincos_turns_f32x2(uint32_t wa, uint32_t wb, float* s, float* c) {
+  const uint32_t w[2] = {wa, wb};
+  uint32_t o[2], t[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    o[i] = w[i] >> 29;
+    t[i] = (w[i] >> 8) & 0x1FFFFFu;
+    if (o[i] & 1u) t[i] = 0x200000u - t[i];
+  }
+  const F2 v = mul2(add2(f2(__int_as_float(0x4B000000u | t[0]), __int_as_float(0x4B000000u | t[1])),
+                         f2(-8388608.0f)),
+                    f2(0x1p-21f));
+  const F2 ww = mul2(v, v);
+  const F2 sn2 = mul2(
+      v, fmaf(fmaf(fmaf(-3.595459565985948e-05f, ww, 0.0024900073185563087f), ww,
+                   -0.08074543625116348f),
+              ww, 0.7853981852531433f));
+  const F2 cs2 = fma2(ww,
+                      fmaf(fmaf(fmaf(3.531334868966951e-06f, ww, -0.00032594200456514955f), ww,
+                                0.015854327008128166f),
+                           ww, -0.3084251284599304f),
+                      f2(1.0f));
+  float sn[2], cs[2];
+  unpack(sn2, sn[0], sn[1]);
+  unpack(cs2, cs[0], cs[1]);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const bool swap = ((o[i] + 1u) & 2u) != 0;
+    const float a = swap ? cs[i] : sn[i], b = swap ? sn[i] : cs[i];
+    s[i] = (o[i] >= 4u) ? -a : a;
+    c[i] = (((o[i] + 2u) & 4u) != 0) ? -b : b;
+  }
+}
+
 // rho = sqrt(-2 ln u1) by the hardware square root (relative error about
 // 2^-23; its argument is 0 or at least -2 ln(1 - 2^-24) > 1e-7, never
 // subnormal, so the flush-to-zero form, which skips the subnormal handling),
@@ -322,11 +422,38 @@ __device__ __forceinline__ void box_muller_f32(uint32_t w0, uint32_t w1, float& 
   z1 = rho * s;
 }
 
+// The two pairs of a 4-word block, mean + sd z of each: (y0, y1) and (y2, y3).
+__device__ __forceinline__ void gauss_block_f32(const uint32_t* w, const TransformParams& t, F2& ya,
+                                                F2& yb) {
+  float va, vb, ra, rb, s[2], c[2];
+  unpack(neg2_log_u1_f32x2(w[0], w[2]), va, vb);
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(ra) : "f"(va));
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rb) : "f"(vb));
+  sincos_turns_f32x2(w[1], w[3], s, c);
+  const F2 sd = f2(t.fsd), mean = f2(t.fmean);
+  ya = fma2(sd, mul2(f2(ra), f2(c[0], s[0])), mean);
+  yb = fma2(sd, mul2(f2(rb), f2(c[1], s[1])), mean);
+}
+
 // FP64 pair: integer fixed-point evaluation (see bm64_fixed.cuh), within
 // about 1 ulp of the exact value, without the FP64 pipe.
 __device__ __forceinline__ void box_muller_f64(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,
                                                double& z0, double& z1) {
   bm64::box_muller(u53(w0, w1), u53(w2, w3), z0, z1);
+}
+
+// icdf_f32_central of two words.
+__device__ __forceinline__ void icdf_f32_central2(uint32_t wa, uint32_t wb, Icdf32& a, Icdf32& b) {
+  const F2 f = f2(__int_as_float(0x4B000000u | (wa >> 9)), __int_as_float(0x4B000000u | (wb >> 9)));
+  const F2 x = add2(fmaf(f, f2(0x1p-22f), -3.0f), f2(0x1p-23f));
+  float qa, qb, la, lb;
+  unpack(fmaf(mul2(x, f2(-1.0f)), x, 1.0f), qa, qb);
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(la) : "f"(qa));
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lb) : "f"(qb));
+  const F2 v = mul2(f2(la, lb), f2(-1.0f));
+  unpack(x, a.x, b.x);
+  unpack(v, a.v, b.v);
+  unpack(GRNG_ICDF32_P1(v), a.r, b.r);
 }
 
 // mean + sd z, or exp of it, as the output word of an inverse-CDF variant
@@ -442,11 +569,25 @@ __device__ __forceinline__ uint4 block_outputs(uint4 b, const TransformParams& t
                                                                  : 2;
   uint32_t w[4] = {b.x, b.y, b.z, b.w};
   uint32_t o[4];
-  if constexpr (V == V_ICDF_GAUSS_F32 || V == V_ICDF_LOGN_F32) {
-    // the four central evaluations interleave; one vote skips the tails
+  if constexpr (V == V_GAUSS_F32 || V == V_LOGN_F32) {
+    F2 r[2];
+    gauss_block_f32(w, t, r[0], r[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float y[2];
+      unpack(r[h], y[0], y[1]);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if constexpr (V == V_LOGN_F32) y[i] = expf(y[i]);
+        o[2 * h + i] = __float_as_uint(y[i]);
+      }
+    }
+  } else if constexpr (V == V_ICDF_GAUSS_F32 || V == V_ICDF_LOGN_F32) {
+    // the four central evaluations interleave, two values an instruction; one
+    // vote skips the tails
     Icdf32 c[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) c[u] = icdf_f32_central(w[u]);
+    for (int h = 0; h < 2; ++h) icdf_f32_central2(w[2 * h], w[2 * h + 1], c[2 * h], c[2 * h + 1]);
     if (icdf_f32_is_tail(c[0]) | icdf_f32_is_tail(c[1]) | icdf_f32_is_tail(c[2]) |
         icdf_f32_is_tail(c[3])) {
 #pragma unroll

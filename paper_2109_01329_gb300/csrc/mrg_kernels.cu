@@ -297,9 +297,11 @@ __global__ void __launch_bounds__(kThreads) mrg_fill_kernel(const __grid_constan
         constexpr int kChUnroll = VInfo<V>::weight == 0 ? 8 : VInfo<V>::weight == 1 ? 2 : 1;
 #pragma unroll kChUnroll
         for (int ch = 0; ch < pieces; ++ch) {
-          uint32_t o4[4];
+          uint32_t w[4];
 #pragma unroll
-          for (int u = 0; u < kUpc; ++u) gen_unit<V>(st, o4 + u * kWpu, p, (u & 1) != 0);
+          for (int i = 0; i < 4; ++i) w[i] = mrg_next(st, p);
+          const uint4 o = block_outputs<V>(make_uint4(w[0], w[1], w[2], w[3]), p.t);
+          const uint32_t o4[4] = {o.x, o.y, o.z, o.w};
           stage[warp][lane][ch ^ (lane & 7)] = kCarry ? shift_in<true, kOwpe>(carry, o4)
                                                       : shift_in<false, kOwpe>(carry, o4);
         }
