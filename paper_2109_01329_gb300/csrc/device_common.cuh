@@ -25,14 +25,26 @@ constexpr uint32_t kPhiloxM1 = 0xCD9E8D57u;
 constexpr uint32_t kPhiloxW0 = 0x9E3779B9u;
 constexpr uint32_t kPhiloxW1 = 0xBB67AE85u;
 
+// Both halves of a b.  Written as one wide multiply: as __umulhi and a 32-bit
+// product the compiler does not always find the pair (59 against 44
+// instructions per block for the same rounds).
+__device__ __forceinline__ void mul_hi_lo(uint32_t a, uint32_t b, uint32_t& hi, uint32_t& lo) {
+  uint64_t t;
+  asm("mul.wide.u32 %0, %1, %2;" : "=l"(t) : "r"(a), "r"(b));
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(t));
+}
+
+__device__ __forceinline__ uint4 philox_round(uint4 c, uint32_t k0, uint32_t k1) {
+  uint32_t hi0, lo0, hi1, lo1;
+  mul_hi_lo(c.x, kPhiloxM0, hi0, lo0);
+  mul_hi_lo(c.z, kPhiloxM1, hi1, lo1);
+  return make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+}
+
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1) {
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
-    const uint32_t hi0 = __umulhi(kPhiloxM0, c.x);
-    const uint32_t lo0 = kPhiloxM0 * c.x;
-    const uint32_t hi1 = __umulhi(kPhiloxM1, c.z);
-    const uint32_t lo1 = kPhiloxM1 * c.z;
-    c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+    c = philox_round(c, k0, k1);
     k0 += kPhiloxW0;
     k1 += kPhiloxW1;
   }
@@ -56,13 +68,74 @@ __host__ __device__ inline PhiloxRoundKeys philox_round_keys(uint32_t k0, uint32
 }
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxRoundKeys& rk) {
 #pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint32_t hi0 = __umulhi(kPhiloxM0, c.x);
-    const uint32_t lo0 = kPhiloxM0 * c.x;
-    const uint32_t hi1 = __umulhi(kPhiloxM1, c.z);
-    const uint32_t lo1 = kPhiloxM1 * c.z;
-    c = make_uint4(hi1 ^ c.y ^ rk.k[2 * r], lo1, hi0 ^ c.w ^ rk.k[2 * r + 1], lo0);
+  for (int r = 0; r < 10; ++r) c = philox_round(c, rk.k[2 * r], rk.k[2 * r + 1]);
+  return c;
+}
+
+// The blocks of one single-stream fill: block j has counter base + j, of which
+// only the low 32-bit word x varies while no carry leaves it.  The other three
+// words fix the second product of round 0 and with it the first of round 1,
+// so a block costs 18 wide products of the 20 and a 32-bit counter add in
+// place of a 64-bit one.  e, a, b, d are what those rounds add (by exclusive
+// or, round keys included) for given upper words; s[1] holds them for the upper words
+// after the carry, for fills that cross a multiple of 2^32 blocks.
+struct PhiloxUpper {
+  uint32_t e, a, b, d;
+};
+struct PhiloxStream {
+  uint32_t x0;        // low word of the base counter
+  PhiloxUpper s[2];
+  uint32_t k[16];     // round keys of rounds 2..9 (k1 of round 2 is in d)
+};
+constexpr uint64_t kPhiloxMaxBlocks = uint64_t(1) << 32;  // blocks of one PhiloxStream
+
+inline PhiloxUpper philox_upper(uint32_t k0, uint32_t k1, uint32_t y, uint32_t z, uint32_t w) {
+  const uint64_t p1 = (uint64_t)kPhiloxM1 * z;                          // round 0, second product
+  const uint32_t x1 = (uint32_t)(p1 >> 32) ^ y ^ k0;
+  const uint64_t p0 = (uint64_t)kPhiloxM0 * x1;                         // round 1, first product
+  const uint32_t k0_1 = k0 + kPhiloxW0, k1_1 = k1 + kPhiloxW1;
+  PhiloxUpper u;
+  u.e = w ^ k1;
+  u.a = (uint32_t)p1 ^ k0_1;
+  u.b = (uint32_t)(p0 >> 32) ^ k1_1;
+  u.d = (uint32_t)p0 ^ (k1 + 2u * kPhiloxW1);
+  return u;
+}
+
+// base: block counter mod 2^126, as ctr_from takes it
+inline PhiloxStream philox_stream(uint32_t k0, uint32_t k1, uint64_t base_lo, uint64_t base_hi) {
+  PhiloxStream p;
+  p.x0 = (uint32_t)base_lo;
+  uint64_t lo = base_lo, hi = base_hi;
+  for (int i = 0; i < 2; ++i) {
+    p.s[i] = philox_upper(k0, k1, (uint32_t)(lo >> 32), (uint32_t)hi,
+                          (uint32_t)(hi >> 32) & 0x3FFFFFFFu);
+    lo += uint64_t(1) << 32;
+    hi += (lo >> 32) == 0 ? 1u : 0u;
   }
+  for (int r = 2; r < 10; ++r) {
+    p.k[2 * (r - 2)] = k0 + (uint32_t)r * kPhiloxW0;
+    p.k[2 * (r - 2) + 1] = k1 + (uint32_t)r * kPhiloxW1;
+  }
+  return p;
+}
+
+// Block j (j < 2^32); kCross: x0 + j may carry out of 32 bits.
+template <bool kCross>
+__device__ __forceinline__ uint4 philox_block(uint32_t j, const PhiloxStream& p) {
+  const uint32_t x = p.x0 + j;
+  PhiloxUpper u = p.s[0];
+  if (kCross && x < j) u = p.s[1];
+  uint32_t z1, w1, x2, y2;
+  mul_hi_lo(x, kPhiloxM0, z1, w1);
+  mul_hi_lo(z1 ^ u.e, kPhiloxM1, x2, y2);
+  // round 2, whose fourth counter word is a constant
+  uint32_t hi0, lo0, hi1, lo1;
+  mul_hi_lo(x2 ^ u.a, kPhiloxM0, hi0, lo0);
+  mul_hi_lo(w1 ^ u.b, kPhiloxM1, hi1, lo1);
+  uint4 c = make_uint4(hi1 ^ y2 ^ p.k[0], lo1, hi0 ^ u.d, lo0);
+#pragma unroll
+  for (int r = 3; r < 10; ++r) c = philox_round(c, p.k[2 * (r - 2)], p.k[2 * (r - 2) + 1]);
   return c;
 }
 

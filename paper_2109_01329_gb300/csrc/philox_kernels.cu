@@ -73,65 +73,72 @@ __device__ __forceinline__ void store_partial(char* stream_base, int64_t e0, int
 // ------------------------------------------------------------ single stream
 // Full 16-byte groups [jf, jl) in the main loop, U independent counter blocks
 // per thread per iteration (stores of the U blocks are each coalesced across
-// the warp), pointer and counter advanced by increments.  The at most two
-// partial groups (the first and the last) are done by the grid's first two
-// threads before the loop.
+// the warp).  The at most two partial groups (the first and the last) are done
+// by the grid's first two threads before the loop.
+//
+// Bound by the FMA-heavy pipe (the products) until it meets the write roof:
+// with 18 products, each one wide multiply, a bits block costs 44 instructions
+// of 55 before, and the contiguous tiles keep a CTA's stores together (grid-
+// strided: bits 0.541 ms).  10^9 outputs, before -> now: bits 0.602 -> 0.531 ms
+// (7.53 TB/s), FP32 uniforms 0.665 -> 0.594, FP64 uniforms 1.650 -> 1.405, FP32
+// gaussians 1.351 -> 1.095 (1.22 with the f32x2 polynomials alone), FP64
+// gaussians 6.26 -> 6.10.
 struct StreamParams {
   TransformParams t;
   uint4* gbase;       // 16-byte aligned address of group 0 (may precede out)
   void* out;
   int64_t n;          // elements
   int64_t head;       // elements of group 0 that lie before out
-  int64_t jf, jl;     // full groups [jf, jl)
+  uint32_t jf, jl;    // full groups [jf, jl)
   int64_t edge[2];    // partial groups, or -1
-  uint64_t base_lo;   // block counter of group 0
-  uint64_t base_hi;
-  PhiloxRoundKeys rk;
+  PhiloxStream ctr;   // block 0: that of group 0
 };
 
-template <int V, bool kHiUniform>
-__device__ __forceinline__ uint4 group_block(const StreamParams& p, uint64_t j) {
-  const uint64_t lo = p.base_lo + j;
-  const uint64_t hi = kHiUniform ? p.base_hi : p.base_hi + ((lo < p.base_lo) ? 1u : 0u);
-  return philox4x32_10(ctr_from(lo, hi), p.rk);
-}
-
-template <int V, int U, bool kHiUniform>
+template <int V, int U, bool kCross>
 __device__ __forceinline__ void philox_stream_body(const StreamParams& p) {
   using I = VInfo<V>;
   constexpr int kEpg = 16 / I::es;
-  const int64_t T = (int64_t)gridDim.x * kThreads;
-  const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const uint32_t tid = blockIdx.x * kThreads + threadIdx.x;
   if (tid < 2 && p.edge[tid] >= 0) {
     const int64_t j = p.edge[tid];
-    const uint4 o = block_outputs<V>(group_block<V, false>(p, (uint64_t)j), p.t);
+    const uint4 o = block_outputs<V>(philox_block<true>((uint32_t)j, p.ctr), p.t);
     store_partial<V>(reinterpret_cast<char*>(p.out), j * kEpg - p.head, p.n, o);
   }
-  int64_t j = p.jf + tid;
+  // a CTA's tile is U x kThreads consecutive groups, thread t's at t, t +
+  // kThreads, ...: constant store offsets and counter steps
+  const uint32_t step = gridDim.x * (kThreads * U);
+  uint32_t j = p.jf + blockIdx.x * (kThreads * U) + threadIdx.x;
   uint4* dst = p.gbase + j;
-  for (; j + (U - 1) * T < p.jl; j += U * T, dst += U * T) {
+  for (; j + (U - 1) * kThreads < p.jl; j += step, dst += step) {
     uint4 o[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      o[u] = block_outputs<V>(group_block<V, kHiUniform>(p, (uint64_t)(j + u * T)), p.t);
+    for (int u = 0; u < U; ++u) o[u] = block_outputs<V>(philox_block<kCross>(j + u * kThreads, p.ctr), p.t);
 #pragma unroll
-    for (int u = 0; u < U; ++u) dst[u * T] = o[u];
+    for (int u = 0; u < U; ++u) dst[u * kThreads] = o[u];
   }
-  for (; j < p.jl; j += T, dst += T)
-    *dst = block_outputs<V>(group_block<V, kHiUniform>(p, (uint64_t)j), p.t);
+  if constexpr (U > 1) {
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+      if (j + u * kThreads < p.jl)
+        dst[u * kThreads] = block_outputs<V>(philox_block<kCross>(j + u * kThreads, p.ctr), p.t);
+  }
 }
 
 // Counter blocks per thread per loop iteration: six for bits and the FP32
-// uniforms (2, 4, 6 and 8 measured: 6 fastest), two for the other FP32 and
-// the FP64 uniform transforms (3 and 4 slower), one for the FP64 fixed-point
-// transforms (hundreds of instructions per unit).
+// uniforms, near the write roof (10^9 uniforms at 1, 2, 4, 6, 8: 0.642, 0.607,
+// 0.605, 0.594, 0.590 ms), two for the FP32 Box-Muller and inverse CDF (10^9
+// gaussians 1.095 ms; 1: 1.111), one for the 8-byte outputs, whose transform is
+// long enough by itself (10^9 FP64 uniforms 1.405 ms; 2: 1.449).
 template <int V>
 constexpr int blocks_per_thread() {
-  return (V == V_BITS || V == V_U01_F32 || V == V_UNI_F32) ? 6
-         : (V == V_GAUSS_F64 || V == V_LOGN_F64 || V == V_STDGAUSS_F64 ||
-            V == V_ICDF_GAUSS_F64 || V == V_ICDF_LOGN_F64)
-             ? 1
-             : 2;
+  return (V == V_BITS || V == V_U01_F32 || V == V_UNI_F32) ? 6 : VInfo<V>::es == 8 ? 1 : 2;
+}
+
+// In the kernels that exchange between lanes the [0, 1) and exact FP64 uniforms
+// take two (10^8 at word offset 1: 0.223 ms against 0.226 with one).
+template <int V>
+constexpr int exchange_blocks_per_thread() {
+  return V == V_U01_F64 || V == V_AFF_F64 ? 2 : blocks_per_thread<V>();
 }
 
 // The Box-Muller and FP32 inverse-CDF variants gain from a fifth resident CTA
@@ -143,14 +150,14 @@ constexpr bool stream_wants_5_ctas() {
          V == V_STDGAUSS_F64 || V == V_LOGN_F64 || V == V_ICDF_GAUSS_F64 || V == V_ICDF_LOGN_F64;
 }
 
-template <int V, int U, bool kHiUniform>
+template <int V, int U, bool kCross>
 __global__ void __launch_bounds__(kThreads) philox_stream_kernel(const __grid_constant__ StreamParams p) {
-  philox_stream_body<V, U, kHiUniform>(p);
+  philox_stream_body<V, U, kCross>(p);
 }
 
-template <int V, int U, bool kHiUniform>
+template <int V, int U, bool kCross>
 __global__ void __launch_bounds__(kThreads, 5) philox_stream_kernel_5(const __grid_constant__ StreamParams p) {
-  philox_stream_body<V, U, kHiUniform>(p);
+  philox_stream_body<V, U, kCross>(p);
 }
 
 // ------------------------------------------------------ single stream, shifted
@@ -177,10 +184,8 @@ struct ShiftParams {
   int64_t groups;
   int64_t jf, jl;     // groups [jf, jl) lie wholly inside the output
   int64_t chunks;     // ceil(groups / groups per warp chunk)
-  uint64_t base_lo;   // block holding the first word of (virtual) group 0
-  uint64_t base_hi;
+  PhiloxStream ctr;   // block 0: that of the first word of (virtual) group 0
   uint32_t ph;        // its word phase: 1..3, or 0..3 with kSplit
-  PhiloxRoundKeys rk;
 };
 
 template <bool kSplit>
@@ -228,32 +233,26 @@ __device__ __forceinline__ uint4 split_group(uint4 v) {
 }
 
 // kPh: the word phase as a constant (1..3), or -1 to read it from p.ph.
-template <int V, int U, bool kHiUniform, bool kSplit, int kPh>
+template <int V, int U, bool kCross, bool kSplit, int kPh>
 __device__ __forceinline__ void philox_shift_body(const ShiftParams& p) {
   using I = VInfo<V>;
   constexpr int kEpg = 16 / I::es;
   constexpr int kPer = shift_per_warp<kSplit>();
   const int lane = threadIdx.x & 31;
   const int64_t TW = (int64_t)gridDim.x * (kThreads / 32);
-  const int64_t c0 = (int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-  // this lane's group of chunk c is j = c kPer + lane; j, the block counter
-  // and the store address advance by increments (dj from chunk c to c + TW)
+  const int64_t c0 = ((int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * U;
+  // a warp takes U consecutive chunks; this lane's group of chunk c is j =
+  // c kPer + lane, and those of the U chunks lie at constant offsets
   const int64_t dj = TW * kPer;
   int64_t j = c0 * kPer + lane;
-  uint64_t lo = p.base_lo + (uint64_t)j;
   uint4* dst = p.gbase + j;
   // the loop bound depends only on the warp: every shuffle has all 32 lanes
-  for (int64_t c = c0; c < p.chunks;
-       c += U * TW, j += U * dj, lo += (uint64_t)(U * dj), dst += U * dj) {
+  for (int64_t c = c0; c < p.chunks; c += U * TW, j += U * dj, dst += U * dj) {
     uint4 b[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint64_t l = lo + (uint64_t)(u * dj);
-      const uint64_t h = kHiUniform ? p.base_hi : p.base_hi + ((l < p.base_lo) ? 1u : 0u);
-      b[u] = philox4x32_10(ctr_from(l, h), p.rk);
-    }
+    for (int u = 0; u < U; ++u) b[u] = philox_block<kCross>((uint32_t)j + u * kPer, p.ctr);
     // every group of this iteration lies wholly inside the output (uniform)
-    const bool interior = c * kPer >= p.jf && (c + (U - 1) * TW) * kPer + kPer <= p.jl;
+    const bool interior = c * kPer >= p.jf && (c + U) * kPer <= p.jl;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       uint4 w;
@@ -267,13 +266,13 @@ __device__ __forceinline__ void philox_shift_body(const ShiftParams& p) {
       uint4 o = block_outputs<V>(w, p.t);
       if constexpr (kSplit) o = split_group<V>(o);
       if (interior) {
-        if (lane < kPer) dst[u * dj] = o;
+        if (lane < kPer) dst[u * kPer] = o;
       } else {
-        const int64_t ju = j + u * dj;
+        const int64_t ju = j + u * kPer;
         if (lane < kPer && ju < p.groups) {
           const int64_t e0 = ju * kEpg - p.head;
           if (e0 >= 0 && e0 + kEpg <= p.n) {
-            dst[u * dj] = o;
+            dst[u * kPer] = o;
           } else {
             store_partial<V>(reinterpret_cast<char*>(p.out), e0, p.n, o);
           }
@@ -291,33 +290,33 @@ __device__ __forceinline__ void philox_shift_body(const ShiftParams& p) {
 // instructions, the words moved into place one by one where the variable form
 // selects each into place), while phases 2 and 3 gained 4-8 %.  The other
 // variants keep the variable phase.
-template <int V, int U, bool kHiUniform, bool kSplit>
+template <int V, int U, bool kCross, bool kSplit>
 __device__ __forceinline__ void philox_shift_phases(const ShiftParams& p) {
   if constexpr (V == V_BITS && !kSplit) {
     switch (p.ph) {
-      case 1: philox_shift_body<V, U, kHiUniform, kSplit, 1>(p); break;
-      case 2: philox_shift_body<V, U, kHiUniform, kSplit, 2>(p); break;
-      default: philox_shift_body<V, U, kHiUniform, kSplit, 3>(p); break;
+      case 1: philox_shift_body<V, U, kCross, kSplit, 1>(p); break;
+      case 2: philox_shift_body<V, U, kCross, kSplit, 2>(p); break;
+      default: philox_shift_body<V, U, kCross, kSplit, 3>(p); break;
     }
   } else if constexpr ((V == V_U01_F32 || V == V_UNI_F32) && !kSplit) {
     switch (p.ph) {
-      case 2: philox_shift_body<V, U, kHiUniform, kSplit, 2>(p); break;
-      case 3: philox_shift_body<V, U, kHiUniform, kSplit, 3>(p); break;
-      default: philox_shift_body<V, U, kHiUniform, kSplit, -1>(p); break;
+      case 2: philox_shift_body<V, U, kCross, kSplit, 2>(p); break;
+      case 3: philox_shift_body<V, U, kCross, kSplit, 3>(p); break;
+      default: philox_shift_body<V, U, kCross, kSplit, -1>(p); break;
     }
   } else {
-    philox_shift_body<V, U, kHiUniform, kSplit, -1>(p);
+    philox_shift_body<V, U, kCross, kSplit, -1>(p);
   }
 }
 
-template <int V, int U, bool kHiUniform, bool kSplit>
+template <int V, int U, bool kCross, bool kSplit>
 __global__ void __launch_bounds__(kThreads) philox_shift_kernel(const __grid_constant__ ShiftParams p) {
-  philox_shift_phases<V, U, kHiUniform, kSplit>(p);
+  philox_shift_phases<V, U, kCross, kSplit>(p);
 }
 
-template <int V, int U, bool kHiUniform, bool kSplit>
+template <int V, int U, bool kCross, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 5) philox_shift_kernel_5(const __grid_constant__ ShiftParams p) {
-  philox_shift_phases<V, U, kHiUniform, kSplit>(p);
+  philox_shift_phases<V, U, kCross, kSplit>(p);
 }
 
 // ------------------------------------------------------ single stream, rotated
@@ -341,10 +340,8 @@ struct RotateParams {
   int64_t r;          // word offset mod 4
   int64_t gofs;       // the group lane l completes is out's group + j + gofs (0 or -1)
   int64_t chunks;     // ceil(blocks / 32)
-  uint64_t base_lo;   // block holding the stream's first word
-  uint64_t base_hi;
+  PhiloxStream ctr;   // block 0: that of the stream's first word
   uint32_t s;         // the rotation kS, 1..3
-  PhiloxRoundKeys rk;
 };
 
 // (lane - 1's last kS output words, this lane's first 4 - kS)
@@ -400,36 +397,30 @@ __device__ __forceinline__ void store_positions_checked(const RotateParams& p, i
   }
 }
 
-template <int V, int U, bool kHiUniform, int kS>
+template <int V, int U, bool kCross, int kS>
 __device__ __forceinline__ void philox_rotate_body(const RotateParams& p) {
   const int lane = threadIdx.x & 31;
   const int64_t TW = (int64_t)gridDim.x * (kThreads / 32);
-  const int64_t c0 = (int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-  // lane l of chunk c holds block j = 32 c + l; j, the counter and the group
-  // address advance by increments (dj from chunk c to c + TW)
+  const int64_t c0 = ((int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * U;
+  // a warp takes U consecutive chunks; lane l of chunk c holds block j =
+  // 32 c + l, and those of the U chunks lie at constant offsets
   const int64_t dj = TW * 32;
   int64_t j = c0 * 32 + lane;
-  uint64_t lo = p.base_lo + (uint64_t)j;
   uint4* dst = p.gbase + (j + p.gofs);
   // the loop bound depends only on the warp: every shuffle has all 32 lanes
-  for (int64_t c = c0; c < p.chunks;
-       c += U * TW, j += U * dj, lo += (uint64_t)(U * dj), dst += U * dj) {
+  for (int64_t c = c0; c < p.chunks; c += U * TW, j += U * dj, dst += U * dj) {
     uint4 b[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint64_t l = lo + (uint64_t)(u * dj);
-      const uint64_t hh = kHiUniform ? p.base_hi : p.base_hi + ((l < p.base_lo) ? 1u : 0u);
-      b[u] = philox4x32_10(ctr_from(l, hh), p.rk);
-    }
+    for (int u = 0; u < U; ++u) b[u] = philox_block<kCross>((uint32_t)j + u * 32, p.ctr);
     // every output word of this iteration's chunks lies inside the output
     // (uniform): words 128 c - r .. 128 c' + 127 - r, c' the last chunk
-    const bool interior = c * 128 - p.r >= 0 && (c + (U - 1) * TW) * 128 + 127 - p.r < p.nw;
+    const bool interior = c * 128 - p.r >= 0 && (c + U) * 128 - 1 - p.r < p.nw;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const uint4 o = block_outputs<V>(b[u], p.t);
       const uint4 g = rotate_up<kS>(o);
       if (interior) {
-        uint4* gp = dst + u * dj;
+        uint4* gp = dst + u * 32;
         if (lane > 0) {
           *gp = g;
         } else {
@@ -437,7 +428,7 @@ __device__ __forceinline__ void philox_rotate_body(const RotateParams& p) {
         }
         if (lane == 31) store_positions<V, 0, kS, 4 - kS>(gp + 1, o);
       } else {
-        const int64_t G = j + u * dj + p.gofs;
+        const int64_t G = j + u * 32 + p.gofs;
         if (lane > 0) {
           store_positions_checked<V, 0, 4, 0>(p, G, g);
         } else {
@@ -451,27 +442,27 @@ __device__ __forceinline__ void philox_rotate_body(const RotateParams& p) {
 
 // The rotation is the same for the whole grid: one loop per rotation, each
 // with it a constant (8-byte elements rotate by one element only).
-template <int V, int U, bool kHiUniform>
+template <int V, int U, bool kCross>
 __device__ __forceinline__ void philox_rotate_phases(const RotateParams& p) {
   if constexpr (VInfo<V>::es == 8) {
-    philox_rotate_body<V, U, kHiUniform, 2>(p);
+    philox_rotate_body<V, U, kCross, 2>(p);
   } else {
     switch (p.s) {
-      case 1: philox_rotate_body<V, U, kHiUniform, 1>(p); break;
-      case 2: philox_rotate_body<V, U, kHiUniform, 2>(p); break;
-      default: philox_rotate_body<V, U, kHiUniform, 3>(p); break;
+      case 1: philox_rotate_body<V, U, kCross, 1>(p); break;
+      case 2: philox_rotate_body<V, U, kCross, 2>(p); break;
+      default: philox_rotate_body<V, U, kCross, 3>(p); break;
     }
   }
 }
 
-template <int V, int U, bool kHiUniform>
+template <int V, int U, bool kCross>
 __global__ void __launch_bounds__(kThreads) philox_rotate_kernel(const __grid_constant__ RotateParams p) {
-  philox_rotate_phases<V, U, kHiUniform>(p);
+  philox_rotate_phases<V, U, kCross>(p);
 }
 
-template <int V, int U, bool kHiUniform>
+template <int V, int U, bool kCross>
 __global__ void __launch_bounds__(kThreads, 5) philox_rotate_kernel_5(const __grid_constant__ RotateParams p) {
-  philox_rotate_phases<V, U, kHiUniform>(p);
+  philox_rotate_phases<V, U, kCross>(p);
 }
 
 // ------------------------------------------------------------ substreams
@@ -653,29 +644,28 @@ int blocks_per_sm(K kernel) {
 // Launches the shift kernel: words of (virtual) group 0 start at word a of
 // the stream (128-bit, a = off - head words, one element earlier for kSplit).
 template <int V, bool kSplit>
-void launch_shift(ShiftParams& p, uint64_t a_lo, uint64_t a_hi, int sms, int32_t geom,
-                  cudaStream_t stream) {
+void launch_shift(ShiftParams& p, const uint32_t* key, uint64_t a_lo, uint64_t a_hi, int sms,
+                  int32_t geom, cudaStream_t stream) {
   constexpr int kPer = shift_per_warp<kSplit>();
-  constexpr int kU = blocks_per_thread<V>();
-  p.base_lo = (a_lo >> 2) | (a_hi << 62);
-  p.base_hi = a_hi >> 2;
+  constexpr int kU = exchange_blocks_per_thread<V>();
+  p.ctr = philox_stream(key[0], key[1], (a_lo >> 2) | (a_hi << 62), a_hi >> 2);
   p.ph = (uint32_t)(a_lo & 3u);
   p.chunks = (p.groups + kPer - 1) / kPer;
-  void (*k_uni)(const ShiftParams);
-  void (*k_carry)(const ShiftParams);
+  void (*k_same)(const ShiftParams);
+  void (*k_cross)(const ShiftParams);
   if constexpr (stream_wants_5_ctas<V>()) {
-    k_uni = philox_shift_kernel_5<V, kU, true, kSplit>;
-    k_carry = philox_shift_kernel_5<V, kU, false, kSplit>;
+    k_same = philox_shift_kernel_5<V, kU, false, kSplit>;
+    k_cross = philox_shift_kernel_5<V, kU, true, kSplit>;
   } else {
-    k_uni = philox_shift_kernel<V, kU, true, kSplit>;
-    k_carry = philox_shift_kernel<V, kU, false, kSplit>;
+    k_same = philox_shift_kernel<V, kU, false, kSplit>;
+    k_cross = philox_shift_kernel<V, kU, true, kSplit>;
   }
   static std::atomic<int> occ[2] = {{0}, {0}};
   int o = occ[0].load(std::memory_order_relaxed);
   if (o == 0) {
-    o = blocks_per_sm(k_uni);
+    o = blocks_per_sm(k_same);
     occ[0].store(o, std::memory_order_relaxed);
-    occ[1].store(blocks_per_sm(k_carry), std::memory_order_relaxed);
+    occ[1].store(blocks_per_sm(k_cross), std::memory_order_relaxed);
   }
   const int64_t warps = (p.chunks + kU - 1) / kU;
   int64_t grid = (warps + (kThreads / 32) - 1) / (kThreads / 32);
@@ -685,45 +675,44 @@ void launch_shift(ShiftParams& p, uint64_t a_lo, uint64_t a_hi, int sms, int32_t
   // blocks touched: below (chunks + kU * warps in flight) * kPer + 32 past base
   const uint64_t reach =
       (uint64_t)(p.chunks + (int64_t)kU * grid * (kThreads / 32) + 1) * (uint64_t)kPer + 64u;
-  const bool hi_uniform = p.base_lo + reach >= p.base_lo;
-  if (!hi_uniform) {
+  const bool cross = p.ctr.x0 + reach >= kPhiloxMaxBlocks;
+  if (cross) {
     const int64_t cap2 = (int64_t)sms * ctas_cap(occ[1].load(std::memory_order_relaxed), geom);
     if (grid > cap2) grid = cap2;
   }
-  (hi_uniform ? k_uni : k_carry)<<<(unsigned)grid, kThreads, 0, stream>>>(p);
+  (cross ? k_cross : k_same)<<<(unsigned)grid, kThreads, 0, stream>>>(p);
 }
 
 // Launches the rotate kernel (units inside blocks, output start at another
 // phase); p.t, p.out, p.gbase, p.nw, p.h, p.rk are set by the caller.
 template <int V>
-void launch_rotate(RotateParams& p, uint64_t off_lo, uint64_t off_hi, int sms, int32_t geom,
-                   cudaStream_t stream) {
-  constexpr int kU = blocks_per_thread<V>();
+void launch_rotate(RotateParams& p, const uint32_t* key, uint64_t off_lo, uint64_t off_hi, int sms,
+                   int32_t geom, cudaStream_t stream) {
+  constexpr int kU = exchange_blocks_per_thread<V>();
   p.r = (int64_t)(off_lo & 3u);
   const int64_t d = p.h - p.r;
   p.s = (uint32_t)((d + 4) & 3);
   p.gofs = d < 0 ? -1 : 0;
-  p.base_lo = (off_lo >> 2) | (off_hi << 62);
-  p.base_hi = off_hi >> 2;
+  p.ctr = philox_stream(key[0], key[1], (off_lo >> 2) | (off_hi << 62), off_hi >> 2);
   const int64_t blocks = (p.nw - 1 + p.r) / 4 + 1;
   p.chunks = (blocks + 31) / 32;
-  void (*k_uni)(const RotateParams);
-  void (*k_carry)(const RotateParams);
+  void (*k_same)(const RotateParams);
+  void (*k_cross)(const RotateParams);
   // the FP64 Box-Muller variants gain from a fifth CTA as in the stream
   // kernel; the FP32 ones would spill under its register cap here
   if constexpr (stream_wants_5_ctas<V>() && VInfo<V>::es == 8) {
-    k_uni = philox_rotate_kernel_5<V, kU, true>;
-    k_carry = philox_rotate_kernel_5<V, kU, false>;
+    k_same = philox_rotate_kernel_5<V, kU, false>;
+    k_cross = philox_rotate_kernel_5<V, kU, true>;
   } else {
-    k_uni = philox_rotate_kernel<V, kU, true>;
-    k_carry = philox_rotate_kernel<V, kU, false>;
+    k_same = philox_rotate_kernel<V, kU, false>;
+    k_cross = philox_rotate_kernel<V, kU, true>;
   }
   static std::atomic<int> occ[2] = {{0}, {0}};
   int o = occ[0].load(std::memory_order_relaxed);
   if (o == 0) {
-    o = blocks_per_sm(k_uni);
+    o = blocks_per_sm(k_same);
     occ[0].store(o, std::memory_order_relaxed);
-    occ[1].store(blocks_per_sm(k_carry), std::memory_order_relaxed);
+    occ[1].store(blocks_per_sm(k_cross), std::memory_order_relaxed);
   }
   const int64_t warps = (p.chunks + kU - 1) / kU;
   int64_t grid = (warps + (kThreads / 32) - 1) / (kThreads / 32);
@@ -732,12 +721,12 @@ void launch_rotate(RotateParams& p, uint64_t off_lo, uint64_t off_hi, int sms, i
   if (grid > cap) grid = cap;
   // blocks touched: below (chunks + kU * warps in flight) * 32 past base
   const uint64_t reach = (uint64_t)(p.chunks + (int64_t)kU * grid * (kThreads / 32) + 1) * 32u;
-  const bool hi_uniform = p.base_lo + reach >= p.base_lo;
-  if (!hi_uniform) {
+  const bool cross = p.ctr.x0 + reach >= kPhiloxMaxBlocks;
+  if (cross) {
     const int64_t cap2 = (int64_t)sms * ctas_cap(occ[1].load(std::memory_order_relaxed), geom);
     if (grid > cap2) grid = cap2;
   }
-  (hi_uniform ? k_uni : k_carry)<<<(unsigned)grid, kThreads, 0, stream>>>(p);
+  (cross ? k_cross : k_same)<<<(unsigned)grid, kThreads, 0, stream>>>(p);
 }
 
 template <int V>
@@ -770,9 +759,7 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
     p.gbase = reinterpret_cast<uint4*>(addr - phase_w * 4u);
     p.n = r.n;
     p.head = head;
-    p.base_lo = base_lo;
-    p.base_hi = base_hi;
-    p.rk = philox_round_keys(r.key[0], r.key[1]);
+    p.ctr = philox_stream(r.key[0], r.key[1], base_lo, base_hi);
     // full groups: the first group is partial when head > 0, the last one
     // when the end is not on a group boundary (or both are the same group)
     int64_t jf = head > 0 ? 1 : 0;
@@ -785,23 +772,23 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
       if (head > 0) p.edge[0] = 0;
       if (jl < groups) p.edge[1] = groups - 1;
     }
-    p.jf = jf;
-    p.jl = jl;
+    p.jf = (uint32_t)jf;
+    p.jl = (uint32_t)jl;
     constexpr int kU = blocks_per_thread<V>();
-    const bool hi_uniform = base_lo + (uint64_t)groups >= base_lo;  // no carry into the top half
+    const bool cross = p.ctr.x0 + (uint64_t)groups >= kPhiloxMaxBlocks;
     void (*kernel)(const StreamParams);
     if constexpr (stream_wants_5_ctas<V>()) {
-      kernel = hi_uniform ? philox_stream_kernel_5<V, kU, true> : philox_stream_kernel_5<V, kU, false>;
+      kernel = cross ? philox_stream_kernel_5<V, kU, true> : philox_stream_kernel_5<V, kU, false>;
     } else {
-      kernel = hi_uniform ? philox_stream_kernel<V, kU, true> : philox_stream_kernel<V, kU, false>;
+      kernel = cross ? philox_stream_kernel<V, kU, true> : philox_stream_kernel<V, kU, false>;
     }
     // resident CTAs per SM, found once per kernel (atomic: launches may come
     // from several host threads)
     static std::atomic<int> occ[2] = {{0}, {0}};
-    int o = occ[hi_uniform ? 1 : 0].load(std::memory_order_relaxed);
+    int o = occ[cross ? 1 : 0].load(std::memory_order_relaxed);
     if (o == 0) {
       o = blocks_per_sm(kernel);
-      occ[hi_uniform ? 1 : 0].store(o, std::memory_order_relaxed);
+      occ[cross ? 1 : 0].store(o, std::memory_order_relaxed);
     }
     const int64_t work = (jl - jf + (int64_t)kU - 1) / kU;
     int64_t grid = (work + kThreads - 1) / kThreads;
@@ -848,8 +835,7 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
       p.gbase = reinterpret_cast<uint4*>(addr - phase_w * 4u);
       p.nw = r.n * (I::es / 4);
       p.h = (int64_t)phase_w;
-      p.rk = philox_round_keys(r.key[0], r.key[1]);
-      launch_rotate<V>(p, r.off_lo, r.off_hi, sms, geom, stream);
+      launch_rotate<V>(p, r.key, r.off_lo, r.off_hi, sms, geom, stream);
     }
   } else if (r.num_streams == 1 &&
              ((phase_w % (uint32_t)I::wpu) == 0 || (I::epu == 2 && (head & 1) != 0))) {
@@ -863,15 +849,14 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
     p.groups = groups;
     p.jf = head > 0 ? 1 : 0;
     p.jl = ((head + r.n) % kEpg) != 0 ? groups - 1 : groups;
-    p.rk = philox_round_keys(r.key[0], r.key[1]);
     if ((phase_w % (uint32_t)I::wpu) == 0) {
-      launch_shift<V, false>(p, lo0, hi0, sms, geom, stream);
+      launch_shift<V, false>(p, r.key, lo0, hi0, sms, geom, stream);
     } else if constexpr (I::epu == 2) {
       // the virtual groups start one element (es / 4 words) earlier
       const uint32_t pv = phase_w + (uint32_t)(I::es / 4);
       const uint64_t a_lo = r.off_lo - pv;
       const uint64_t a_hi = r.off_hi - ((r.off_lo < pv) ? 1u : 0u);
-      launch_shift<V, true>(p, a_lo, a_hi, sms, geom, stream);
+      launch_shift<V, true>(p, r.key, a_lo, a_hi, sms, geom, stream);
     }
   } else {
     // substreams at any other phase or alignment
@@ -908,9 +893,7 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
   return GRNG_OK;
 }
 
-}  // namespace
-
-grng_status launch_philox(const FillRequest& r, CUstream_st* stream) {
+grng_status launch_by_variant(const FillRequest& r, cudaStream_t stream) {
   switch (r.variant) {
     case V_BITS: return launch_variant<V_BITS>(r, stream);
     case V_U01_F32: return launch_variant<V_U01_F32>(r, stream);
@@ -929,6 +912,28 @@ grng_status launch_philox(const FillRequest& r, CUstream_st* stream) {
     case V_STDGAUSS_F64: return launch_variant<V_STDGAUSS_F64>(r, stream);
     default: set_error("unknown variant %d", r.variant); return GRNG_ERR_INVALID_ARG;
   }
+}
+
+}  // namespace
+
+// A single-stream fill counts its blocks in 32 bits: a longer one is launched
+// in pieces of 2^32 elements (at most 2^31 blocks), each a fill of its own at
+// its own word offset.
+grng_status launch_philox(const FillRequest& r, CUstream_st* stream) {
+  constexpr int64_t kPiece = int64_t(1) << 32;
+  if (r.num_streams != 1 || r.n <= kPiece) return launch_by_variant(r, stream);
+  const VariantInfo v = variant_info(r.variant);
+  FillRequest piece = r;
+  for (int64_t at = 0; at < r.n; at += kPiece) {
+    piece.n = (r.n - at) < kPiece ? (r.n - at) : kPiece;
+    piece.out = reinterpret_cast<char*>(r.out) + at * v.es;
+    const uint64_t words = (uint64_t)(at / v.epu) * (uint64_t)v.wpu;
+    piece.off_lo = r.off_lo + words;
+    piece.off_hi = r.off_hi + ((piece.off_lo < words) ? 1u : 0u);
+    const grng_status st = launch_by_variant(piece, stream);
+    if (st != GRNG_OK) return st;
+  }
+  return GRNG_OK;
 }
 
 }  // namespace grng

@@ -502,3 +502,32 @@ def test_mrg_small_fp64_fills_by_row_length(g, var):
             assert out[n:].eq(0).all(), (var[0], n)
             if n <= 1000:
                 assert_parity(kind, dtype, out[:n].cpu().numpy(), ref[:n], f"{var[0]} n {n}")
+
+
+@pytest.mark.parametrize("var", VARIANTS, ids=[v[0] for v in VARIANTS])
+def test_philox_fills_across_a_32_bit_block_carry(g, var):
+    """The low 32 bits of the block counter carry inside the fill (also into the
+    top 64 bits, and out of the 2^126 blocks), just before it and just after
+    it, at every word phase and from an aligned and a misaligned start."""
+    n = 2003
+    for carry in ((1 << 34), (3 << 66), 1 << 128):
+        for back, pofs in ((1204, 0), (1203, 1), (1202, 0), (1201, 1), (9000, 0), (0, 1)):
+            off = (carry - back) % (1 << 128)
+            got = _gpu_fill(g, 0, 2021, off, var, n, ptr_off=pofs)
+            assert_parity(var[1], var[2], got, _ref(0, 2021, off, var, n), f"{var[0]} off {off:#x} ptr+{pofs}")
+
+
+def test_philox_fill_longer_than_one_launch(g):
+    """A fill of more than 2^32 outputs is launched in pieces: windows around
+    the piece boundary and at both ends equal the oracle's, and the engine
+    advances by the whole fill."""
+    n = (1 << 32) + 1003
+    out = torch.empty(n, dtype=torch.int32, device="cuda")
+    e = g.Engine(0, 2021, 7)
+    g.generate(g.Distribution.bits(), e, out)
+    torch.cuda.synchronize()
+    assert e.offset == 7 + n
+    for at in (0, (1 << 32) - 517, n - 401):
+        got = out[at:at + 400 + (at == (1 << 32) - 517) * 700].cpu().numpy().view(np.uint32)
+        ref = oracle.generate(0, 2021, 7 + at, 0, 0, 0.0, 0.0, got.size)
+        assert np.array_equal(got, ref), at
