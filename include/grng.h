@@ -251,7 +251,8 @@ GRNG_API grng_status grng_generate_host(const grng_distribution* dist, grng_engi
                                grng_stream_t stream);
 
 /* ---------------------------------------------------------- fill geometry
- * Launch geometry of grng_generate / grng_generate_substreams, one integer
+ * Launch geometry of grng_generate / grng_generate_substreams (aligned Philox
+ * substreams of 256 groups or more choose their own tiles), one integer
  * per (engine kind, distribution variant, size bucket = bit length of the
  * element count): Philox4x32-10, the CTAs per SM of its grid-stride kernels
  * (1..16: a cap on the resident CTAs; 17..64: value - 16 waves of resident

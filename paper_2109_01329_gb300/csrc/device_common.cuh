@@ -72,7 +72,7 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxRoundKeys& r
   return c;
 }
 
-// The blocks of one single-stream fill: block j has counter base + j, of which
+// The blocks of one stream: block j has counter base + j, of which
 // only the low 32-bit word x varies while no carry leaves it.  The other three
 // words fix the second product of round 0 and with it the first of round 1,
 // so a block costs 18 wide products of the 20 and a 32-bit counter add in
@@ -85,11 +85,12 @@ struct PhiloxUpper {
 struct PhiloxStream {
   uint32_t x0;        // low word of the base counter
   PhiloxUpper s[2];
-  uint32_t k[16];     // round keys of rounds 2..9 (k1 of round 2 is in d)
+  PhiloxRoundKeys rk;
 };
 constexpr uint64_t kPhiloxMaxBlocks = uint64_t(1) << 32;  // blocks of one PhiloxStream
 
-inline PhiloxUpper philox_upper(uint32_t k0, uint32_t k1, uint32_t y, uint32_t z, uint32_t w) {
+__host__ __device__ inline PhiloxUpper philox_upper(uint32_t k0, uint32_t k1, uint32_t y, uint32_t z,
+                                                    uint32_t w) {
   const uint64_t p1 = (uint64_t)kPhiloxM1 * z;                          // round 0, second product
   const uint32_t x1 = (uint32_t)(p1 >> 32) ^ y ^ k0;
   const uint64_t p0 = (uint64_t)kPhiloxM0 * x1;                         // round 1, first product
@@ -113,11 +114,24 @@ inline PhiloxStream philox_stream(uint32_t k0, uint32_t k1, uint64_t base_lo, ui
     lo += uint64_t(1) << 32;
     hi += (lo >> 32) == 0 ? 1u : 0u;
   }
-  for (int r = 2; r < 10; ++r) {
-    p.k[2 * (r - 2)] = k0 + (uint32_t)r * kPhiloxW0;
-    p.k[2 * (r - 2) + 1] = k1 + (uint32_t)r * kPhiloxW1;
-  }
+  p.rk = philox_round_keys(k0, k1);
   return p;
+}
+
+// The block whose low counter word is x, for the upper words of u.
+__device__ __forceinline__ uint4 philox_block(uint32_t x, const PhiloxUpper& u,
+                                              const PhiloxRoundKeys& rk) {
+  uint32_t z1, w1, x2, y2;
+  mul_hi_lo(x, kPhiloxM0, z1, w1);
+  mul_hi_lo(z1 ^ u.e, kPhiloxM1, x2, y2);
+  // round 2, whose fourth counter word is a constant
+  uint32_t hi0, lo0, hi1, lo1;
+  mul_hi_lo(x2 ^ u.a, kPhiloxM0, hi0, lo0);
+  mul_hi_lo(w1 ^ u.b, kPhiloxM1, hi1, lo1);
+  uint4 c = make_uint4(hi1 ^ y2 ^ rk.k[4], lo1, hi0 ^ u.d, lo0);
+#pragma unroll
+  for (int r = 3; r < 10; ++r) c = philox_round(c, rk.k[2 * r], rk.k[2 * r + 1]);
+  return c;
 }
 
 // Block j (j < 2^32); kCross: x0 + j may carry out of 32 bits.
@@ -126,17 +140,7 @@ __device__ __forceinline__ uint4 philox_block(uint32_t j, const PhiloxStream& p)
   const uint32_t x = p.x0 + j;
   PhiloxUpper u = p.s[0];
   if (kCross && x < j) u = p.s[1];
-  uint32_t z1, w1, x2, y2;
-  mul_hi_lo(x, kPhiloxM0, z1, w1);
-  mul_hi_lo(z1 ^ u.e, kPhiloxM1, x2, y2);
-  // round 2, whose fourth counter word is a constant
-  uint32_t hi0, lo0, hi1, lo1;
-  mul_hi_lo(x2 ^ u.a, kPhiloxM0, hi0, lo0);
-  mul_hi_lo(w1 ^ u.b, kPhiloxM1, hi1, lo1);
-  uint4 c = make_uint4(hi1 ^ y2 ^ p.k[0], lo1, hi0 ^ u.d, lo0);
-#pragma unroll
-  for (int r = 3; r < 10; ++r) c = philox_round(c, p.k[2 * (r - 2)], p.k[2 * (r - 2) + 1]);
-  return c;
+  return philox_block(x, u, p.rk);
 }
 
 // Philox counter of a block index given as (lo, hi) 64-bit halves.  Word

@@ -134,6 +134,14 @@ constexpr int blocks_per_thread() {
   return (V == V_BITS || V == V_U01_F32 || V == V_UNI_F32) ? 6 : VInfo<V>::es == 8 ? 1 : 2;
 }
 
+// Substream tiles: eight for bits and the FP32 uniforms (16384 x 16384 uniforms
+// at 4, 6, 8: 169.2, 170.9, 168.8 us), the others as above.
+template <int V>
+constexpr int multi_blocks_per_thread() {
+  return (V == V_BITS || V == V_U01_F32 || V == V_UNI_F32) ? 8 : blocks_per_thread<V>();
+}
+constexpr int64_t kMultiTile = 16 * kThreads;  // groups; at most (8: 5 % slower, 32: idle SMs)
+
 // In the kernels that exchange between lanes the [0, 1) and exact FP64 uniforms
 // take two (10^8 at word offset 1: 0.223 ms against 0.226 with one).
 template <int V>
@@ -505,6 +513,69 @@ __global__ void __launch_bounds__(kThreads) philox_multi_kernel(const __grid_con
   }
 }
 
+// The same for streams of 256 groups or more (512 for the light transforms:
+// 16384 x 1024 FP32 uniforms, 256 groups, take 27.2 us here and 25.5 above): a CTA takes a tile of one stream,
+// so that the stream's counter base (a 128-bit product), its upper words'
+// constants and the position are found once per tile, and its groups go as
+// in the single-stream kernel (one group at a time with 128-bit counters took
+// 90 instructions a block against 64 there).  16384 x 16384: FP32 uniforms
+// 258 -> 169 us (159 in one stream), bits 230 -> 147, FP64 uniforms 540 -> 402,
+// FP32 gaussians 428 -> 311, FP64 gaussians 1791 -> 1656.
+struct MultiTileParams {
+  TransformParams t;
+  uint4* out;
+  uint32_t groups;    // groups per stream
+  uint32_t tile;      // groups per tile
+  uint32_t tps;       // tiles per stream
+  uint64_t base_lo, base_hi;
+  uint64_t sb_lo, sb_hi;  // block-counter stride between streams
+  PhiloxRoundKeys rk;
+};
+
+template <int V, int U>
+__device__ __forceinline__ void philox_multi_tile_body(const MultiTileParams& p) {
+  const uint32_t s = blockIdx.x / p.tps, first = (blockIdx.x - s * p.tps) * p.tile;
+  uint64_t lo = p.base_lo, hi = p.base_hi;  // block counter of group 0 of stream s
+  add128(lo, hi, (uint64_t)s * p.sb_lo, __umul64hi((uint64_t)s, p.sb_lo) + (uint64_t)s * p.sb_hi);
+  const uint32_t x0 = (uint32_t)lo;
+  const PhiloxUpper up = philox_upper(p.rk.k[0], p.rk.k[1], (uint32_t)(lo >> 32), (uint32_t)hi,
+                                      (uint32_t)(hi >> 32) & 0x3FFFFFFFu);
+  // the low word carries inside the stream (the same for the whole CTA)
+  const bool cross = x0 + p.groups < x0;
+  const uint32_t end = p.groups - first < p.tile ? p.groups : first + p.tile;
+  uint32_t j = first + threadIdx.x;
+  uint4* dst = p.out + ((uint64_t)s * p.groups + j);
+  if (cross) {
+    for (; j < end; j += kThreads, dst += kThreads) {
+      uint64_t c_lo = lo, c_hi = hi;
+      add128(c_lo, c_hi, j, 0);
+      *dst = block_outputs<V>(philox4x32_10(ctr_from(c_lo, c_hi), p.rk), p.t);
+    }
+    return;
+  }
+  for (; j + (U - 1) * kThreads < end; j += U * kThreads, dst += U * kThreads) {
+    uint4 o[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      o[u] = block_outputs<V>(philox_block(x0 + j + u * kThreads, up, p.rk), p.t);
+#pragma unroll
+    for (int u = 0; u < U; ++u) dst[u * kThreads] = o[u];
+  }
+  if constexpr (U > 1)
+    for (; j < end; j += kThreads, dst += kThreads)
+      *dst = block_outputs<V>(philox_block(x0 + j, up, p.rk), p.t);
+}
+
+template <int V, int U>
+__global__ void __launch_bounds__(kThreads) philox_multi_tile_kernel(const __grid_constant__ MultiTileParams p) {
+  philox_multi_tile_body<V, U>(p);
+}
+
+template <int V, int U>
+__global__ void __launch_bounds__(kThreads, 5) philox_multi_tile_kernel_5(const __grid_constant__ MultiTileParams p) {
+  philox_multi_tile_body<V, U>(p);
+}
+
 // Substreams at any word phase and pointer alignment: stream s writes
 // out + s n elements from word offset off + s stride, and its 16-byte groups
 // are found as in the shift kernel, per stream.  A warp takes one chunk of
@@ -533,11 +604,13 @@ struct ShiftStream {
   int64_t head;     // elements of group 0 before sbase
   int64_t groups, jf, jl;
   uint64_t b_lo, b_hi;  // block of the first word of (virtual) group 0
+  PhiloxUpper up;       // its upper words' constants
   uint32_t ph;
   bool split;
+  bool cross;           // the low counter word may carry inside the stream
 };
 
-template <int V>
+template <int V, bool kLong>
 __device__ __forceinline__ ShiftStream shift_stream(const MultiShiftParams& p, int64_t s) {
   using I = VInfo<V>;
   constexpr int kEpg = 16 / I::es;
@@ -559,12 +632,19 @@ __device__ __forceinline__ ShiftStream shift_stream(const MultiShiftParams& p, i
   t.b_hi = a_hi >> 2;
   t.ph = (uint32_t)a_lo & 3u;
   t.groups = (t.head + p.n + kEpg - 1) / kEpg;
+  t.cross = !kLong || (uint64_t)(uint32_t)t.b_lo + (uint64_t)t.groups + 32u >= kPhiloxMaxBlocks;
+  if (!t.cross)
+    t.up = philox_upper(p.rk.k[0], p.rk.k[1], (uint32_t)(t.b_lo >> 32), (uint32_t)t.b_hi,
+                        (uint32_t)(t.b_hi >> 32) & 0x3FFFFFFFu);
   t.jf = t.head > 0 ? 1 : 0;
   t.jl = ((t.head + p.n) % kEpg) != 0 ? t.groups - 1 : t.groups;
   return t;
 }
 
-template <int V>
+// kLong: warps take four chunks or more, so that making the upper counter
+// words' constants per stream pays; the short form, whole counters throughout,
+// is also the smaller program (1000 x 1023 FP64 uniforms 9.1 us against 10.8).
+template <int V, bool kLong>
 __global__ void __launch_bounds__(kThreads) philox_multishift_kernel(
     const __grid_constant__ MultiShiftParams p) {
   using I = VInfo<V>;
@@ -582,16 +662,12 @@ __global__ void __launch_bounds__(kThreads) philox_multishift_kernel(
   if (c >= c_end) return;
   int64_t s = c / p.cps;
   int64_t k = c - s * p.cps;
-  ShiftStream t = shift_stream<V>(p, s);
-  for (; c < c_end; ++c) {
-    const int64_t j = k * kPer + lane;
-    const uint64_t c_lo = t.b_lo + (uint64_t)j;
-    const uint64_t c_hi = t.b_hi + ((c_lo < t.b_lo) ? 1u : 0u);
-    const uint4 b = philox4x32_10(ctr_from(c_lo, c_hi), p.rk);
+  ShiftStream t = shift_stream<V, kLong>(p, s);
+  // groups [k kPer, (k + 1) kPer) of the stream, from this lane's block
+  auto emit = [&](int64_t k, int64_t j, uint4 b) {
     // the stream's phase and split are the same for the whole warp, so the
     // exchanges run on all 32 lanes or on none: a stream at phase 0 skips the
-    // word exchange (16384 x 65537 at a stride of 2^40 + 1, half the streams
-    // at phase 0: bits 1.108 -> 1.030 ms, FP32 uniform 1.219 -> 1.145 ms)
+    // word exchange
     uint4 w = b;
     if (t.ph != 0) w = shift_words(b, t.ph);
     uint4 o = block_outputs<V>(w, p.t);
@@ -608,11 +684,29 @@ __global__ void __launch_bounds__(kThreads) philox_multishift_kernel(
         store_partial<V>(t.sbase, e0, p.n, o);
       }
     }
-    if (++k == p.cps) {
-      k = 0;
-      ++s;
-      if (c + 1 < c_end) t = shift_stream<V>(p, s);
+  };
+  while (true) {
+    // the run's chunks in this stream, in a loop of their own where the upper
+    // counter words are fixed (16384 x 16385 at a stride of 2^40 + 1: FP32
+    // uniforms 302 -> 263 us, FP32 gaussians 518 -> 446)
+    const int64_t k_end = k + (c_end - c) < p.cps ? k + (c_end - c) : p.cps;
+    c += k_end - k;
+    if (!t.cross) {
+      for (; k < k_end; ++k) {
+        const int64_t j = k * kPer + lane;
+        emit(k, j, philox_block((uint32_t)t.b_lo + (uint32_t)j, t.up, p.rk));
+      }
+    } else {
+      for (; k < k_end; ++k) {
+        const int64_t j = k * kPer + lane;
+        uint64_t c_lo = t.b_lo, c_hi = t.b_hi;
+        add128(c_lo, c_hi, (uint64_t)j, 0);
+        emit(k, j, philox4x32_10(ctr_from(c_lo, c_hi), p.rk));
+      }
     }
+    if (c >= c_end) return;
+    k = 0;
+    t = shift_stream<V, kLong>(p, ++s);
   }
 }
 
@@ -796,6 +890,36 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
     const int64_t cap = (int64_t)sms * ctas_cap(o, geom);
     if (grid > cap) grid = cap;
     kernel<<<(unsigned)grid, kThreads, 0, stream>>>(p);
+  } else if (fast && head == 0 && (stream_bytes % 16u) == 0 && groups >= (I::weight == 0 ? 2 : 1) * kThreads &&
+             groups <= (int64_t(1) << 31)) {
+    MultiTileParams p;
+    p.t = r.t;
+    p.out = reinterpret_cast<uint4*>(r.out);
+    p.groups = (uint32_t)groups;
+    p.base_lo = base_lo;
+    p.base_hi = base_hi;
+    p.sb_lo = (r.stride_lo >> 2) | (r.stride_hi << 62);
+    p.sb_hi = r.stride_hi >> 2;
+    p.rk = philox_round_keys(r.key[0], r.key[1]);
+    constexpr int kU = multi_blocks_per_thread<V>();
+    // at most kMultiTile, less where the fill is small (8 CTAs per SM at least,
+    // 32 for the longer transforms, whose last wave weighs more), and a
+    // stream's tiles alike
+    const int64_t ctas = (int64_t)sms * (I::weight == 0 ? 8 : 32);
+    int64_t cap = groups * r.num_streams / (ctas * kThreads) * kThreads;
+    if (cap > kMultiTile) cap = kMultiTile;
+    if (cap < kThreads) cap = kThreads;
+    const int64_t tiles = (groups + cap - 1) / cap;
+    const int64_t tile = ((groups + tiles - 1) / tiles + kThreads - 1) / kThreads * kThreads;
+    p.tile = (uint32_t)tile;
+    const int64_t tps = (groups + tile - 1) / tile;
+    p.tps = (uint32_t)tps;
+    const int64_t grid = tps * r.num_streams;
+    if constexpr (stream_wants_5_ctas<V>()) {
+      philox_multi_tile_kernel_5<V, kU><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+    } else {
+      philox_multi_tile_kernel<V, kU><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+    }
   } else if (fast && head == 0 && (stream_bytes % 16u) == 0) {
     MultiParams p;
     p.t = r.t;
@@ -876,14 +1000,15 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
     static std::atomic<int> occ_cache{0};
     int occ = occ_cache.load(std::memory_order_relaxed);
     if (occ == 0) {
-      occ = blocks_per_sm(philox_multishift_kernel<V>);
+      occ = blocks_per_sm(philox_multishift_kernel<V, true>);
       occ_cache.store(occ, std::memory_order_relaxed);
     }
     int64_t grid = (p.total + (kThreads / 32) - 1) / (kThreads / 32);
     const int64_t cap = (int64_t)sms * ctas_cap(occ, geom);
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
-    philox_multishift_kernel<V><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+    const bool is_long = p.total >= 4 * grid * (kThreads / 32);
+    (is_long ? philox_multishift_kernel<V, true> : philox_multishift_kernel<V, false>)<<<(unsigned)grid, kThreads, 0, stream>>>(p);
   }
   const cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) {

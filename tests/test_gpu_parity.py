@@ -531,3 +531,40 @@ def test_philox_fill_longer_than_one_launch(g):
         got = out[at:at + 400 + (at == (1 << 32) - 517) * 700].cpu().numpy().view(np.uint32)
         ref = oracle.generate(0, 2021, 7 + at, 0, 0, 0.0, 0.0, got.size)
         assert np.array_equal(got, ref), at
+
+
+@pytest.mark.parametrize("var", VARIANTS, ids=[v[0] for v in VARIANTS])
+def test_philox_substreams_by_length_and_carry(g, var):
+    """Substreams around the lengths where the kernels change (256 groups, whole
+    and ragged tiles, long runs of chunks per warp), starting before, across and
+    after a carry out of the low 32 bits of the block counter."""
+    _, kind, dtype, p0, p1 = var
+    epg = 2 if dtype == 2 else 4
+    d = g.Distribution(kind, dtype, p0, p1)
+    for groups, extra, stride in ((255, 0, 1 << 40), (256, 0, 1 << 40), (257, 0, 1 << 34), (4096, 0, 1 << 34),
+                                  (4352 + 1, 0, (1 << 76) + 4), (300, 1, 1 << 34), (4400, 1, (1 << 40) + 1)):
+        n, S = groups * epg + extra, 5 if groups < 4000 else 3
+        for off in (0, (1 << 34) - 4 * 200, (1 << 66) - 4 * 3):
+            out = torch.empty(S * n, dtype=_torch_dtype(dtype), device="cuda")
+            g.generate_substreams(d, g.Engine(0, 77, off), out, n, S, stride)
+            torch.cuda.synchronize()
+            host = out.cpu().numpy()
+            for s in range(S):
+                ref = oracle.generate(0, 77, off + s * stride, kind, dtype, p0, p1, n)
+                got = host[s * n:(s + 1) * n]
+                assert_parity(kind, dtype, got.view(np.uint32) if dtype == 0 else got, ref,
+                              f"{var[0]} groups {groups} extra {extra} off {off:#x} stream {s}")
+
+
+def test_philox_multi_shift_long_runs_across_a_carry(g):
+    """Enough odd-length substreams that a warp takes several chunks: the streams
+    whose low block counter word carries equal the oracle's, and so do the others."""
+    S, n, stride = 64, 400_003, 1 << 34
+    off = (1 << 34) - 400_003 // 2
+    out = torch.empty(S * n, dtype=torch.int32, device="cuda")
+    for o in (off, 5):
+        g.generate_substreams(g.Distribution.bits(), g.Engine(0, 77, o), out, n, S, stride)
+        torch.cuda.synchronize()
+        for s in (0, 1, 31, 63):
+            got = out[s * n:(s + 1) * n].cpu().numpy().view(np.uint32)
+            assert np.array_equal(got, oracle.generate(0, 77, o + s * stride, 0, 0, 0.0, 0.0, n)), (o, s)
