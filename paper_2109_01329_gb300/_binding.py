@@ -520,9 +520,10 @@ class Batch:
     requests: list of (engine, distribution, out_tensor[, n]).  The device
     workspace is allocated here as a torch tensor and kept alive with the
     batch; with tunable=True it is sized for ipt = 1, so that autotune() may
-    try every geometry.  launch() enqueues the persistent fill and the
-    device-side offset advance (capturable in a CUDA graph); commit() moves
-    the engines to the device-resident offsets.
+    try every geometry.  launch() enqueues the persistent fill, which counts
+    its launches on the device so that each continues the sequences
+    (capturable in a CUDA graph); commit() moves the engines to where the
+    launches left them.
     """
 
     def __init__(self, requests, ipt: int = 8, stream=None, tunable: bool = True):

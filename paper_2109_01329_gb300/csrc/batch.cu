@@ -6,15 +6,13 @@
 // variant, parameters, output pointer, 16-byte group count and starting word
 // offset; a tile -> request map; and per request the words its engine
 // advances per launch.  The tables live in a caller-provided device
-// workspace.  grng_batch_launch then enqueues two kernels:
-//   1. batch_fill_kernel: CTAs walk the tiles (a tile is kThreads * ipt
-//      16-byte groups of one request) with a static grid stride; each thread
-//      produces ipt groups of its tile;
-//   2. batch_advance_kernel: adds each request's advance to its device-
-//      resident 128-bit offset,
-// so launching again (or replaying a CUDA graph of the launch) continues every
-// generator's sequence with no host work.  grng_batch_commit copies the device
-// offsets back into the engines.
+// workspace.  grng_batch_launch then enqueues one kernel: CTAs walk the tiles (a
+// tile is kThreads * ipt 16-byte groups of one request) with a static grid
+// stride, up to eight at a time, and the last CTA to finish counts the launch in the
+// workspace.  A request's offset is its start plus that count times its
+// advance, so launching again (or replaying a CUDA graph of the launch)
+// continues every generator's sequence with no host work.  grng_batch_commit
+// reads the count and moves the engines.
 //
 // A request whose word offset matches its pointer's 16-byte phase maps each
 // 16-byte group to one Philox block; at any other phase a warp computes 32
@@ -41,8 +39,14 @@ using namespace dev;
 constexpr int kThreads = 256;
 
 // Workspace layout (each part 256-byte aligned):
-//   BatchReq reqs[count] | uint64_t off[count][2] | int32_t tile_req[tiles]
+//   BatchReq reqs[count] | uint64_t off[count][2] | BatchCount | int32_t tile_req[tiles]
 size_t align256(size_t x) { return (x + 255u) & ~(size_t)255u; }
+
+// Launches of a batch so far, and the CTAs of the running one that are done.
+struct BatchCount {
+  uint64_t launches;
+  uint32_t done;
+};
 
 // Stores the elements of group (first element e0) that lie in [0, n).
 template <int V>
@@ -67,61 +71,94 @@ __device__ __forceinline__ void store_group(char* base, int64_t e0, int64_t n, u
   }
 }
 
-// The groups [g0, g0 + kThreads ipt) of one request (the whole CTA works on
-// one tile, so every branch below is uniform across it).  Group 0 starts
-// head elements (pw = head es / 4 words) before the output.  When pw is a
-// multiple of the unit size, group g is the 4 words from word off - pw + 4 g:
-// exactly Philox block (off - pw)/4 + g when off - pw is a multiple of 4,
-// else the tail of one block and the head of the next, exchanged between
-// neighbouring lanes.  Otherwise (a Box-Muller pair split by the output's
-// start) lanes transform pair-aligned virtual groups one element earlier and
-// exchange the straddling element by shuffle.
+// Blocks per thread at once in a tile whose groups are blocks.
 template <int V>
-__device__ __forceinline__ void batch_tile(const BatchReq& r, uint64_t off_lo, uint64_t off_hi,
-                                           int64_t g0, int ipt) {
+constexpr int kTileBlocks = VInfo<V>::es == 8 ? 1 : VInfo<V>::weight == 0 ? 4 : 2;
+
+// The blocks of a tile from block (b_lo, b_hi) on: the round keys and, where
+// the low counter word does not carry inside the tile, the upper words'
+// constants, made once per tile.
+struct TileBlocks {
+  PhiloxRoundKeys rk;
+  PhiloxUpper up;
+  uint64_t b_lo, b_hi;
+  __device__ __forceinline__ TileBlocks(uint32_t k0, uint32_t k1, uint64_t lo, uint64_t hi)
+      : rk(philox_round_keys(k0, k1)),
+        up(philox_upper(k0, k1, (uint32_t)(lo >> 32), (uint32_t)hi,
+                        (uint32_t)(hi >> 32) & 0x3FFFFFFFu)),
+        b_lo(lo),
+        b_hi(hi) {}
+  template <bool kCross>
+  __device__ __forceinline__ uint4 at(uint32_t i) const {
+    if constexpr (!kCross) return philox_block((uint32_t)b_lo + i, up, rk);
+    const uint64_t lo = b_lo + i;
+    return philox4x32_10(ctr_from(lo, b_hi + ((lo < b_lo) ? 1u : 0u)), rk);
+  }
+};
+
+// A tile's groups: `count` from group 0 at dst, those of [wf, wl) whole inside the
+// request, at most the first and the last not; the first element of group 0 is
+// element e0 of the request.
+struct TileOut {
+  uint4* dst;
+  uint32_t count, wf, wl;
+  char* base;
+  int64_t e0, n;
+};
+
+template <int V>
+__device__ __forceinline__ void tile_store(const TileOut& o, uint32_t i, uint4 v) {
+  if (i >= o.wf && i < o.wl) {
+    o.dst[i] = v;
+  } else {
+    store_group<V>(o.base, o.e0 + (int64_t)i * (16 / VInfo<V>::es), o.n, v);
+  }
+}
+
+// Group i is block i.
+template <int V>
+__device__ __forceinline__ void tile_blocks_loop(const TransformParams& t, const TileBlocks& q,
+                                                 const TileOut& out) {
+  constexpr uint32_t U = kTileBlocks<V>;
+  if (threadIdx.x < 2) {  // the groups that are not whole
+    const uint32_t i = threadIdx.x == 0 ? 0u : out.count - 1u;
+    if ((i < out.wf || i >= out.wl) && (threadIdx.x == 0 || out.count > 1))
+      tile_store<V>(out, i, block_outputs<V>(q.at<false>(i), t));
+  }
+  uint32_t i = out.wf + threadIdx.x;
+  uint4* dst = out.dst + i;
+  for (; i + (U - 1) * kThreads < out.wl; i += U * kThreads, dst += U * kThreads) {
+    uint4 o[U];
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) o[u] = block_outputs<V>(q.at<false>(i + u * kThreads), t);
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) dst[u * kThreads] = o[u];
+  }
+  if constexpr (U > 1)
+    for (; i < out.wl; i += kThreads, dst += kThreads) *dst = block_outputs<V>(q.at<false>(i), t);
+}
+
+// The same where a group straddles two blocks (word phase ph), where the low
+// counter word carries (kCross; any ph) or, kSplit, where the output's start
+// splits a Box-Muller pair (an odd head; any ph): a warp computes 32
+// consecutive blocks and emits 31 or 30 groups, exchanging the straddling
+// words, and elements, between neighbouring lanes as in the single-stream
+// shift kernel.  The loop bound depends only on the warp, so every shuffle has
+// all 32 lanes.
+template <int V, bool kCross, bool kSplit>
+__device__ __forceinline__ void tile_shift_loop(const TransformParams& t, const TileBlocks& q,
+                                                uint32_t ph, const TileOut& out) {
   using I = VInfo<V>;
-  constexpr int kEpg = 16 / I::es;
-  constexpr int kWpu = I::wpu, kEpu = I::epu;
-  const int64_t n = r.n, groups = r.groups, head = r.head;
-  const uint32_t k0 = r.key0, k1 = r.key1;
-  char* base = reinterpret_cast<char*>(r.out);
-  const TransformParams t = r.t;
-  const uint32_t pw = (uint32_t)head * (uint32_t)(I::es / 4);
-  if ((pw % (uint32_t)kWpu) == 0) {
-    // group g is the 4 words from word off - pw + 4 g: the block of that
-    // word from phase ph on, and the first ph words of the next block
-    const uint64_t a_lo = off_lo - pw, a_hi = off_hi - ((off_lo < pw) ? 1u : 0u);
-    const uint64_t b_lo = (a_lo >> 2) | (a_hi << 62), b_hi = a_hi >> 2;
-    const uint32_t ph = (uint32_t)a_lo & 3u;
-    if (ph == 0) {
-      for (int i = 0; i < ipt; ++i) {
-        const int64_t g = g0 + (int64_t)i * kThreads + threadIdx.x;
-        if (g >= groups) break;
-        const uint64_t c_lo = b_lo + (uint64_t)g;
-        const uint64_t c_hi = b_hi + ((c_lo < b_lo) ? 1u : 0u);
-        const uint4 o = block_outputs<V>(philox4x32_10(ctr_from(c_lo, c_hi), k0, k1), t);
-        store_group<V>(base, g * kEpg - head, n, o);
-      }
-      return;
-    }
-    // Each warp computes 32 consecutive blocks and emits the 31 groups that
-    // start in its lanes 0..30, taking the next block's words from lane + 1
-    // by shuffle: no shared memory and no barrier.  The loop bound depends
-    // only on the warp, so every shuffle has all 32 lanes.
-    const int lane = threadIdx.x & 31;
-    const int64_t g_end = (g0 + (int64_t)kThreads * ipt) < groups ? (g0 + (int64_t)kThreads * ipt)
-                                                                   : groups;
-    constexpr int kPerWarp = 31;
-    for (int64_t gs = g0 + (int64_t)(threadIdx.x >> 5) * kPerWarp; gs < g_end;
-         gs += (int64_t)kPerWarp * (kThreads / 32)) {
-      const int64_t g = gs + lane;
-      const uint64_t c_lo = b_lo + (uint64_t)g;
-      const uint64_t c_hi = b_hi + ((c_lo < b_lo) ? 1u : 0u);
-      const uint4 b = philox4x32_10(ctr_from(c_lo, c_hi), k0, k1);
+  constexpr uint32_t kPerWarp = kSplit ? 30 : 31;
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t c = (threadIdx.x >> 5) * kPerWarp; c < out.count; c += kPerWarp * (kThreads / 32)) {
+    const uint32_t i = c + lane;
+    const uint4 b = q.at<kCross>(i);
+    uint4 w = b;
+    if ((!kSplit && !kCross) || ph != 0) {
       const uint32_t n0 = __shfl_down_sync(0xFFFFFFFFu, b.x, 1);
       const uint32_t n1 = __shfl_down_sync(0xFFFFFFFFu, b.y, 1);
       const uint32_t n2 = __shfl_down_sync(0xFFFFFFFFu, b.z, 1);
-      uint4 w;
       if (ph == 1) {
         w = make_uint4(b.y, b.z, b.w, n0);
       } else if (ph == 2) {
@@ -129,92 +166,156 @@ __device__ __forceinline__ void batch_tile(const BatchReq& r, uint64_t off_lo, u
       } else {
         w = make_uint4(b.w, n0, n1, n2);
       }
-      if (lane < kPerWarp && g < g_end) store_group<V>(base, g * kEpg - head, n, block_outputs<V>(w, t));
     }
-    return;
-  }
-  if constexpr (kEpu == 2) {
-    // A Box-Muller pair split by the output's start (odd head): virtual group
-    // g starts one element before output group g, on a pair boundary, at
-    // word off - pw - es / 4 + 4 g.  Each lane transforms its virtual group
-    // (words from its block and, at a non-zero phase, the next lane's) and
-    // output group g is virtual group g without its first element plus the
-    // first element of virtual group g + 1, taken from lane + 1: 30 groups
-    // per warp, every pair transformed once, no shared memory.
-    constexpr uint32_t kPv = (uint32_t)(I::es / 4);
-    const uint64_t a_lo = off_lo - (pw + kPv);
-    const uint64_t a_hi = off_hi - ((off_lo < (uint64_t)(pw + kPv)) ? 1u : 0u);
-    const uint64_t b_lo = (a_lo >> 2) | (a_hi << 62), b_hi = a_hi >> 2;
-    const uint32_t ph = (uint32_t)a_lo & 3u;
-    const int lane = threadIdx.x & 31;
-    const int64_t g_end = (g0 + (int64_t)kThreads * ipt) < groups ? (g0 + (int64_t)kThreads * ipt)
-                                                                   : groups;
-    constexpr int kPerWarp = 30;
-    for (int64_t gs = g0 + (int64_t)(threadIdx.x >> 5) * kPerWarp; gs < g_end;
-         gs += (int64_t)kPerWarp * (kThreads / 32)) {
-      const int64_t g = gs + lane;
-      const uint64_t c_lo = b_lo + (uint64_t)g;
-      const uint64_t c_hi = b_hi + ((c_lo < b_lo) ? 1u : 0u);
-      const uint4 b = philox4x32_10(ctr_from(c_lo, c_hi), k0, k1);
-      const uint32_t n0 = __shfl_down_sync(0xFFFFFFFFu, b.x, 1);
-      const uint32_t n1 = __shfl_down_sync(0xFFFFFFFFu, b.y, 1);
-      const uint32_t n2 = __shfl_down_sync(0xFFFFFFFFu, b.z, 1);
-      uint4 w = b;
-      if (ph == 1) {
-        w = make_uint4(b.y, b.z, b.w, n0);
-      } else if (ph == 2) {
-        w = make_uint4(b.z, b.w, n0, n1);
-      } else if (ph == 3) {
-        w = make_uint4(b.w, n0, n1, n2);
-      }
-      const uint4 v = block_outputs<V>(w, t);
-      const uint32_t m0 = __shfl_down_sync(0xFFFFFFFFu, v.x, 1);
-      const uint32_t m1 = __shfl_down_sync(0xFFFFFFFFu, v.y, 1);
-      const uint4 o = I::es == 4 ? make_uint4(v.y, v.z, v.w, m0) : make_uint4(v.z, v.w, m0, m1);
-      if (lane < kPerWarp && g < g_end) store_group<V>(base, g * kEpg - head, n, o);
+    uint4 o = block_outputs<V>(w, t);
+    if constexpr (kSplit) {
+      const uint32_t m0 = __shfl_down_sync(0xFFFFFFFFu, o.x, 1);
+      const uint32_t m1 = __shfl_down_sync(0xFFFFFFFFu, o.y, 1);
+      o = I::es == 4 ? make_uint4(o.y, o.z, o.w, m0) : make_uint4(o.z, o.w, m0, m1);
     }
+    if (lane < kPerWarp && i < out.count) tile_store<V>(out, i, o);
   }
 }
 
-__global__ void __launch_bounds__(kThreads) batch_fill_kernel(const BatchReq* __restrict__ reqs,
+// The groups [g0, end) of one request (the whole CTA works on them, so every
+// branch below is uniform across it).  Group 0 starts head elements (pw =
+// head es / 4 words) before the output.  When pw is a multiple of the unit
+// size, group g is the 4 words from word off - pw + 4 g: exactly Philox block
+// (off - pw)/4 + g when off - pw is a multiple of 4, else the tail of one
+// block and the head of the next.  Otherwise (a Box-Muller pair split by the
+// output's start) lanes transform pair-aligned virtual groups one element
+// earlier.
+template <int V>
+__device__ __forceinline__ void batch_tile(const BatchReq& r, uint64_t off_lo, uint64_t off_hi,
+                                           int64_t g0, int64_t end) {
+  using I = VInfo<V>;
+  constexpr int kEpg = 16 / I::es;
+  const TransformParams& t = r.t;
+  const uint32_t pw = (uint32_t)r.head * (uint32_t)(I::es / 4);
+  const bool split = I::epu == 2 && (pw % (uint32_t)I::wpu) != 0;
+  // word of (virtual) group 0, and the block of group g0's first word
+  const uint32_t back = pw + (split ? (uint32_t)(I::es / 4) : 0u);
+  const uint64_t a_lo = off_lo - back, a_hi = off_hi - ((off_lo < back) ? 1u : 0u);
+  const uint32_t ph = (uint32_t)a_lo & 3u;
+  uint64_t b_lo = (a_lo >> 2) | (a_hi << 62), b_hi = a_hi >> 2;
+  add128(b_lo, b_hi, (uint64_t)g0);
+  TileOut out;
+  out.base = reinterpret_cast<char*>(r.out);
+  out.n = r.n;
+  out.count = (uint32_t)(end - g0);
+  out.e0 = g0 * kEpg - r.head;
+  out.dst = reinterpret_cast<uint4*>(out.base + out.e0 * I::es);
+  out.wf = out.e0 < 0 ? 1u : 0u;
+  out.wl = out.e0 + (end - g0) * kEpg <= r.n ? out.count : out.count - 1u;
+  const bool cross = (uint64_t)(uint32_t)b_lo + out.count + 64u >= kPhiloxMaxBlocks;
+  const TileBlocks q(r.key0, r.key1, b_lo, b_hi);
+  if (I::epu == 2 && split) {
+    if constexpr (I::epu == 2) {
+      if (!cross) {
+        tile_shift_loop<V, false, true>(t, q, ph, out);
+      } else {
+        tile_shift_loop<V, true, true>(t, q, ph, out);
+      }
+    }
+  } else if (cross) {
+    tile_shift_loop<V, true, false>(t, q, ph, out);
+  } else if (ph == 0) {
+    tile_blocks_loop<V>(t, q, out);
+  } else {
+    tile_shift_loop<V, false, false>(t, q, ph, out);
+  }
+}
+
+// One kernel for all variants of a batch; kHeavy also those of the FP64
+// fixed-point transforms, whose registers a batch without them need not carry.
+// Bound by issue and the FMA-heavy pipe (bits: 59 instructions per group, 44 in
+// the single-stream kernel; the rest is the set-up per run of tiles and
+// fewer blocks in flight).  The table of 4096 requests at the built-in geometry:
+// 858 -> 603 us a launch (five CTAs per SM, 48 registers and 376 bytes spilled:
+// 5 % slower than four).
+template <bool kHeavy>
+__global__ void __launch_bounds__(kThreads, 4) batch_fill_kernel(const BatchReq* __restrict__ reqs,
                                                               const uint64_t* __restrict__ off,
                                                               const int32_t* __restrict__ tile_req,
-                                                              int64_t tiles, int ipt) {
-  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int32_t ri = tile_req[t];
-    const BatchReq& r = reqs[ri];
-    const uint64_t off_lo = off[2 * ri], off_hi = off[2 * ri + 1];
-    const int64_t g0 = (t - r.first_tile) * (int64_t)kThreads * ipt;
-    switch (r.variant) {  // uniform per tile
-      case V_BITS: batch_tile<V_BITS>(r, off_lo, off_hi, g0, ipt); break;
-      case V_U01_F32: batch_tile<V_U01_F32>(r, off_lo, off_hi, g0, ipt); break;
-      case V_UNI_F32: batch_tile<V_UNI_F32>(r, off_lo, off_hi, g0, ipt); break;
-      case V_U01_F64: batch_tile<V_U01_F64>(r, off_lo, off_hi, g0, ipt); break;
-      case V_AFF_F64: batch_tile<V_AFF_F64>(r, off_lo, off_hi, g0, ipt); break;
-      case V_UNI_F64: batch_tile<V_UNI_F64>(r, off_lo, off_hi, g0, ipt); break;
-      case V_GAUSS_F32: batch_tile<V_GAUSS_F32>(r, off_lo, off_hi, g0, ipt); break;
-      case V_LOGN_F32: batch_tile<V_LOGN_F32>(r, off_lo, off_hi, g0, ipt); break;
-      case V_GAUSS_F64: batch_tile<V_GAUSS_F64>(r, off_lo, off_hi, g0, ipt); break;
-      case V_LOGN_F64: batch_tile<V_LOGN_F64>(r, off_lo, off_hi, g0, ipt); break;
-      case V_ICDF_GAUSS_F32: batch_tile<V_ICDF_GAUSS_F32>(r, off_lo, off_hi, g0, ipt); break;
-      case V_ICDF_LOGN_F32: batch_tile<V_ICDF_LOGN_F32>(r, off_lo, off_hi, g0, ipt); break;
-      case V_ICDF_GAUSS_F64: batch_tile<V_ICDF_GAUSS_F64>(r, off_lo, off_hi, g0, ipt); break;
-      case V_STDGAUSS_F64: batch_tile<V_STDGAUSS_F64>(r, off_lo, off_hi, g0, ipt); break;
-      default: batch_tile<V_ICDF_LOGN_F64>(r, off_lo, off_hi, g0, ipt); break;
+                                                              int64_t tiles, int ipt, int run,
+                                                              BatchCount* count, bool advance) {
+  const uint64_t launches = count != nullptr ? count->launches : 0;
+  // a CTA takes `run` consecutive tiles at a time; those of one request are
+  // one longer tile, so that a request's set-up is shared
+  for (int64_t t0 = (int64_t)blockIdx.x * run; t0 < tiles; t0 += (int64_t)gridDim.x * run) {
+    const int64_t t1 = t0 + run < tiles ? t0 + run : tiles;
+    for (int64_t t = t0; t < t1;) {
+      const int32_t ri = tile_req[t];
+      const BatchReq& r = reqs[ri];
+      uint64_t off_lo = off[2 * ri], off_hi = off[2 * ri + 1];
+      {
+        const uint64_t add = r.adv_lo * launches;
+        off_lo += add;
+        off_hi += r.adv_hi * launches + __umul64hi(r.adv_lo, launches) + (off_lo < add ? 1u : 0u);
+      }
+      const int64_t tile = (int64_t)kThreads * ipt;
+      const int64_t g0 = (t - r.first_tile) * tile;
+      const int64_t left = (r.groups - g0 + tile - 1) / tile;
+      const int64_t m = t1 - t < left ? t1 - t : left;
+      const int64_t end = g0 + m * tile < r.groups ? g0 + m * tile : r.groups;
+      t += m;
+      switch (r.variant) {  // uniform per tile
+        case V_BITS: batch_tile<V_BITS>(r, off_lo, off_hi, g0, end); break;
+        case V_U01_F32: batch_tile<V_U01_F32>(r, off_lo, off_hi, g0, end); break;
+        case V_UNI_F32: batch_tile<V_UNI_F32>(r, off_lo, off_hi, g0, end); break;
+        case V_U01_F64: batch_tile<V_U01_F64>(r, off_lo, off_hi, g0, end); break;
+        case V_AFF_F64: batch_tile<V_AFF_F64>(r, off_lo, off_hi, g0, end); break;
+        case V_UNI_F64: batch_tile<V_UNI_F64>(r, off_lo, off_hi, g0, end); break;
+        case V_GAUSS_F32: batch_tile<V_GAUSS_F32>(r, off_lo, off_hi, g0, end); break;
+        case V_LOGN_F32: batch_tile<V_LOGN_F32>(r, off_lo, off_hi, g0, end); break;
+        case V_ICDF_GAUSS_F32: batch_tile<V_ICDF_GAUSS_F32>(r, off_lo, off_hi, g0, end); break;
+        case V_ICDF_LOGN_F32: batch_tile<V_ICDF_LOGN_F32>(r, off_lo, off_hi, g0, end); break;
+        default:
+          if constexpr (kHeavy) {
+            switch (r.variant) {
+              case V_GAUSS_F64: batch_tile<V_GAUSS_F64>(r, off_lo, off_hi, g0, end); break;
+              case V_LOGN_F64: batch_tile<V_LOGN_F64>(r, off_lo, off_hi, g0, end); break;
+              case V_ICDF_GAUSS_F64: batch_tile<V_ICDF_GAUSS_F64>(r, off_lo, off_hi, g0, end); break;
+              case V_STDGAUSS_F64: batch_tile<V_STDGAUSS_F64>(r, off_lo, off_hi, g0, end); break;
+              default: batch_tile<V_ICDF_LOGN_F64>(r, off_lo, off_hi, g0, end); break;
+            }
+          }
+          break;
+      }
     }
   }
-}
-
-__global__ void batch_advance_kernel(const BatchReq* __restrict__ reqs, uint64_t* off,
-                                     int32_t count) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const uint64_t lo = off[2 * i] + reqs[i].adv_lo;
-  off[2 * i + 1] += reqs[i].adv_hi + ((lo < off[2 * i]) ? 1u : 0u);
-  off[2 * i] = lo;
+  // every thread of the grid has read the launch count by the time the last
+  // CTA arrives: it counts this launch (a kernel of its own for the offsets took
+  // 2.5 us a launch)
+  if (count != nullptr && advance) {
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&count->done, 1u) == gridDim.x - 1) {
+      count->done = 0;
+      count->launches = launches + 1;
+    }
+  }
 }
 
 }  // namespace
+
+// Consecutive tiles a CTA takes at a time: up to eight, while that leaves 16
+// such runs per SM (at 8 groups per thread, runs of at most 1, 4, 8: 4096
+// requests 683, 610, 590 us; 1024 requests at most 4, 8: 151, 153).
+static int run_of(int64_t tiles) {
+  int dev = 0;
+  const int64_t r = tiles / ((int64_t)current_device_sms(&dev) * 16);
+  return (int)(r < 1 ? 1 : r < 8 ? r : 8);
+}
+
+static void launch_tiles(const BatchReq* reqs, const uint64_t* offs, const int32_t* tile_req,
+                         int64_t tiles, int ipt, bool heavy, int64_t grid, BatchCount* count,
+                         bool advance, cudaStream_t stream) {
+  const int run = run_of(tiles);
+  if (grid > (tiles + run - 1) / run) grid = (tiles + run - 1) / run;
+  if (grid < 1) grid = 1;
+  (heavy ? batch_fill_kernel<true> : batch_fill_kernel<false>)<<<(unsigned)grid, kThreads, 0, stream>>>(
+      reqs, offs, tile_req, tiles, ipt, run, count, advance);
+}
 
 int64_t plan_parts(const PartDesc* parts, int32_t count, int ipt, BatchReq* reqs_out,
                    uint64_t* offs_out, int32_t* tiles_out, int64_t tile_cap) {
@@ -247,11 +348,9 @@ int64_t plan_parts(const PartDesc* parts, int32_t count, int ipt, BatchReq* reqs
 }
 
 grng_status enqueue_fill(const BatchReq* d_reqs, const uint64_t* d_offs, const int32_t* d_tiles,
-                         int64_t tiles, int ipt, int64_t grid, cudaStream_t stream) {
+                         int64_t tiles, int ipt, bool heavy, int64_t grid, cudaStream_t stream) {
   if (tiles <= 0) return GRNG_OK;
-  if (grid > tiles) grid = tiles;
-  if (grid < 1) grid = 1;
-  batch_fill_kernel<<<(unsigned)grid, kThreads, 0, stream>>>(d_reqs, d_offs, d_tiles, tiles, ipt);
+  launch_tiles(d_reqs, d_offs, d_tiles, tiles, ipt, heavy, grid, nullptr, false, stream);
   const cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) {
     set_error("batch fill launch failed: %s", cudaGetErrorString(err));
@@ -267,11 +366,12 @@ struct grng_batch {
   int64_t tiles;
   int32_t ipt;           // groups per thread per tile
   int32_t ctas_per_sm;
+  bool heavy;            // some request takes an FP64 fixed-point transform
   int32_t sms;
   int32_t device;
   void* workspace;
   size_t workspace_bytes;
-  size_t reqs_off, offs_off, tiles_off;
+  size_t reqs_off, offs_off, count_off, tiles_off;
   std::vector<grng::BatchReq> host_reqs;  // the request records as uploaded
   std::vector<int64_t> groups;            // per request
   int64_t groups_total;
@@ -347,7 +447,7 @@ grng_status grng_batch_workspace_bytes(const grng_request* reqs, int32_t count, 
   grng_status st = plan_sizes(reqs, count, ipt, &tiles, &groups, &heads, &variants, &tps);
   if (st != GRNG_OK) return st;
   *bytes = align256(sizeof(BatchReq) * (size_t)count) + align256(16u * (size_t)count) +
-           align256(4u * (size_t)(tiles > 0 ? tiles : 1));
+           align256(sizeof(BatchCount)) + align256(4u * (size_t)(tiles > 0 ? tiles : 1));
   return GRNG_OK;
 }
 
@@ -381,12 +481,15 @@ grng_status grng_batch_create(grng_batch_t* out, const grng_request* reqs, int32
   b->count = count;
   b->tiles = tiles;
   b->ipt = ipt;
-  b->ctas_per_sm = 4;
+  b->ctas_per_sm = 32;  // resident CTAs eight times over, so that the SMs refill
+  b->heavy = false;
+  for (int v : variants) b->heavy = b->heavy || variant_is_heavy(v);
   b->sms = current_device_sms(&b->device);
   b->workspace = dev_workspace;
   b->reqs_off = 0;
   b->offs_off = align256(sizeof(BatchReq) * (size_t)count);
-  b->tiles_off = b->offs_off + align256(16u * (size_t)count);
+  b->count_off = b->offs_off + align256(16u * (size_t)count);
+  b->tiles_off = b->count_off + align256(sizeof(BatchCount));
   b->groups_total = 0;
 
   // Requests of one engine follow each other in its sequence, in table order.
@@ -466,6 +569,8 @@ grng_status grng_batch_create(grng_batch_t* out, const grng_request* reqs, int32
   if (err == cudaSuccess)
     err = cudaMemcpyAsync(ws + b->offs_off, offs.data(), 16u * (size_t)count,
                           cudaMemcpyHostToDevice, (cudaStream_t)stream);
+  if (err == cudaSuccess)
+    err = cudaMemsetAsync(ws + b->count_off, 0, sizeof(BatchCount), (cudaStream_t)stream);
   if (err == cudaSuccess && tiles > 0)
     err = cudaMemcpyAsync(ws + b->tiles_off, tile_req.data(), 4u * (size_t)tiles,
                           cudaMemcpyHostToDevice, (cudaStream_t)stream);
@@ -514,7 +619,7 @@ grng_status replan(grng_batch* b, int ipt, cudaStream_t stream) {
     for (int64_t k = 0; k < nt; ++k) tile_req[(size_t)(t + k)] = i;
     t += nt;
   }
-  // the offsets are not touched: the device copy is the live one
+  // the launch count is not touched: the device copy is the live one
   char* ws = reinterpret_cast<char*>(b->workspace);
   cudaError_t err = cudaMemcpyAsync(ws + b->reqs_off, h.data(), sizeof(BatchReq) * h.size(),
                                     cudaMemcpyHostToDevice, stream);
@@ -556,16 +661,11 @@ grng_status grng_batch_set_config(grng_batch_t b, int32_t ipt, int32_t ctas_per_
 static grng_status batch_enqueue(grng_batch_t b, cudaStream_t stream, bool advance) {
   char* ws = reinterpret_cast<char*>(b->workspace);
   const BatchReq* reqs = reinterpret_cast<const BatchReq*>(ws + b->reqs_off);
-  uint64_t* offs = reinterpret_cast<uint64_t*>(ws + b->offs_off);
+  const uint64_t* offs = reinterpret_cast<const uint64_t*>(ws + b->offs_off);
   const int32_t* tile_req = reinterpret_cast<const int32_t*>(ws + b->tiles_off);
-  if (b->tiles > 0) {
-    int64_t grid = (int64_t)b->sms * b->ctas_per_sm;
-    if (grid > b->tiles) grid = b->tiles;
-    batch_fill_kernel<<<(unsigned)grid, kThreads, 0, stream>>>(reqs, offs, tile_req, b->tiles,
-                                                               b->ipt);
-  }
-  if (advance)
-    batch_advance_kernel<<<(b->count + 255) / 256, 256, 0, stream>>>(reqs, offs, b->count);
+  if (b->tiles > 0)
+    launch_tiles(reqs, offs, tile_req, b->tiles, b->ipt, b->heavy, (int64_t)b->sms * b->ctas_per_sm,
+                 reinterpret_cast<BatchCount*>(ws + b->count_off), advance, stream);
   const cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) {
     set_error("batch launch failed: %s", cudaGetErrorString(err));
@@ -590,7 +690,7 @@ grng_status grng_batch_autotune(grng_batch_t b, grng_stream_t stream_in, int32_t
   }
   cudaStream_t stream = (cudaStream_t)stream_in;
   const int32_t ipts[] = {1, 2, 4, 8, 16, 32};
-  const int32_t ctas[] = {1, 2, 4, 6, 8, 12, 16};
+  const int32_t ctas[] = {1, 2, 4, 6, 8, 12, 16, 24, 32};
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     set_error("event creation failed");
@@ -643,24 +743,28 @@ grng_status grng_batch_commit(grng_batch_t b, grng_stream_t stream) {
     set_error("batch is NULL");
     return GRNG_ERR_INVALID_ARG;
   }
-  std::vector<uint64_t> offs(2 * (size_t)b->count);
+  BatchCount done;
   const char* ws = reinterpret_cast<const char*>(b->workspace);
-  cudaError_t err = cudaMemcpyAsync(offs.data(), ws + b->offs_off, 16u * (size_t)b->count,
-                                    cudaMemcpyDeviceToHost, (cudaStream_t)stream);
+  cudaError_t err = cudaMemcpyAsync(&done, ws + b->count_off, sizeof(done), cudaMemcpyDeviceToHost,
+                                    (cudaStream_t)stream);
   if (err == cudaSuccess) err = cudaStreamSynchronize((cudaStream_t)stream);
   if (err != cudaSuccess) {
     set_error("batch commit failed: %s", cudaGetErrorString(err));
     cudaGetLastError();
     return GRNG_ERR_CUDA;
   }
-  // an engine continues where the device offset of its first request points
-  // (its start plus the launches' advances): skip it ahead to that offset
+  // an engine continues at its first request's start plus the launches'
+  // advances: skip it ahead to that offset
   for (int32_t i = 0; i < b->count; ++i) {
     if (b->first_req_of_engine[i] != i) continue;
     grng_engine_state es;
     grng_engine_get_state(b->engines[i], &es);
-    const uint64_t d_lo = offs[2 * i] - es.offset_lo;
-    const uint64_t d_hi = offs[2 * i + 1] - es.offset_hi - ((offs[2 * i] < es.offset_lo) ? 1u : 0u);
+    const BatchReq& r = b->host_reqs[i];
+    const unsigned __int128 at =
+        (((unsigned __int128)b->start_hi[i] << 64) | b->start_lo[i]) +
+        (((unsigned __int128)r.adv_hi << 64) | r.adv_lo) * done.launches;
+    const unsigned __int128 skip = at - (((unsigned __int128)es.offset_hi << 64) | es.offset_lo);
+    const uint64_t d_lo = (uint64_t)skip, d_hi = (uint64_t)(skip >> 64);
     grng_engine_skip_ahead(b->engines[i], d_lo, d_hi);
   }
   return GRNG_OK;

@@ -50,6 +50,12 @@ inline VariantInfo variant_info(int v) {
   }
 }
 
+// The FP64 fixed-point transforms (hundreds of instructions per unit).
+inline bool variant_is_heavy(int v) {
+  return v == V_GAUSS_F64 || v == V_LOGN_F64 || v == V_STDGAUSS_F64 || v == V_ICDF_GAUSS_F64 ||
+         v == V_ICDF_LOGN_F64;
+}
+
 // Distribution parameters as the kernels use them.
 struct TransformParams {
   float fa, fd, fb, fbprev;   // F32 uniform: a, b - a, b, largest float below b
@@ -119,9 +125,10 @@ struct PartDesc {
 int64_t plan_parts(const PartDesc* parts, int32_t count, int ipt, BatchReq* reqs_out,
                    uint64_t* offs_out, int32_t* tiles_out, int64_t tile_cap);
 
-// Enqueues the batched fill over device copies of those tables.
+// Enqueues the batched fill over device copies of those tables; heavy: some
+// part's variant is heavy.
 grng_status enqueue_fill(const BatchReq* d_reqs, const uint64_t* d_offs, const int32_t* d_tiles,
-                         int64_t tiles, int ipt, int64_t grid, CUstream_st* stream);
+                         int64_t tiles, int ipt, bool heavy, int64_t grid, CUstream_st* stream);
 
 // Kernel launchers; return GRNG_OK or GRNG_ERR_CUDA (detail via set_error).
 grng_status launch_philox(const FillRequest& r, CUstream_st* stream);

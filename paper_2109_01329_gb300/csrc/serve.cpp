@@ -253,6 +253,7 @@ void scheduler(grng_server* S) {
     S->batches += 1;
     S->batch_reqs += (int64_t)batch.size();
     parts.clear();
+    bool heavy = false;
     for (uint64_t t : batch) {
       const Req& r = S->reqs[t];
       uint64_t lo = r.spec.offset_lo, hi = r.spec.offset_hi;
@@ -265,6 +266,7 @@ void scheduler(grng_server* S) {
         d.off_lo = lo;
         d.off_hi = hi;
         fill_transform_params(&sp.dist, &d.t, &d.variant);
+        heavy = heavy || variant_is_heavy(d.variant);
         d.es = sp.dist.dtype == GRNG_F64 ? 8 : 4;
         d.n = sp.n;
         d.out = (uint64_t)(uintptr_t)(S->out_base + r.off + r.part_off[k]);
@@ -289,7 +291,7 @@ void scheduler(grng_server* S) {
       err = cudaMemcpyAsync(slot->d_tiles, slot->h_tiles, 4u * (size_t)tiles,
                             cudaMemcpyHostToDevice, slot->stream);
     if (err == cudaSuccess &&
-        enqueue_fill(slot->d_reqs, slot->d_offs, slot->d_tiles, tiles, kIpt, S->grid,
+        enqueue_fill(slot->d_reqs, slot->d_offs, slot->d_tiles, tiles, kIpt, heavy, S->grid,
                      slot->stream) != GRNG_OK)
       err = cudaErrorLaunchFailure;
     if (err == cudaSuccess) err = cudaLaunchHostFunc(slot->stream, on_batch_done, slot);

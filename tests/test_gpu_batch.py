@@ -230,3 +230,33 @@ def test_set_config_refuses_a_map_that_does_not_fit(g):
     b.set_config(16, 4)  # larger tiles: a smaller map, fits
     with pytest.raises(g.GrngError):
         b.set_config(1, 4)
+
+
+@pytest.mark.parametrize("heavy", [False, True])
+def test_launches_continue_across_carries_and_tile_runs(g, heavy):
+    """Requests long enough for runs of several tiles, starting before, across and
+    after a carry out of the low 32 bits of the block counter, at every word
+    phase and from misaligned outputs: each of three launches equals the
+    per-request calls bit for bit, and commit moves the engines by all three.
+    Without the FP64 fixed-point transforms the lighter kernel takes them."""
+    dists = [(0, 0), (1, 1), (1, 2), (2, 1), (3, 1), (4, 1)] + ([(2, 2), (3, 2), (4, 2)] if heavy else [])
+    reqs, refs = [], []
+    for i, (kind, dtype) in enumerate(dists * 4):
+        n = (3, 1001, 8191 * 4 + 1, 300_003)[i // len(dists)]
+        off = ((1 << 34) - 2 * n + i, (1 << 66) - n // 2 - i, i, 5 + i)[i % 4]
+        d = g.Distribution(kind, dtype, 0.0, 1.0 if kind else 0.0)
+        buf = torch.zeros(n + 4, dtype=TDT[dtype], device="cuda")
+        reqs.append((g.Engine(0, 100 + i, off), d, buf[i % 3:i % 3 + n]))
+        refs.append((g.Engine(0, 100 + i, off), d, torch.zeros(n, dtype=TDT[dtype], device="cuda"), buf, i % 3))
+    b = g.Batch(reqs)
+    for _ in range(3):
+        b.launch()
+        for (_, d, out), (e, _, ref, buf, lead) in zip(reqs, refs):
+            g.generate(d, e, ref)
+        torch.cuda.synchronize()
+        for i, ((_, d, out), (_, _, ref, buf, lead)) in enumerate(zip(reqs, refs)):
+            assert torch.equal(out.contiguous().view(torch.uint8), ref.view(torch.uint8)), (i, d)
+            assert not buf[:lead].any() and not buf[lead + ref.numel():].any(), (i, d)
+    b.commit()
+    for (e, _, _), (r, _, _, _, _) in zip(reqs, refs):
+        assert e.offset == r.offset
