@@ -269,3 +269,32 @@ def test_icdf_f64_tails(g, kind):
     got = _gpu(g, kind, 2, 0.0, 1.0, w, wa.size)
     ref = oracle.transform_words(kind, 2, 0.0, 1.0, wa.size, w)
     _check(kind, 2, got, ref, f"ICDF FP64 kind {kind}")
+
+
+@pytest.mark.parametrize("var", [(0, 0, 0.0, 0.0), (1, 1, -2.5, 7.0), (1, 2, 2.0, 5.0), (1, 2, -1.0, 1.0),
+                                 (2, 1, 0.5, 2.0), (3, 1, 0.0, 1.0), (2, 2, 0.0, 1.0), (3, 2, 0.25, 0.5),
+                                 (4, 1, 0.0, 1.0), (5, 2, 0.0, 0.5)])
+def test_transform_words_at_every_alignment(g, var):
+    """The words and the output each at every 4-byte phase of 16 bytes, at sizes
+    below a group, around the tiles and ragged: the same outputs bit for bit as
+    from the aligned call, and nothing written around them."""
+    kind, dtype, p0, p1 = var
+    d = g.Distribution(kind, dtype, p0, p1)
+    dt = {0: torch.int32, 1: torch.float32, 2: torch.float64}[dtype]
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    top = 9001
+    pool = torch.randint(-(1 << 31), 1 << 31, (2 * top + 16,), dtype=torch.int32, device="cuda", generator=gen)
+    want = torch.empty(top, dtype=dt, device="cuda")
+    g.transform_words(d, pool[:2 * top + 8], want, top - 1)
+    for n in (1, 2, 3, 4, 5, 7, 1023, 1024, 1025, 4096, 4099, top - 2):
+        # even n: a pair cut in two has a second output that a longer call would write
+        for wo in range(4):
+            words = torch.empty(2 * top + 16, dtype=torch.int32, device="cuda")[wo:]
+            words[:2 * top] = pool[:2 * top]
+            for oo in range(4 if dtype != 2 else 2):
+                buf = torch.zeros(n + 8, dtype=dt, device="cuda")
+                g.transform_words(d, words, buf[oo:], n)
+                torch.cuda.synchronize()
+                assert torch.equal(buf[oo:oo + n].contiguous().view(torch.uint8),
+                                   want[:n].view(torch.uint8)), (var, n, wo, oo)
+                assert not buf[:oo].any() and not buf[oo + n:].any(), (var, n, wo, oo)
