@@ -90,6 +90,8 @@ _lib = None
 def load() -> ctypes.CDLL:
     """Loads libgrng.so (built in-tree); raises if it is missing."""
     global _lib
+    if _lib is not None:  # set once, complete
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -180,6 +182,36 @@ def _check(status: int, where: str) -> None:
         raise GrngError(status, where, detail)
 
 
+_torch = None
+
+
+def _t():
+    """The torch module (imported on first use)."""
+    global _torch
+    if _torch is None:
+        import torch
+
+        _torch = torch
+    return _torch
+
+
+def _on_device(index: int, stream, where: str, fn, *args) -> None:
+    """fn(*args, stream) with device `index` current, on `stream` or that
+    device's current one.  Where the device is current already, as it nearly
+    always is, the call goes straight through: the guard and the Stream object of
+    the general way cost 5 us a call, more than the launch."""
+    torch = _t()
+    if torch._C._cuda_getDevice() == index:
+        raw = torch._C._cuda_getCurrentRawStream(index) if stream is None \
+            else _stream_ptr(index, stream)
+        status = fn(*args, raw)
+    else:
+        with torch.cuda.device(index):
+            status = fn(*args, _stream_ptr(index, stream))
+    if status:
+        _check(status, where)
+
+
 def _split128(v: int):
     v %= 1 << 128
     return v & ((1 << 64) - 1), v >> 64
@@ -196,6 +228,23 @@ class Distribution:
 
     def _c(self) -> _Dist:
         return _Dist(self.kind, self.dtype, float(self.p0), float(self.p1))
+
+    def __post_init__(self):
+        # the fields are frozen: the C form is made once (read-only to the library)
+        object.__setattr__(self, "_cached", None)
+
+    def _ref(self) -> _Dist:
+        if self._cached is None:
+            object.__setattr__(self, "_cached", self._c())
+        return self._cached
+
+    def __getstate__(self):
+        return {"kind": self.kind, "dtype": self.dtype, "p0": self.p0, "p1": self.p1}
+
+    def __setstate__(self, state):
+        for k, v in state.items():
+            object.__setattr__(self, k, v)
+        object.__setattr__(self, "_cached", None)
 
     @staticmethod
     def bits() -> "Distribution":
@@ -308,8 +357,7 @@ class Engine:
 
 def words_for(dist: Distribution, n: int) -> int:
     out = ctypes.c_uint64()
-    d = dist._c()
-    _check(load().grng_words_for(ctypes.byref(d), n, ctypes.byref(out)), "grng_words_for")
+    _check(load().grng_words_for(dist._ref(), n, ctypes.byref(out)), "grng_words_for")
     return int(out.value)
 
 
@@ -317,8 +365,7 @@ _TORCH_DTYPES = {}
 
 
 def _torch_dtype_ok(t, dtype: int) -> bool:
-    import torch
-
+    torch = _t()
     if dtype == F32:
         return t.dtype == torch.float32
     if dtype == F64:
@@ -336,9 +383,9 @@ def _stream_ptr(device, stream) -> int:
 
 def generate_ptr(dist: Distribution, engine: Engine, n: int, dev_ptr: int, stream_ptr: int) -> None:
     """grng_generate on a raw device address and a raw cudaStream_t value."""
-    d = dist._c()
-    _check(load().grng_generate(ctypes.byref(d), engine.handle, n, ctypes.c_void_p(dev_ptr),
-                                ctypes.c_void_p(stream_ptr)), "grng_generate")
+    status = load().grng_generate(dist._ref(), engine.handle, n, dev_ptr, stream_ptr)
+    if status:
+        _check(status, "grng_generate")
 
 
 def generate(dist: Distribution, engine: Engine, out, n: int | None = None, stream=None):
@@ -347,19 +394,19 @@ def generate(dist: Distribution, engine: Engine, out, n: int | None = None, stre
     out may be a view at any element offset; n defaults to out.numel().
     Returns out.
     """
-    import torch
-
     if not out.is_cuda:
         raise ValueError("out must be a CUDA tensor")
     if not out.is_contiguous():
         raise ValueError("out must be contiguous")
     if not _torch_dtype_ok(out, dist.dtype):
         raise ValueError(f"tensor dtype {out.dtype} does not match distribution dtype {dist.dtype}")
-    n = out.numel() if n is None else n
-    if n > out.numel():
+    numel = out.numel()
+    if n is None:
+        n = numel
+    elif n > numel:
         raise ValueError("n exceeds the tensor size")
-    with torch.cuda.device(out.device):
-        generate_ptr(dist, engine, n, out.data_ptr(), _stream_ptr(out.device, stream))
+    _on_device(out.get_device(), stream, "grng_generate", load().grng_generate, dist._ref(),
+               engine.handle, n, out.data_ptr())
     return out
 
 
@@ -367,20 +414,14 @@ def generate_substreams(dist: Distribution, engine: Engine, out, n_per_stream: i
                         num_streams: int, stride: int, stream=None):
     """Substream s fills out[s * n_per_stream : (s + 1) * n_per_stream] from word
     offset engine.offset + s * stride.  The engine does not advance."""
-    import torch
-
     if not out.is_cuda or not out.is_contiguous() or not _torch_dtype_ok(out, dist.dtype):
         raise ValueError("out must be a contiguous CUDA tensor of the distribution's dtype")
     if n_per_stream * num_streams > out.numel():
         raise ValueError("out is too small")
     lo, hi = _split128(stride)
-    d = dist._c()
-    with torch.cuda.device(out.device):
-        _check(load().grng_generate_substreams(ctypes.byref(d), engine.handle, n_per_stream,
-                                               num_streams, lo, hi,
-                                               ctypes.c_void_p(out.data_ptr()),
-                                               ctypes.c_void_p(_stream_ptr(out.device, stream))),
-               "grng_generate_substreams")
+    _on_device(out.get_device(), stream, "grng_generate_substreams",
+               load().grng_generate_substreams, dist._ref(), engine.handle, n_per_stream,
+               num_streams, lo, hi, out.data_ptr())
     return out
 
 
@@ -496,8 +537,6 @@ def tune_reset() -> None:
 
 def transform_words(dist: Distribution, words, out, n: int | None = None, stream=None):
     """grng_transform_words: applies dist to the device words tensor (int32 / uint32)."""
-    import torch
-
     if not (words.is_cuda and out.is_cuda and words.is_contiguous() and out.is_contiguous()):
         raise ValueError("words and out must be contiguous CUDA tensors")
     if not _torch_dtype_ok(out, dist.dtype):
@@ -505,12 +544,8 @@ def transform_words(dist: Distribution, words, out, n: int | None = None, stream
     n = out.numel() if n is None else n
     if words.numel() * words.element_size() < 4 * words_for(dist, n):
         raise ValueError("not enough words")
-    d = dist._c()
-    with torch.cuda.device(out.device):
-        _check(load().grng_transform_words(ctypes.byref(d), ctypes.c_void_p(words.data_ptr()), n,
-                                           ctypes.c_void_p(out.data_ptr()),
-                                           ctypes.c_void_p(_stream_ptr(out.device, stream))),
-               "grng_transform_words")
+    _on_device(out.get_device(), stream, "grng_transform_words", load().grng_transform_words,
+               dist._ref(), words.data_ptr(), n, out.data_ptr())
     return out
 
 
@@ -551,6 +586,7 @@ class Batch:
                                             ctypes.byref(nbytes)), "grng_batch_workspace_bytes")
         self.workspace = torch.empty(max(nbytes.value, 256), dtype=torch.uint8, device=dev)
         self._dev = dev
+        self._dev_index = self.workspace.get_device()
         self._h = ctypes.c_void_p()
         with torch.cuda.device(dev):
             _check(L.grng_batch_create(ctypes.byref(self._h), arr, len(arr), ipt,
@@ -559,11 +595,7 @@ class Batch:
                    "grng_batch_create")
 
     def launch(self, stream=None):
-        import torch
-
-        with torch.cuda.device(self._dev):
-            _check(load().grng_batch_launch(self._h, ctypes.c_void_p(_stream_ptr(self._dev, stream))),
-                   "grng_batch_launch")
+        _on_device(self._dev_index, stream, "grng_batch_launch", load().grng_batch_launch, self._h)
 
     def autotune(self, stream=None):
         """(ipt, CTAs per SM, ms per fill) of the fastest geometry, now in use."""
@@ -630,6 +662,7 @@ class Server:
         self.device = torch.device("cuda", torch.cuda.current_device()) if device is None \
             else torch.device(device)
         self.pool = torch.empty(pool_bytes, dtype=torch.uint8, device=self.device)
+        self._base = self.pool.data_ptr()
         self._h = ctypes.c_void_p()
         with torch.cuda.device(self.device):
             _check(load().grng_server_create(ctypes.byref(self._h),
@@ -639,25 +672,28 @@ class Server:
 
     def submit(self, req: _ServeRequest) -> int:
         t = ctypes.c_uint64()
-        _check(load().grng_server_submit(self._h, ctypes.byref(req), ctypes.byref(t)),
-               "grng_server_submit")
+        status = load().grng_server_submit(self._h, req, t)
+        if status:
+            _check(status, "grng_server_submit")
         return t.value
 
     def wait(self, ticket: int, timeout_s: float = 30.0):
         """(device address, bytes) of a completed request's output."""
         p, b = ctypes.c_void_p(), ctypes.c_size_t()
-        _check(load().grng_server_wait(self._h, ticket, int(timeout_s * 1e6), ctypes.byref(p),
-                                       ctypes.byref(b)), "grng_server_wait")
+        status = load().grng_server_wait(self._h, ticket, int(timeout_s * 1e6), p, b)
+        if status:
+            _check(status, "grng_server_wait")
         return p.value, b.value
 
     def output(self, ticket: int, timeout_s: float = 30.0):
         """The completed request's output bytes as a view of the pool tensor."""
         addr, nbytes = self.wait(ticket, timeout_s)
-        off = addr - self.pool.data_ptr()
-        return self.pool[off:off + nbytes]
+        return self.pool.narrow(0, addr - self._base, nbytes)
 
     def release(self, ticket: int) -> None:
-        _check(load().grng_server_release(self._h, ticket), "grng_server_release")
+        status = load().grng_server_release(self._h, ticket)
+        if status:
+            _check(status, "grng_server_release")
 
     def drain(self, timeout_s: float = 120.0) -> None:
         _check(load().grng_server_drain(self._h, int(timeout_s * 1e6)), "grng_server_drain")
