@@ -7,7 +7,10 @@
 // (round to nearest).
 //
 //   z0 = rho cos(2 pi u2), z1 = rho sin(2 pi u2), rho = sqrt(-2 ln u1),
-//   u1 = (x1 + 1) 2^-53 in (0, 1], u2 = x2 2^-53 in [0, 1), x1, x2 53-bit.
+//   u1 = (x1 + 1) 2^-53 in (0, 1], u2 = x2 2^-53 in [0, 1), x1, x2 53-bit, the
+//   top bits of two words each.  The words are taken as they are, u1 as the
+//   64-bit (x1 + 1) 2^11 and u2 as x2 2^11, and 2 (-ln u1) is kept with an even
+//   exponent throughout, so that neither needs a shift of its own.
 //
 // -ln u1:  u1 = 2^-e (1 - delta), delta in (0, 1/2]; a table factor
 //          c_i ~ 1/(1 - i/1024) reduces -ln(1 - delta) to ln c_i - ln(1 - r),
@@ -54,12 +57,12 @@ struct U64Pair {
 #if defined(__CUDACC__)
 __device__ const ulonglong2 d_sc[GRNG_BM64_SINT_LEN] = GRNG_BM64_SC;
 __device__ const ulonglong2 d_lt[GRNG_BM64_LOGT_LEN] = GRNG_BM64_LT;
-__device__ const uint64_t d_e58[GRNG_BM64_E58_LEN] = GRNG_BM64_E58;
+__device__ const uint64_t d_e57[GRNG_BM64_E57_LEN] = GRNG_BM64_E57;
 __device__ const uint64_t d_exp2t[GRNG_BM64_EXP2T_LEN] = GRNG_BM64_EXP2T;
 #endif
 static const U64Pair h_sc[GRNG_BM64_SINT_LEN] = GRNG_BM64_SC;
 static const U64Pair h_lt[GRNG_BM64_LOGT_LEN] = GRNG_BM64_LT;
-static const uint64_t h_e58[GRNG_BM64_E58_LEN] = GRNG_BM64_E58;
+static const uint64_t h_e57[GRNG_BM64_E57_LEN] = GRNG_BM64_E57;
 static const uint64_t h_exp2t[GRNG_BM64_EXP2T_LEN] = GRNG_BM64_EXP2T;
 
 #if defined(__CUDA_ARCH__)
@@ -67,7 +70,7 @@ static const uint64_t h_exp2t[GRNG_BM64_EXP2T_LEN] = GRNG_BM64_EXP2T;
 #else
 #define GRNG_BM_TABLE(d, h, i) h[i]
 #endif
-GRNG_BM_HD uint64_t e58(uint32_t e) { return GRNG_BM_TABLE(d_e58, h_e58, e); }
+GRNG_BM_HD uint64_t e57(uint32_t e) { return GRNG_BM_TABLE(d_e57, h_e57, e); }
 GRNG_BM_HD uint64_t exp2t(uint32_t j) { return GRNG_BM_TABLE(d_exp2t, h_exp2t, j); }
 #undef GRNG_BM_TABLE
 // sin and cos of 2 pi j / 8192 (2^63 scale)
@@ -81,7 +84,7 @@ GRNG_BM_HD void sincos_tab(uint32_t j, uint64_t& s, uint64_t& c) {
   c = h_sc[j].b;
 #endif
 }
-// ln c_i 2^64 and c_i 2^24
+// ln c_i 2^63 and c_i 2^24
 GRNG_BM_HD void log_tab(uint32_t i, uint64_t& t, uint32_t& c) {
 #if defined(__CUDA_ARCH__)
   const ulonglong2 v = __ldg(&d_lt[i]);
@@ -170,13 +173,6 @@ GRNG_BM_HD uint32_t clz32(uint32_t x) {  // x != 0
 #endif
 }
 
-// floor(log2 x) for 1 <= x < 2^23: x converts exactly through the 2^23
-// shifter, and the float's exponent is the answer (two full-rate
-// operations instead of a quarter-rate leading-zero count).
-GRNG_BM_HD int ilog2_small(uint32_t x) {
-  return (int)(f32_bits(bits_f32(0x4B000000u | x) - 8388608.0f) >> 23) - 127;
-}
-
 // High word of (hi:lo) << s and low word of (hi:lo) >> s, for 0 <= s < 32.
 GRNG_BM_HD uint32_t shl_hi(uint32_t lo, uint32_t hi, uint32_t s) {
 #if defined(__CUDA_ARCH__)
@@ -213,93 +209,87 @@ GRNG_BM_HD float rsqrt_seed(float x) {
 #endif
 }
 
-// -ln(u1) for u1 = m1 2^-53, m1 in [1, 2^53), as lm 2^le with lm normalised
-// (top bit set).  m1 = 2^53 (u1 = 1) is handled by the caller.
-GRNG_BM_HD void neg_log(uint64_t m1, uint64_t& lm, int& le) {
-  // M = m1 << s, s = clz(m1): (1 - delta) 2^64 with its top bit set, and
-  // u1 = 2^-e (1 - delta) with e = s - 11.  Except when m1 < 2^32
-  // (probability 2^-21) the shift is found from the high word alone.
-  const uint32_t m1h = (uint32_t)(m1 >> 32), m1l = (uint32_t)m1;
+// 2 (-ln u1) for u1 = M0 2^-64, M0 = (m0h, m0l) a nonzero multiple of 2^11, as
+// X 2^E with E even and X in [2^62, 2^64).
+GRNG_BM_HD void neg2_log(uint32_t m0h, uint32_t m0l, uint64_t& X, int& E) {
+  // M = M0 << e, e = clz(M0): (1 - delta) 2^64 with its top bit set, and
+  // u1 = 2^-e (1 - delta)
   uint64_t M;
   uint32_t e;
-  if (m1h != 0) {
-    const uint32_t s = clz32(m1h);          // 11..31 (m1h < 2^21)
-    M = join(shl_hi(m1l, m1h, s), m1l << s);
-    e = s - 11u;
+  if (m0h - 1u >= 0xFFBFFFFFu) {              // m0h = 0, or delta < 2^-10 with e = 0
+    if (m0h != 0) {
+      // -ln u1 = delta (1 + f), f = delta/2 + delta^2/3 + ... + delta^5/6
+      // (delta^6/7 is below 2^-62 relative), scaled by the normalised delta
+      // so that no absolute truncation enters
+      const uint64_t D = 0ull - join(m0h, m0l);
+      const int nz = clz64(D);                // 9..53 (D >= 2^11)
+      const uint64_t Dn = D << nz;
+      uint64_t G = kInv6;
+      G = kInv5 + umulhi_apx(D, G);
+      G = kInv4 + umulhi_apx(D, G);
+      G = kInv3 + umulhi_apx(D, G);
+      G = kInv2 + umulhi_apx(D, G);
+      const uint64_t F = umulhi_apx(D, G);    // f 2^64
+      const uint64_t half = Dn >> 1;
+      const uint64_t Ls = half + umulhi_apx(half, F);  // -ln u1 2^(63 + nz), in [2^62, 2^64)
+      // 2 (-ln u1) = Ls 2^(-62 - nz): an odd nz moves one place up or down
+      X = Ls;
+      E = -62 - nz;
+      if (nz & 1) {
+        const bool top = (Ls >> 63) != 0;
+        X = top ? Ls >> 1 : Ls << 1;
+        E += top ? 1 : -1;
+      }
+      return;
+    }
+    const uint32_t s = clz32(m0l);            // M0 < 2^32 (probability 2^-32)
+    M = join(m0l << s, 0u);
+    e = 32u + s;
   } else {
-    const int s = clz64(m1);                // 32..63
-    M = m1 << s;
-    e = (uint32_t)(s - 11);
+    e = clz32(m0h);                           // 0..31
+    M = join(shl_hi(m0l, m0h, e), m0l << e);
   }
-  const uint64_t D = 0ull - M;              // delta 2^64 in (0, 2^63]
-  const uint32_t i = (uint32_t)(D >> 54);   // 0..512
-  if (e == 0 && i == 0) {
-    // delta < 2^-10: -ln u1 = delta (1 + f), f = delta/2 + delta^2/3 + ... +
-    // delta^5/6 (delta^6/7 is below 2^-62 relative), scaled by the
-    // normalised delta so that no absolute truncation enters
-    const int nz = clz64(D);                // 10..53 (D >= 2^11)
-    const uint64_t Dn = D << nz;
-    uint64_t G = kInv6;
-    G = kInv5 + umulhi_apx(D, G);
-    G = kInv4 + umulhi_apx(D, G);
-    G = kInv3 + umulhi_apx(D, G);
-    G = kInv2 + umulhi_apx(D, G);
-    const uint64_t F = umulhi_apx(D, G);    // f 2^64
-    const uint64_t half = Dn >> 1;
-    const uint64_t Ls = half + umulhi_apx(half, F);  // -ln u1 2^(63 + nz), in [2^62, 2^64)
-    const int c = clz64(Ls);                // 0 or 1
-    lm = Ls << c;
-    le = -63 - nz - c;
-    return;
-  }
-  uint64_t Ti;                              // ln c_i 2^64
+  const uint32_t i = (uint32_t)((0ull - M) >> 54);  // delta 2^10, 0..512
+  uint64_t Ti;                              // ln c_i 2^63
   uint32_t C;                               // c_i 2^24
   log_tab(i, Ti, C);
-  // r 2^64 = 2^64 - M C 2^-24 (truncating M C 2^-24 leaves r >= 0); the
-  // 96-bit product M C is exact, and M C 2^-24 = (hi << 8) | (lo32 >> 24)
+  // r 2^63 = 2^63 - M C 2^-25 (truncating M C 2^-25 leaves r >= 0); the
+  // 96-bit product M C is exact, and M C 2^-25 = (hi << 7) | (lo32 >> 25)
   uint64_t mc_hi;
   uint32_t mc_lo;
   mul64x32(M, C, mc_hi, mc_lo);
-  const uint64_t R = 0ull - ((mc_hi << 8) | (uint64_t)(mc_lo >> 24));  // < 2^55
-  // -ln(1 - r) 2^64 = R + R^2/2 + T3 + T4 + T5 + T6 (r^7/7 < 2^-65.8).
-  // With r32 = r 2^41, r^3 comes from 32-bit high products: q = r^2 2^50,
-  // t = r^3 2^59.
-  const uint32_t r32 = (uint32_t)(R >> 23);
+  const uint64_t R = (1ull << 63) - ((mc_hi << 7) | (uint64_t)(mc_lo >> 25));  // < 2^54
+  // -ln(1 - r) 2^63 = R + R^2/2 + T3 + T4 + T5 + T6 (r^7/7 < 2^-65.8), R^2/2
+  // being the high word of R^2.  With r32 = r 2^41, r^3 comes from 32-bit high
+  // products: q = r^2 2^50, t = r^3 2^59.
+  const uint32_t r32 = (uint32_t)(R >> 22);
   const uint32_t q = mulh(r32, r32);
   const uint32_t t = mulh(q, r32);
-  const uint64_t T3 = mulw(t, 0xAAAAAAABu) >> 28;              // t 2^5 / 3
-  // r^4/4 + r^5/5 + r^6/6 stay below 2^26 units of 2^-64, so FP32 is exact
-  // enough (error about 4 units) and keeps them off the integer multiplier,
-  // the busiest pipe: with x = r 2^9 < 1, 2^64 (r^4/4 + r^5/5 + r^6/6) =
-  // x^4 (2^26 + x (2^19/5 + x 2^10/6))
+  const uint64_t T3 = mulw(t, 0xAAAAAAABu) >> 29;              // t 2^4 / 3
+  // r^4/4 + r^5/5 + r^6/6 stay below 2^25 units of 2^-63, so FP32 is exact
+  // enough (error about 2 units) and keeps them off the integer multiplier,
+  // the busiest pipe: with x = r 2^9 < 1, 2^63 (r^4/4 + r^5/5 + r^6/6) =
+  // x^4 (2^25 + x (2^18/5 + x 2^9/6))
   const float x = u32_to_f32(r32) * 0x1p-32f;
   const float x2 = x * x;
   const uint32_t T456 =
-      f32_to_u32_rn(x2 * x2 * fma32(x, fma32(x, 170.66667f, 104857.6f), 67108864.0f));
-  const uint64_t S = R + (sqr_hi(R) >> 1) + T3 + T456;
-  // -ln(1 - delta) 2^64 = ln c_i 2^64 + S < ln 2 2^64 + 2^55; with e >= 1
-  // the sum e ln 2 + ... is kept in units of 2^-58 (below 37 2^58 < 2^64)
-  uint64_t Lf = Ti + S;
-  int lb = -64;
-  if (e != 0) {
-    Lf = e58(e) + (Lf >> 6);
-    lb = -58;
-  }
-  // Lf >= 2^54 (-ln u1 >= ln c_1 > 2^-10 here), so its high word is not 0
+      f32_to_u32_rn(x2 * x2 * fma32(x, fma32(x, 85.333333f, 52428.8f), 33554432.0f));
+  // -ln(1 - delta) 2^63 = ln c_i 2^63 + S < ln 2 2^63 + 2^54; with e >= 1 the
+  // sum e ln 2 + ... is kept in units of 2^-57 (below 37 2^57 < 2^63)
+  const uint64_t S = Ti + R + sqr_hi(R) + T3 + T456;
+  const uint32_t sh = e != 0 ? 6u : 0u;
+  const uint32_t Sh = (uint32_t)(S >> 32), Sl = (uint32_t)S;
+  const uint64_t Lf = e57(e) + join(Sh >> sh, shr_lo(Sl, Sh, sh));
+  // Lf >= 2^53 (-ln u1 >= ln c_1 > 2^-10 here), so its high word is not 0;
+  // an even shift leaves its top bit at bit 63 or 62 and E even
   const uint32_t Lh = (uint32_t)(Lf >> 32), Ll = (uint32_t)Lf;
-  const uint32_t nz = clz32(Lh);            // 0..9 (Lh >= 2^22)
-  lm = join(shl_hi(Ll, Lh, nz), Ll << nz);
-  le = lb - (int)nz;
+  const uint32_t n = clz32(Lh) & 30u;       // 0..10 (Lh >= 2^21)
+  X = join(shl_hi(Ll, Lh, n), Ll << n);
+  E = (int)sh - 62 - (int)n;
 }
 
-// sqrt(2 lm 2^le) as sq 2^se, sq in [2^61, 2^62].
-GRNG_BM_HD void sqrt2x(uint64_t lm, int le, uint64_t& sq, int& se) {
-  int E = le + 1;                           // 2L = lm 2^E
-  uint64_t X = lm;
-  if (E & 1) {                              // make the exponent even
-    X = lm >> 1;
-    E += 1;
-  }
+// sqrt(X 2^E), E even and X in [2^62, 2^64), as sq 2^se, sq in [2^61, 2^62].
+GRNG_BM_HD void sqrt_fixed(uint64_t X, int E, uint64_t& sq, int& se) {
   // x = X 2^-64 in [1/4, 1) as xh + xl, two 23-bit pieces (error < 2^-46)
   const float xh = bits_f32(0x3F800000u | (uint32_t)(X >> 41)) - 1.0f;
   const float xl = (bits_f32(0x3F800000u | ((uint32_t)(X >> 18) & 0x7FFFFFu)) - 1.0f) * 0x1p-23f;
@@ -327,19 +317,23 @@ GRNG_BM_HD void sqrt2x(uint64_t lm, int le, uint64_t& sq, int& se) {
   const int32_t d = (int32_t)((uint32_t)(X >> 4) - (uint32_t)sqr_hi(s0));
   const int32_t y30 = (int32_t)(uint32_t)(Y1 >> 32);
   sq = s0 + (uint64_t)(((int64_t)d * (int64_t)y30) >> 29);
-  // sqrt(2L) = sqrt(X 2^E) = sqrt(x) 2^32 2^(E/2) = sq 2^(E/2 - 30)
+  // sqrt(X 2^E) = sqrt(x) 2^32 2^(E/2) = sq 2^(E/2 - 30)
   se = E / 2 - 30;
 }
 
-// |cos|, |sin| of 2 pi x2 2^-53 in 2^-63 fixed point with the signs.
-GRNG_BM_HD void sincos_turns(uint64_t x2, uint64_t& c_abs, bool& c_neg, uint64_t& s_abs,
-                             bool& s_neg) {
-  const uint32_t o = (uint32_t)(x2 >> 50);          // octant
-  uint64_t t = x2 & ((1ull << 50) - 1);
-  if (o & 1u) t = (1ull << 50) - t;                 // reflect: angle pi/4 - beta
-  const uint32_t j = (uint32_t)(t >> 40);           // 0..1024
-  const uint64_t h = t & ((1ull << 40) - 1);
-  const uint64_t P = umulhi_apx(h << 14, k2Pi61);   // phi 2^64 = 2 pi h 2^11 < 2^53.7
+// |cos|, |sin| of 2 pi u2 in 2^-63 fixed point and their signs (bit 31), u2 =
+// x2 2^-53 the top 53 bits of the words (wa, wb).
+GRNG_BM_HD void sincos_turns(uint32_t wa, uint32_t wb, uint64_t& c_abs, uint32_t& c_sign,
+                             uint64_t& s_abs, uint32_t& s_sign) {
+  // octant o = wa >> 29; the angle within it, t 2^11 (t 50 bits), reflected to
+  // 2^50 - t in odd octants (angle pi/4 - beta)
+  const uint32_t odd = (wa >> 29) & 1u;
+  const uint32_t m = 0u - odd;
+  const uint64_t t = join((wa ^ m) & 0x1FFFFFFFu, (wb ^ m) & 0xFFFFF800u) + (odd << 11);
+  const uint32_t j = (uint32_t)(t >> 51);           // 0..1024
+  // phi 2^64 = 2 pi h 2^11 < 2^53.7, h the low 40 bits of t
+  const uint64_t P = umulhi_apx((t & ((1ull << 51) - 1)) << 3, k2Pi61);
+  // phi 2^64 = 2 pi h 2^11 < 2^53.7
   const uint64_t P2 = sqr_hi(P);                    // phi^2 2^64 < 2^43.4
   const uint32_t a = (uint32_t)(P2 >> 12);          // phi^2 2^52
   const uint32_t b = (uint32_t)(P >> 22);           // phi 2^42
@@ -360,13 +354,38 @@ GRNG_BM_HD void sincos_turns(uint64_t x2, uint64_t& c_abs, bool& c_neg, uint64_t
   const uint64_t k2 = umulhi_apx(Cj, sphi + eps);
   const uint64_t k3 = umulhi_apx(Sj, sphi - eps);
   const uint64_t cs = Cj - k1 - k3;                 // cos(alpha + phi) 2^63 >= 2^62.5
-  const int64_t snv = (int64_t)(Sj + k2 - k1);      // sin(alpha + phi) 2^63, >= -2
-  const uint64_t sn = snv < 0 ? 0ull : (uint64_t)snv;
-  const bool swap = ((o + 1u) & 2u) != 0;           // octants 1, 2, 5, 6
+  // sin(alpha + phi) 2^63: the products truncate by at most 2, the table's
+  // sine is 2 up
+  const uint64_t sn = Sj + k2 - k1;
+  // in Gray code the octant's bits are the swap (octants 1, 2, 5, 6), the
+  // cosine's sign (2..5) and the sine's (4..7)
+  const uint32_t g = wa ^ (wa >> 1);
+  const bool swap = (g & (1u << 29)) != 0;
   s_abs = swap ? cs : sn;
   c_abs = swap ? sn : cs;
-  s_neg = o >= 4u;
-  c_neg = ((o + 2u) & 4u) != 0;                     // octants 2, 3, 4, 5
+  s_sign = g & 0x80000000u;
+  c_sign = (g << 1) & 0x80000000u;
+}
+
+// p 2^k as a double with sign (bit 31), rounded to nearest even, by two adds on
+// the FP64 pipe, otherwise idle: with the halves of p as the low words of
+// 2^(84+k) and 2^(52+k), their sum less the two is p 2^k, the first add exact.
+// p = 0 gives +0 (all three terms take the sign).  kh is k << 20; 2^(84+k) and
+// 2^(52+k) are normal.
+GRNG_BM_HD double to_double(uint64_t p, uint32_t kh, uint32_t sign) {
+  const uint32_t b = kh + sign;
+  const uint64_t H = join(b + 0x45300000u, (uint32_t)(p >> 32));
+  const uint64_t L = join(b + 0x43300000u, (uint32_t)p);
+  const uint64_t C = join(b + 0x45300000u, 0x00100000u);  // 2^(84+k) + 2^(52+k)
+  double h, l, c;
+  std::memcpy(&h, &H, 8);
+  std::memcpy(&l, &L, 8);
+  std::memcpy(&c, &C, 8);
+#if defined(__CUDA_ARCH__)
+  return __dadd_rn(__dadd_rn(h, -c), l);
+#else
+  return (h - c) + l;
+#endif
 }
 
 // p 2^k as a double, rounded to nearest (ties away), with sign; p = 0 gives +0.
@@ -397,32 +416,30 @@ GRNG_BM_HD double assemble(uint64_t p, int k, bool neg) {
   return d;
 }
 
-// The Box-Muller pair in fixed point: z0 = (n0 ? -p0 : p0) 2^k,
-// z1 = (n1 ? -p1 : p1) 2^k, p0, p1 < 2^62; u1 = 1 gives p0 = p1 = 0.
+// The Box-Muller pair in fixed point: z0 = p0 2^k and z1 = p1 2^k with signs
+// (bit 31), p0, p1 < 2^62; u1 = 1 gives p0 = p1 = 0.
 struct FixedPair {
   uint64_t p0, p1;
   int k;
-  bool n0, n1;
+  uint32_t s0, s1;
 };
 
-// The Box-Muller pair for 53-bit x1 (u1 = (x1 + 1) 2^-53) and x2 (u2 = x2 2^-53).
-GRNG_BM_HD FixedPair box_muller_fixed(uint64_t x1, uint64_t x2) {
-  const uint64_t m1 = x1 + 1u;
+// The Box-Muller pair for u1 = (x1 + 1) 2^-53 and u2 = x2 2^-53, x1 and x2 the
+// top 53 bits of the words (w0, w1) and (w2, w3).
+GRNG_BM_HD FixedPair box_muller_fixed(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+  const uint64_t m0 = join(w0, w1 | 0x7FFu) + 1u;  // (x1 + 1) 2^11, 0 for u1 = 1
   uint64_t c_abs, s_abs;
-  bool c_neg, s_neg;
-  sincos_turns(x2, c_abs, c_neg, s_abs, s_neg);
   FixedPair r;
-  r.n0 = c_neg;
-  r.n1 = s_neg;
-  if (m1 >> 53) {  // u1 = 1: rho = 0
+  sincos_turns(w2, w3, c_abs, r.s0, s_abs, r.s1);
+  if (m0 == 0) {  // rho = 0
     r.p0 = r.p1 = 0;
     r.k = 0;
     return r;
   }
-  uint64_t lm, sq;
-  int le, se;
-  neg_log(m1, lm, le);
-  sqrt2x(lm, le, sq, se);
+  uint64_t X, sq;
+  int E, se;
+  neg2_log((uint32_t)(m0 >> 32), (uint32_t)m0, X, E);
+  sqrt_fixed(X, E, sq, se);
   // z = sq 2^se * c 2^-63 = umulhi(sq, c) 2^(se + 1)
   r.p0 = umulhi_apx(sq, c_abs);
   r.p1 = umulhi_apx(sq, s_abs);
@@ -430,10 +447,15 @@ GRNG_BM_HD FixedPair box_muller_fixed(uint64_t x1, uint64_t x2) {
   return r;
 }
 
-GRNG_BM_HD void box_muller(uint64_t x1, uint64_t x2, double& z0, double& z1) {
-  const FixedPair f = box_muller_fixed(x1, x2);
-  z0 = assemble(f.p0, f.k, f.n0);
-  z1 = assemble(f.p1, f.k, f.n1);
+// kBothAdds: both results by the FP64 pipe's adds; else z1 in integers, for
+// callers that put further work on that pipe.
+template <bool kBothAdds>
+GRNG_BM_HD void box_muller(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, double& z0,
+                           double& z1) {
+  const FixedPair f = box_muller_fixed(w0, w1, w2, w3);
+  const uint32_t kh = (uint32_t)f.k << 20;
+  z0 = to_double(f.p0, kh, f.s0);
+  z1 = kBothAdds ? to_double(f.p1, kh, f.s1) : assemble(f.p1, f.k, f.s1 != 0);
 }
 
 // exp(m + s z) for z = (neg ? -p : p) 2^k, written exp(m) 2^(s z log2 e):

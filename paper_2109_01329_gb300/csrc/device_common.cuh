@@ -512,13 +512,6 @@ __device__ __forceinline__ void gauss_block_f32(const uint32_t* w, const Transfo
   yb = fma2(sd, mul2(f2(rb), f2(c[1], s[1])), mean);
 }
 
-// FP64 pair: integer fixed-point evaluation (see bm64_fixed.cuh), within
-// about 1 ulp of the exact value, without the FP64 pipe.
-__device__ __forceinline__ void box_muller_f64(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,
-                                               double& z0, double& z1) {
-  bm64::box_muller(u53(w0, w1), u53(w2, w3), z0, z1);
-}
-
 // icdf_f32_central of two words.
 __device__ __forceinline__ void icdf_f32_central2(uint32_t wa, uint32_t wb, Icdf32& a, Icdf32& b) {
   const F2 f = f2(__int_as_float(0x4B000000u | (wa >> 9)), __int_as_float(0x4B000000u | (wb >> 9)));
@@ -601,14 +594,14 @@ __device__ __forceinline__ void unit_outputs(const uint32_t* w, uint32_t* o,
   } else if constexpr (V == V_LOGN_F64) {
     // exp(m + s z) in fixed point from the fixed-point pair (no FP64
     // instruction); an output outside its range takes the FP64 path
-    const bm64::FixedPair f = bm64::box_muller_fixed(u53(w[0], w[1]), u53(w[2], w[3]));
+    const bm64::FixedPair f = bm64::box_muller_fixed(w[0], w[1], w[2], w[3]);
     double y0, y1;
-    if (!(t.ln_fast && bm64::lognormal_fixed(f.p0, f.k, f.n0, t.ln_em_mant, t.ln_em_exp,
+    if (!(t.ln_fast && bm64::lognormal_fixed(f.p0, f.k, f.s0 != 0, t.ln_em_mant, t.ln_em_exp,
                                              t.ln_s_mant, t.ln_s_exp, y0)))
-      y0 = exp(fma(t.dsd, bm64::assemble(f.p0, f.k, f.n0), t.dmean));
-    if (!(t.ln_fast && bm64::lognormal_fixed(f.p1, f.k, f.n1, t.ln_em_mant, t.ln_em_exp,
+      y0 = exp(fma(t.dsd, bm64::assemble(f.p0, f.k, f.s0 != 0), t.dmean));
+    if (!(t.ln_fast && bm64::lognormal_fixed(f.p1, f.k, f.s1 != 0, t.ln_em_mant, t.ln_em_exp,
                                              t.ln_s_mant, t.ln_s_exp, y1)))
-      y1 = exp(fma(t.dsd, bm64::assemble(f.p1, f.k, f.n1), t.dmean));
+      y1 = exp(fma(t.dsd, bm64::assemble(f.p1, f.k, f.s1 != 0), t.dmean));
     const uint64_t b0 = (uint64_t)__double_as_longlong(y0);
     const uint64_t b1 = (uint64_t)__double_as_longlong(y1);
     o[0] = (uint32_t)b0;
@@ -617,7 +610,8 @@ __device__ __forceinline__ void unit_outputs(const uint32_t* w, uint32_t* o,
     o[3] = (uint32_t)(b1 >> 32);
   } else {  // V_GAUSS_F64, V_STDGAUSS_F64
     double z0, z1;
-    box_muller_f64(w[0], w[1], w[2], w[3], z0, z1);
+    // the affine step takes two more operations on the FP64 pipe
+    bm64::box_muller<V == V_STDGAUSS_F64>(w[0], w[1], w[2], w[3], z0, z1);
     double y0 = z0, y1 = z1;
     // (0, 1) is its own variant rather than a run-time branch: a branch over
     // the two FP64 multiply-adds is predicated, and they would still issue

@@ -4,11 +4,13 @@ Run from this directory: ``python gen_bm64_tables.py > bm64_tables.h``.
 Values are computed with mpmath at 200 bits and rounded to nearest.
 
 Tables (emitted as initializer macros)
-  LT[i], i = 0..512:     (ln(c_i) * 2^64, c_i * 2^24) with c_i = floor(2^24 / (1 - i/1024))
+  LT[i], i = 0..512:     (ln(c_i) * 2^63, c_i * 2^24) with c_i = floor(2^24 / (1 - i/1024))
                          / 2^24, the reduction factor for -ln(1 - delta) with delta in
                          [i/1024, (i+1)/1024)
-  SC[j], j = 0..1024:    (sin, cos(2 pi j / 8192)) * 2^63
-  kE58[e], e = 0..52:    e ln 2 * 2^58
+  SC[j], j = 0..1024:    (sin + 2, cos)(2 pi j / 8192) * 2^63, the sine 2 units up so
+                         that the truncating rotation never leaves it below 0
+  kE57[e], e = 0..52:    e ln 2 * 2^57, half a unit up for e >= 1 (the sum it joins is
+                         truncated to these units)
   kExp2T[j], j = 0..256: 2^(j / 256) * 2^62
 Scalars
   kLn2:    ln 2 * 2^64
@@ -40,13 +42,13 @@ def main():
     for i in range(513):
         c = int(mp.floor(two24 / (1 - mp.mpf(i) / 1024)))
         logc.append(c)
-        logt.append(rnd(mp.log(mp.mpf(c) / two24) * two64))
+        logt.append(rnd(mp.log(mp.mpf(c) / two24) * two63))
     assert logc[0] == 1 << 24 and logc[512] == 1 << 25
     assert all(t < 1 << 64 for t in logt)
-    sint = [rnd(mp.sin(2 * mp.pi * j / 8192) * two63) for j in range(1025)]
+    sint = [rnd(mp.sin(2 * mp.pi * j / 8192) * two63) + 2 for j in range(1025)]
     cost = [rnd(mp.cos(2 * mp.pi * j / 8192) * two63) for j in range(1025)]
-    e58 = [rnd(e * mp.log(2) * mp.mpf(2) ** 58) for e in range(53)]
-    assert all(v < 1 << 64 for v in e58)
+    e57 = [0] + [rnd(e * mp.log(2) * mp.mpf(2) ** 57 + mp.mpf(1) / 2) for e in range(1, 53)]
+    assert all(v < 1 << 64 for v in e57)
     exp2t = [rnd(mp.mpf(2) ** (mp.mpf(j) / 256) * mp.mpf(2) ** 62) for j in range(257)]
     assert exp2t[0] == 1 << 62 and exp2t[256] == 1 << 63
 
@@ -64,7 +66,7 @@ def main():
     out.append(f"#define GRNG_BM64_LOGT_LEN {len(logt)}")
     out.append(f"#define GRNG_BM64_SINT_LEN {len(sint)}")
     # table bodies as macros: the device and host copies are declared where used
-    for name, ctype, vals in [("E58", "uint64_t", e58), ("EXP2T", "uint64_t", exp2t)]:
+    for name, ctype, vals in [("E57", "uint64_t", e57), ("EXP2T", "uint64_t", exp2t)]:
         suffix = "ull" if "64" in ctype else "u"
         out.append(f"#define GRNG_BM64_{name}_LEN {len(vals)}")
         out.append(f"#define GRNG_BM64_{name} {{ \\")

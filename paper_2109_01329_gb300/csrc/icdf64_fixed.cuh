@@ -40,10 +40,10 @@ GRNG_BM_HD int64_t mulhi_su(int64_t a, uint64_t s) {
 
 // t 2^59 with t = -Phi^-1(p), p = m1 2^-53, m1 in [1, 2^52] (p <= 1/2).
 GRNG_BM_HD uint64_t neg_icdf(uint64_t m1) {
-  uint64_t lm, sq;
-  int le, se;
-  bm64::neg_log(m1, lm, le);                 // -ln p = lm 2^le
-  bm64::sqrt2x(lm, le, sq, se);              // w = sqrt(-2 ln p) = sq 2^se
+  uint64_t X, sq;
+  int E, se;
+  bm64::neg2_log((uint32_t)(m1 >> 21), (uint32_t)(m1 << 11), X, E);  // -2 ln p = X 2^E
+  bm64::sqrt_fixed(X, E, sq, se);            // w = sqrt(-2 ln p) = sq 2^se
   const int sh = se + 60;                    // w 2^60 = sq 2^sh, sh in -1..2
   const uint64_t W60 = sh >= 0 ? (sq << sh) : (sq >> (-sh));
   const uint64_t D = W60 > kW0_60 ? W60 - kW0_60 : 0ull;  // (w - w0) 2^60
