@@ -391,9 +391,9 @@ __device__ __forceinline__ float icdf_f32(uint32_t w) {
 // the issue slots.  On this part 8 FFMA and 4 packed ones take the same pipe
 // time (8.9 and 8.6 cycles per warp), but the FP32 fills are bound by issue
 // (71 % of the slots with the pipes 45-65 % busy), not by the FP32 pipes:
-// 10^8 FP32 gaussians 140.2 -> 126.9 us, lognormals 162.2 -> 149.7, inverse
-// CDFs 134.7 -> 128.0.  The uniforms keep their scalar multiply (packed: the
-// same time, 1-2 % slower at word offsets 1-3).  ptxas contracts a packed
+// 10^9 FP32 gaussians 1.295 -> 1.097 ms, lognormals 1.537 -> 1.346 (packing only
+// the logarithm or only the sine and cosine: 1.161, 1.221).  The uniforms keep
+// their scalar multiply (packed: the same time, 1-2 % slower at word offsets 1-3).  ptxas contracts a packed
 // multiply feeding a packed add into one rounding, so no such pair may stand
 // where the two roundings are wanted.
 struct F2 {
@@ -423,7 +423,7 @@ __device__ __forceinline__ F2 add2(F2 a, F2 b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
   return r;
 }
-// the generated polynomials are written as nested fmaf calls
+// Horner steps with scalar coefficients
 __device__ __forceinline__ F2 fmaf(F2 a, F2 b, float c) { return fma2(a, b, f2(c)); }
 __device__ __forceinline__ F2 fmaf(float a, F2 b, float c) { return fma2(f2(a), b, f2(c)); }
 using ::fmaf;
@@ -510,20 +510,6 @@ __device__ __forceinline__ void gauss_block_f32(const uint32_t* w, const Transfo
   const F2 sd = f2(t.fsd), mean = f2(t.fmean);
   ya = fma2(sd, mul2(f2(ra), f2(c[0], s[0])), mean);
   yb = fma2(sd, mul2(f2(rb), f2(c[1], s[1])), mean);
-}
-
-// icdf_f32_central of two words.
-__device__ __forceinline__ void icdf_f32_central2(uint32_t wa, uint32_t wb, Icdf32& a, Icdf32& b) {
-  const F2 f = f2(__int_as_float(0x4B000000u | (wa >> 9)), __int_as_float(0x4B000000u | (wb >> 9)));
-  const F2 x = add2(fmaf(f, f2(0x1p-22f), -3.0f), f2(0x1p-23f));
-  float qa, qb, la, lb;
-  unpack(fmaf(mul2(x, f2(-1.0f)), x, 1.0f), qa, qb);
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(la) : "f"(qa));
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lb) : "f"(qb));
-  const F2 v = mul2(f2(la, lb), f2(-1.0f));
-  unpack(x, a.x, b.x);
-  unpack(v, a.v, b.v);
-  unpack(GRNG_ICDF32_P1(v), a.r, b.r);
 }
 
 // mean + sd z, or exp of it, as the output word of an inverse-CDF variant
@@ -654,11 +640,12 @@ __device__ __forceinline__ uint4 block_outputs(uint4 b, const TransformParams& t
       }
     }
   } else if constexpr (V == V_ICDF_GAUSS_F32 || V == V_ICDF_LOGN_F32) {
-    // the four central evaluations interleave, two values an instruction; one
-    // vote skips the tails
+    // the four central evaluations interleave; one vote skips the tails (two
+    // values an instruction: 10^9 Philox 1.106 ms against 1.094, MRG32k3a 1.546
+    // against 1.509)
     Icdf32 c[4];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) icdf_f32_central2(w[2 * h], w[2 * h + 1], c[2 * h], c[2 * h + 1]);
+    for (int u = 0; u < 4; ++u) c[u] = icdf_f32_central(w[u]);
     if (icdf_f32_is_tail(c[0]) | icdf_f32_is_tail(c[1]) | icdf_f32_is_tail(c[2]) |
         icdf_f32_is_tail(c[3])) {
 #pragma unroll
