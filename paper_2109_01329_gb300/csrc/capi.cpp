@@ -260,6 +260,11 @@ int choose_variant(const grng_distribution* d, TransformParams* t) {
         if (exact_affine_f64(a, b, &A, &e)) {
           t->aff_a = A;
           t->aff_exp = e;
+          // a - d/2 = (A - 2^52) 2^e: at most 53 bits, or 54 of which the last is 0
+          const int64_t low = A - (int64_t(1) << 52);
+          t->aff_add = (low >= -(int64_t(1) << 53) || (low & 1) == 0) ? 1 : 0;
+          t->aff_low = std::ldexp((double)low, e);
+          t->aff_scale = (uint32_t)(e + 53) << 20;
           return V_AFF_F64;
         }
         uniform_f64_consts(a, b, t);

@@ -177,12 +177,22 @@ __device__ __forceinline__ double scaled_u54_to_f64(uint64_t x, int e) {
   return __longlong_as_double((long long)((bexp << 52) | frac));
 }
 
-// Signed form: v 2^e for |v| <= 2^53.  The sign goes in as a bit: negating
-// the double would be an FP64 instruction.
+// Signed form: v 2^e for |v| <= 2^53, as u01_f64 below: unless |v| < 2^32 or
+// |v| = 2^53, |v| = m 2^-s with m in [2^52, 2^53) and s = clz of the high word
+// less 11, and the bit pattern is m + (1074 + e - s) 2^52 with the sign as a bit
+// (negating the double would be an FP64 instruction).
 __device__ __forceinline__ double scaled_i54_to_f64(int64_t v, int e) {
+  const uint32_t sign = (uint32_t)((uint64_t)v >> 32) & 0x80000000u;
   const uint64_t mag = v < 0 ? (uint64_t)(-v) : (uint64_t)v;
-  const uint64_t bits = (uint64_t)__double_as_longlong(scaled_u54_to_f64(mag, e));
-  return __longlong_as_double((long long)(bits | (v < 0 ? (1ull << 63) : 0ull)));
+  const uint32_t h = (uint32_t)(mag >> 32), l = (uint32_t)mag;
+  if (h - 1u >= 0x1FFFFFu) {
+    const uint64_t bits = (uint64_t)__double_as_longlong(scaled_u54_to_f64(mag, e));
+    return __longlong_as_double((long long)(bits | ((uint64_t)sign << 32)));
+  }
+  const uint32_t c = (uint32_t)__clz((int)h);      // 11..31
+  const uint32_t s = c - 11u;
+  const uint32_t hi = __funnelshift_l(l, h, s) + ((uint32_t)(1085 + e) << 20) - (c << 20) + sign;
+  return __hiloint2double((int)hi, (int)(l << s));
 }
 
 // The 53-bit integer of an FP64 uniform: ((w_a << 32) | w_b) >> 11.
@@ -250,6 +260,19 @@ __device__ __forceinline__ double u01_f64_dadd(uint32_t wa, uint32_t wb) {
   const uint32_t l = __funnelshift_r(wb, wa, 11);   // low 32 bits of x
   const double B = __hiloint2double((int)((h & 0xFFFFFu) | 0x3FE00000u), (int)l);
   return __dadd_rn(B, (h >> 20) != 0u ? 0.0 : -0.5);
+}
+
+// The exact affine uniform a + d u, d = 2^(e + 53), by one FP64 add: d times the
+// double B above plus a or a - d/2, both doubles (checked on the host), with
+// the sum exact by the variant's condition.  Every second unit takes it (both:
+// 154 cycles of the FP64 pipe per warp and group, more than the write roof's
+// 95): 10^8 outputs on [-1, 1) 215 -> 168 us, with the integer form from 32-bit
+// halves for the others.
+__device__ __forceinline__ double aff_f64_dadd(uint32_t wa, uint32_t wb, const TransformParams& t) {
+  const uint32_t h = wa >> 11;
+  const uint32_t l = __funnelshift_r(wb, wa, 11);
+  const double B = __hiloint2double((int)(((h & 0xFFFFFu) | 0x3FE00000u) + t.aff_scale), (int)l);
+  return __dadd_rn(B, (h >> 20) != 0u ? t.da : t.aff_low);
 }
 
 // ---------------------------------------------------------- range transform
@@ -538,7 +561,8 @@ __device__ __forceinline__ void unit_outputs(const uint32_t* w, uint32_t* o,
     if constexpr (V == V_U01_F64) {
       r = odd ? u01_f64_dadd(w[0], w[1]) : u01_f64(w[0], w[1]);
     } else if constexpr (V == V_AFF_F64) {
-      r = scaled_i54_to_f64(t.aff_a + (int64_t)u53(w[0], w[1]), t.aff_exp);
+      r = odd && t.aff_add ? aff_f64_dadd(w[0], w[1], t)
+                           : scaled_i54_to_f64(t.aff_a + (int64_t)u53(w[0], w[1]), t.aff_exp);
     } else {
       r = odd ? uniform_ab_f64<false>(w[0], w[1], t) : uniform_ab_f64<true>(w[0], w[1], t);
     }

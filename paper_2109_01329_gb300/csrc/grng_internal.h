@@ -71,6 +71,11 @@ struct TransformParams {
   double dmean, dsd;          // F64 gaussian / lognormal
   int64_t aff_a;              // F64 exact affine: r = (aff_a + x) 2^aff_exp, x = 53-bit word
   int32_t aff_exp;
+  // the same by one FP64 add (aff_add = 1: a - d/2 = aff_low is a double):
+  // d = 2^(aff_exp + 53), its exponent in the high word aff_scale
+  int32_t aff_add;
+  uint32_t aff_scale;
+  double aff_low;
   // F64 lognormal in fixed point: exp(m) = ln_em_mant 2^ln_em_exp, s = ln_s_mant 2^ln_s_exp;
   // ln_fast = 0 keeps every output on the FP64 path
   int32_t ln_fast;

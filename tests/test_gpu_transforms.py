@@ -298,3 +298,22 @@ def test_transform_words_at_every_alignment(g, var):
                 assert torch.equal(buf[oo:oo + n].contiguous().view(torch.uint8),
                                    want[:n].view(torch.uint8)), (var, n, wo, oo)
                 assert not buf[:oo].any() and not buf[oo + n:].any(), (var, n, wo, oo)
+
+
+@pytest.mark.parametrize("a,b", [(-1.0, 1.0), (-0.25, 0.75), (-2.0, 0.0), (0.0, 4.0), (-(1.0 - 2.0**-53), 2.0**-53),
+                                 (-3.0, 1.0), (-0.5, 0.5), (-2.0**900, 2.0**900), (-2.0**-900, 0.0)])
+def test_exact_affine_f64_both_forms(g, a, b):
+    """FP64 uniforms whose a + (b - a) u is exact, by one add and in integers (units
+    alternate; an odd a - d/2 beyond 53 bits keeps the integers): bit-exact with
+    the oracle where the result is 0, near it, at both ends and where the
+    leading bit of the 53-bit word changes."""
+    d = b - a
+    zero = int(-a / d * 2.0**53)
+    xs = [0, 1, 2, M53, M53 - 1, (1 << 52) - 1, 1 << 52, (1 << 52) + 1]
+    xs += [min(M53, max(0, zero + k)) for k in (-(1 << 33), -(1 << 32), -(1 << 31), -2, -1, 0, 1, 2, 1 << 31, 1 << 32)]
+    rng = np.random.Generator(np.random.PCG64(11))
+    xs += [int(v) >> int(s) for v, s in zip(rng.integers(0, 1 << 53, 3000), rng.integers(0, 53, 3000))]
+    words = np.array([w for x in xs for _ in (0, 1) for w in ((x << 11) >> 32, (x << 11) & 0xFFFFFFFF)], dtype=np.uint32)
+    got = _gpu(g, 1, 2, a, b, words, 2 * len(xs))
+    ref = oracle.transform_words(1, 2, a, b, 2 * len(xs), words)
+    assert np.array_equal(got.view(np.uint64), ref.view(np.uint64))
