@@ -8,18 +8,16 @@
 //      A^(k 2^(5 d));
 //   2. steps the two component recursions in registers, with products
 //      reduced by folding 2^32 = c (mod 2^32 - c) instead of dividing;
-//   3. transforms each 16 bytes of outputs and writes them to its row of a
-//      per-warp shared-memory stage (swizzled: no bank conflicts);
-//   4. with its warp, copies the 32 staged rows out with 16-byte stores, 8
-//      lanes per 128-byte row.
+//   3. transforms each 16 bytes of outputs and stores them, 32 bytes at a time
+//      where the output allows: a whole sector, so that the lanes' strided
+//      stores move no more memory than coalesced ones.
 // Chunks are placed so that every chunk starts on a 16-byte output boundary
 // (the first chunk of a stream has virtual head units), hence aligned rows.
 // When the output's start splits a Box-Muller pair (an odd element offset
 // into a 16-byte group) each chunk starts one pair earlier, with the pair
-// that straddles its first 16-byte boundary, and stages its outputs shifted
-// by one element (a one-element carry from pair to pair), so the rows are
-// again whole 16-byte groups; the straddling pair is computed by both
-// neighbouring chunks.
+// that straddles its first 16-byte boundary, and stores its outputs shifted
+// by one element (a one-element carry from pair to pair), again in whole
+// 16-byte groups; the straddling pair is computed by both neighbouring chunks.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -37,7 +35,6 @@ namespace {
 using namespace dev;
 
 constexpr int kThreads = 256;
-constexpr int kRowLg = 3;  // log2 of the 16-byte pieces of a staged row (128 bytes)
 
 struct MrgParams {
   TransformParams t;
@@ -45,11 +42,10 @@ struct MrgParams {
   int64_t n;                  // elements per stream
   int64_t units;              // units per stream
   int64_t out_words;          // output words per stream (n * es / 4)
-  int64_t chunk_units;        // units per thread (multiple of 32 / wpu)
+  int64_t chunk_units;        // units per thread (multiple of 8 / wpu: 32 bytes)
   int64_t chunks_per_stream;
   int64_t total_chunks;
   int64_t head_units;         // virtual units before `out` in the first chunk
-  int32_t row_lg;             // log2 of a row's 16-byte pieces (mode 4; else kRowLg)
   uint64_t stride_lo, stride_hi;  // word stride between streams
   uint32_t m1, m2;            // the moduli, as operands the compiler does not know
   uint32_t x[6];              // state at the call's word offset
@@ -181,7 +177,7 @@ __device__ __forceinline__ void gen_unit(MrgRegs& st, uint32_t* o, const MrgPara
   unit_outputs<V>(w, o, p.t, odd);
 }
 
-// The 16-byte stage chunk from 4 new output words: as they are, or (carry
+// The 16-byte group from 4 new output words: as they are, or (carry
 // mode) shifted up by one element of kOwpe words behind the carried element,
 // whose place the new last element takes.
 template <bool kCarry, int kOwpe>
@@ -200,28 +196,26 @@ __device__ __forceinline__ uint4 shift_in(uint32_t* carry, const uint32_t* o4) {
   }
 }
 
+// A warp's lanes store 32 bytes each, a chunk apart.  Staging 32 rows per warp in
+// shared memory to store them coalesced took 3 instructions per word more: 10^9
+// bits 0.958 -> 0.840 ms, FP64 uniforms 2.41 -> 2.14, FP32 gaussians 1.575 ->
+// 1.440, FP64 gaussians 7.06 -> 6.67.  With 16-byte stores, half a sector each, the
+// FP64 gaussians took 8.08 ms.
+__device__ __forceinline__ void store32(void* p, uint4 a, uint4 b) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y),
+               "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+               : "memory");
+}
+
 // kMode: 1 chunks start on 16-byte boundaries at unit boundaries; 2 chunks start on
 // 16-byte boundaries one element into a Box-Muller pair (carry mode);
 // 3 substreams of unequal 16-byte phase: each stream has its own head, and
-// its own carry mode when its start splits a pair (a warp's 32 chunks lie in
-// one stream, so both are warp-uniform); 4 is 1 with rows shorter than 128
-// bytes (a small fill; their length a run-time value costs a long fill 1 %).
+// its own carry mode when its start splits a pair.
 template <int V, int kMode>
 __global__ void __launch_bounds__(kThreads) mrg_fill_kernel(const __grid_constant__ MrgParams p) {
   constexpr bool kPerStream = kMode == 3;
   constexpr int kWpu = VInfo<V>::wpu;
   constexpr int kOwpe = VInfo<V>::ow_per_elem;
-  // 16-byte pieces of a row, and its units (a sub-chunk of the chunk)
-  const int lg = kMode == 4 ? p.row_lg : kRowLg;
-  const int pieces = 1 << lg;
-  const int su = 4 * pieces / kWpu;
-  constexpr int kCopyUnroll = kMode == 4 ? 1 : 8;
-  // per warp: 32 rows (one per lane) of 8 16-byte chunks; chunk q of row r is
-  // kept at position q ^ (r & 7), so a lane's chunk stores and the copy-out's
-  // row loads are both free of bank conflicts
-  extern __shared__ uint4 stage[][32][8];
-  const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
   const int64_t cid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = cid < p.total_chunks;
   int64_t s = 0, c = active ? cid : 0;
@@ -269,94 +263,63 @@ __global__ void __launch_bounds__(kThreads) mrg_fill_kernel(const __grid_constan
 #pragma unroll
     for (int i = 0; i < kOwpe; ++i) carry[i] = o[kOwpe + i];
   }
-  const int64_t nsub = p.chunk_units / su;
-  uint32_t* out_words = reinterpret_cast<uint32_t*>(p.out);
-  // Copy-out: of 8-piece rows a lane copies piece (lane & 7) of rows
-  // it * 4 + (lane >> 3), it = 0..7, and likewise of shorter ones.  The host
-  // makes chunks_per_stream a multiple of 32 when there are several streams,
-  // so the 32 chunks of a warp lie in one stream and row r is chunk cw + r of
-  // that stream.
-  const int64_t cw = ((int64_t)blockIdx.x * blockDim.x + warp * 32);  // warp's first chunk id
-  const int64_t sw = __shfl_sync(0xFFFFFFFFu, s, 0);
-  const int64_t cw_in = cw - sw * p.chunks_per_stream;
-  const int64_t lim_chunks = (sw + 1) * p.chunks_per_stream < p.total_chunks
-                                 ? (sw + 1) * p.chunks_per_stream
-                                 : p.total_chunks;
-  const int rows_active = (int)((lim_chunks - cw) < 32 ? (lim_chunks - cw) : 32);
-  const int piece = lane & (pieces - 1), row0 = lane >> lg, row_step = 32 >> lg;
-  const int64_t row_stride = row_step * p.chunk_units * kWpu;  // words between rows it and it + 1
-  const int64_t ow_lane = ((cw_in + row0) * p.chunk_units - hu) * kWpu +
-                          (kCarry ? kOwpe : 0) + piece * 4;
-  uint32_t* stream_out = out_words + sw * p.out_words;
-  for (int64_t q = 0; q < nsub; ++q) {
-    // first unit of this sub-chunk (in carry mode after the straddling one)
-    const int64_t ub = u_first + (kCarry ? 1 : 0) + q * su;
-    constexpr int kUpc = 4 / kWpu;          // units per 16-byte chunk
-    if (active) {
-      if (ub >= 0 && ub + su <= p.units) {
-        constexpr int kChUnroll = VInfo<V>::weight == 0 ? 8 : VInfo<V>::weight == 1 ? 2 : 1;
-#pragma unroll kChUnroll
-        for (int ch = 0; ch < pieces; ++ch) {
-          uint32_t w[4];
+  if (!active) return;
+  // the chunk's output words: its first 16-byte group starts at word w of the
+  // stream, before word 0 in a first chunk with head units
+  const int64_t w = u_first * kWpu + (kCarry ? kOwpe : 0);
+  const int64_t left = p.out_words - w;
+  const int64_t count = p.chunk_units * kWpu < left ? p.chunk_units * kWpu : left;  // words to write
+  uint32_t* dst = reinterpret_cast<uint32_t*>(p.out) + s * p.out_words + w;
+  // a group at either end of the stream: virtual units make no words, and each
+  // output word is checked
+  auto edge = [&](int64_t at) {
+    uint32_t o4[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-          for (int i = 0; i < 4; ++i) w[i] = mrg_next(st, p);
-          const uint4 o = block_outputs<V>(make_uint4(w[0], w[1], w[2], w[3]), p.t);
-          const uint32_t o4[4] = {o.x, o.y, o.z, o.w};
-          stage[warp][lane][ch ^ (lane & 7)] = kCarry ? shift_in<true, kOwpe>(carry, o4)
-                                                      : shift_in<false, kOwpe>(carry, o4);
-        }
-      } else {
-        for (int ch = 0; ch < pieces; ++ch) {
-          uint32_t o4[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-          for (int u = 0; u < kUpc; ++u) {
-            const int64_t unit = ub + ch * kUpc + u;
-            if (unit >= 0 && unit < p.units) gen_unit<V>(st, o4 + u * kWpu, p);
-          }
-          stage[warp][lane][ch ^ (lane & 7)] = kCarry ? shift_in<true, kOwpe>(carry, o4)
-                                                      : shift_in<false, kOwpe>(carry, o4);
-        }
-      }
+    for (int u = 0; u < 4 / kWpu; ++u) {
+      const int64_t unit = u_first + (kCarry ? 1 : 0) + at / kWpu + u;
+      if (unit >= 0 && unit < p.units) gen_unit<V>(st, o4 + u * kWpu, p);
     }
-    __syncwarp();
-    // interior sub-chunks (every row present and inside the stream, the
-    // common case) store without per-row checks
-    const int64_t ow0 = ow_lane + q * (4 * pieces);
-    const bool inside = ow0 >= 0 && ow0 + (pieces - 1) * row_stride + 4 <= p.out_words;
-    if (__all_sync(0xFFFFFFFFu, inside && rows_active == 32)) {
-      uint32_t* dst = stream_out + ow0;
-      if (lg == kRowLg) {
+    const uint4 v = kCarry ? shift_in<true, kOwpe>(carry, o4) : shift_in<false, kOwpe>(carry, o4);
+    const uint32_t src[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int it = 0; it < 8; ++it) {
-          const int r = it * 4 + (lane >> 3);
-          store16(dst + it * row_stride, stage[warp][r][(lane & 7) ^ (r & 7)]);
-        }
-      } else {
-        for (int it = 0; it < pieces; ++it) {
-          const int r = it * row_step + row0;
-          store16(dst + it * row_stride, stage[warp][r][piece ^ (r & 7)]);
-        }
-      }
-      __syncwarp();
-      continue;
-    }
-#pragma unroll kCopyUnroll
-    for (int it = 0; it < pieces; ++it) {
-      const int r = it * row_step + row0;
-      if (r >= rows_active) continue;
-      const int64_t ow = ow_lane + it * row_stride + q * (4 * pieces);
-      const uint4 v = stage[warp][r][piece ^ (r & 7)];
-      if (ow >= 0 && ow + 4 <= p.out_words) {
-        store16(stream_out + ow, v);
-      } else {
-        const uint32_t src[4] = {v.x, v.y, v.z, v.w};
+    for (int i = 0; i < 4; ++i)
+      if (w + at + i >= 0 && at + i < count) dst[at + i] = src[i];
+  };
+  auto group = [&]() {
+    uint32_t x[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (ow + i >= 0 && ow + i < p.out_words) stream_out[ow + i] = src[i];
-      }
-    }
-    __syncwarp();
+    for (int i = 0; i < 4; ++i) x[i] = mrg_next(st, p);
+    const uint4 o = block_outputs<V>(make_uint4(x[0], x[1], x[2], x[3]), p.t);
+    const uint32_t o4[4] = {o.x, o.y, o.z, o.w};
+    return kCarry ? shift_in<true, kOwpe>(carry, o4) : shift_in<false, kOwpe>(carry, o4);
+  };
+  int64_t at = 0;
+  if (w < 0 && count > 0) {
+    edge(0);
+    at = 4;
   }
+  uint32_t* q = dst + at;
+  uint32_t* const end = dst + (at < count ? at + (count - at) / 4 * 4 : at);  // whole groups
+  if (q != end && ((uintptr_t)q & 31u) != 0) {
+    store16(q, group());
+    q += 4;
+  }
+  uint32_t* const end32 = end - ((end - q) & 4);
+  // 48 or 24 words a turn: a multiple of three steps leaves the state where it
+  // was without moves (10^9 bits at 24, 32, 48 words: 0.860, 0.852, 0.840 ms;
+  // FP32 gaussians at 8, 24, 48: 1.476, 1.440, 1.420, lognormals 1.704, -,
+  // 1.683); the FP64 fixed-point bodies would leave the instruction cache
+  constexpr int kUnroll = VInfo<V>::weight == 0 ? 6 : VInfo<V>::weight == 1 ? 3 : 1;
+#pragma unroll kUnroll
+  for (; q != end32; q += 8) {
+    const uint4 a = group();
+    store32(q, a, group());
+  }
+  if (q != end) {
+    store16(q, group());
+    q += 4;
+  }
+  if (q - dst < count) edge(q - dst);
 }
 
 template <int V>
@@ -392,65 +355,53 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
                  : carry ? (head_e + 1) / 2
                  : per_stream ? hu_max : 0;
 
-  // Threads per SM of the chunk plan, one chunk each: 3072 (several waves,
-  // so that an SM refills as its CTAs finish) while that leaves a thread 256
-  // words or more, else 2048; or the tuned count.  10^9 bits 0.990 -> 0.958
-  // ms, 10^9 FP64 uniforms 2.518 -> 2.410 ms with 3072; 10^8 bits 0.1125
-  // with 2048, 0.1149 with 3072.
+  // Threads per SM of the chunk plan, one chunk each, or the tuned count: 3072
+  // for long fills (several waves, so that an SM refills as its CTAs finish:
+  // 10^9 FP64 gaussians 6.67 ms, with 2048 6.78), 1536 for middling ones of the
+  // shorter transforms (10^8 bits 96 us, with 2048 99), 2048 below.
   const int32_t geom = fill_geometry(GRNG_MRG32K3A, V, r.n * r.num_streams);
   const int64_t span = p.units + p.head_units;
   const int64_t words = span * I::wpu * r.num_streams;
-  const int64_t target_threads =
-      (int64_t)sms * (geom > 0 ? 256 * (int64_t)geom : words >= (int64_t)sms * 3072 * 256 ? 3072 : 2048);
+  const int64_t per_sm = geom > 0                                              ? 256 * (int64_t)geom
+                         : words >= (int64_t)sms * (I::weight == 2 ? 786432 : 2621440) ? 3072
+                         : I::weight < 2 && words >= (int64_t)sms * 393216              ? 1536
+                                                                                        : 2048;
+  const int64_t target_threads = (int64_t)sms * per_sm;
   int64_t per_stream_threads = target_threads / r.num_streams;
   if (per_stream_threads < 1) per_stream_threads = 1;
-  // Rows of 128 bytes; in a small fill of the FP64 fixed-point transforms,
-  // whose pair or inverse CDF is a long serial chain, shorter rows share that
-  // chain among more threads, up to 256 per SM (FP64 gaussians: 10^3 13.4 ->
-  // 3.7 us, 10^5 9.7 -> 5.3; with up to 512 per SM 3 10^5 take 9.6 us in place
-  // of 7.0, the jumps outweighing the chain).
-  int lg = kRowLg;
-  if (I::weight == 2 && aligned)
-    while (lg > 0 && words < ((int64_t)sms * 256 << (lg + 2))) --lg;
-  p.row_lg = lg;
-  const int64_t su = (4 << lg) / I::wpu;
-  // At least two rows a thread where that leaves 4 warps per scheduler: the
-  // jump costs a thread about 20 words' steps (10^7 FP32 uniforms 18.1 us
-  // with 64 words a thread, 20.1 with 32; 10^6 4.9 with 32, 5.3 with 64).
-  const int64_t min_cu = words >= (int64_t)sms * 512 * (8 << lg) ? 2 * su : su;
+  // Chunks of whole 32-byte pieces: at least 32 words a thread, since the jump
+  // costs about 20 words' steps, and 64 where that leaves 4 warps per
+  // scheduler (10^7 FP32 uniforms 18.1 us with 64 words a thread, 20.1 with 32;
+  // 10^6 4.9 with 32, 5.3 with 64); the FP64 fixed-point transforms, whose pair
+  // or inverse CDF is a long serial chain, down to 8 in small fills, up to 256
+  // threads per SM (FP64 gaussians: 10^3 13.4 -> 3.7 us, 10^5 9.7 -> 5.3).
+  const int64_t su = 8 / I::wpu;
+  int64_t min_words = words >= (int64_t)sms * 512 * 64 ? 64 : 32;
+  if (I::weight == 2)
+    while (min_words > 8 && words < (int64_t)sms * 256 * min_words) min_words /= 2;
+  const int64_t min_cu = min_words / I::wpu;
   int64_t cu = (span + per_stream_threads - 1) / per_stream_threads;
   if (cu < min_cu) cu = min_cu;
   cu = (cu + su - 1) / su * su;
   int64_t cps = (span + cu - 1) / cu;
-  if (r.num_streams > 1) {
-    // a multiple of 32 chunks per stream keeps each warp's 32 chunks inside
-    // one stream; the units are spread over all of them
-    cps = (cps + 31) / 32 * 32;
-    cu = (span + cps - 1) / cps;
-    cu = (cu + su - 1) / su * su;
-  }
   p.chunk_units = cu;
   p.chunks_per_stream = cps;
   p.total_chunks = p.chunks_per_stream * r.num_streams;
-  // Threads per CTA: 128 spreads a small fill's warps over more SMs and fits
-  // the light kernels' registers better (10^8 FP32 uniforms 116.6 us against
-  // 122.5 with 256, 10^5 3.7 against 4.5); the long chunks of the FP64
-  // fixed-point transforms keep 256 (10^9 FP64 gaussians 6.99 ms against 7.09).
+  // Threads per CTA: 128 spreads a small fill's warps over more SMs (10^5 FP32
+  // uniforms 3.7 us against 4.5 with 256); the long chunks of the FP64
+  // fixed-point transforms keep 256.
   const int threads = I::weight == 2 && cu * I::wpu >= 1024 ? 256 : 128;
   const int64_t grid = (p.total_chunks + threads - 1) / threads;
-  const size_t smem = (size_t)(threads / 32) * 32 * 8 * sizeof(uint4);
   if (grid > 0x7FFFFFFF) {
     set_error("MRG32k3a fill: grid too large");
     return GRNG_ERR_UNSUPPORTED;
   }
-  if (lg != kRowLg) {
-    if constexpr (I::weight == 2) mrg_fill_kernel<V, 4><<<(unsigned)grid, threads, smem, stream>>>(p);
-  } else if (aligned) {
-    mrg_fill_kernel<V, 1><<<(unsigned)grid, threads, smem, stream>>>(p);
+  if (aligned) {
+    mrg_fill_kernel<V, 1><<<(unsigned)grid, threads, 0, stream>>>(p);
   } else if (carry) {
-    if constexpr (I::epu == 2) mrg_fill_kernel<V, 2><<<(unsigned)grid, threads, smem, stream>>>(p);
+    if constexpr (I::epu == 2) mrg_fill_kernel<V, 2><<<(unsigned)grid, threads, 0, stream>>>(p);
   } else {
-    mrg_fill_kernel<V, 3><<<(unsigned)grid, threads, smem, stream>>>(p);
+    mrg_fill_kernel<V, 3><<<(unsigned)grid, threads, 0, stream>>>(p);
   }
   const cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) {
