@@ -259,7 +259,9 @@ __device__ __forceinline__ double u01_f64_dadd(uint32_t wa, uint32_t wb) {
   const uint32_t h = wa >> 11;                      // x >> 32: 21 bits
   const uint32_t l = __funnelshift_r(wb, wa, 11);   // low 32 bits of x
   const double B = __hiloint2double((int)((h & 0xFFFFFu) | 0x3FE00000u), (int)l);
-  return __dadd_rn(B, (h >> 20) != 0u ? 0.0 : -0.5);
+  // 0 or -1/2 by a mask of the top bit (selecting it: 10^9 1.409 ms, 1.383 so)
+  const uint32_t c = ~(uint32_t)((int32_t)wa >> 31) & 0xBFE00000u;
+  return __dadd_rn(B, __hiloint2double((int)c, 0));
 }
 
 // The exact affine uniform a + d u, d = 2^(e + 53), by one FP64 add: d times the

@@ -448,18 +448,70 @@ __device__ __forceinline__ void philox_rotate_body(const RotateParams& p) {
   }
 }
 
+// The transforms longer than a few operations do without the exchange: each
+// lane stores its own block in pieces of 8 (and, kOdd, 4, 8, 4) bytes, back to
+// back, and the pieces of a sector meet in L2.  Blocks [jf, jl) lie wholly inside
+// the output; the at most two others are checked word by word.
+template <bool kOdd>
+__device__ __forceinline__ void store_pieces(uint32_t* d, uint4 o) {
+  if constexpr (kOdd) {
+    d[0] = o.x;
+    *reinterpret_cast<uint2*>(d + 1) = make_uint2(o.y, o.z);
+    d[3] = o.w;
+  } else {
+    *reinterpret_cast<uint2*>(d) = make_uint2(o.x, o.y);
+    *reinterpret_cast<uint2*>(d + 2) = make_uint2(o.z, o.w);
+  }
+}
+
+template <int V, int U, bool kCross, bool kOdd>
+__device__ __forceinline__ void philox_pieces_body(const RotateParams& p) {
+  uint32_t* out = reinterpret_cast<uint32_t*>(p.out) - p.r;  // block j's words at 4 j
+  const uint32_t jf = p.r > 0 ? 1u : 0u, jl = (uint32_t)((p.nw + p.r) / 4);
+  const uint32_t tid = blockIdx.x * kThreads + threadIdx.x;
+  if (tid < 2) {
+    const uint32_t j = tid == 0 ? 0u : jl;
+    if ((tid == 0 ? jf > 0 : 4 * (int64_t)jl - p.r < p.nw) && (tid == 0 || jl > 0 || jf == 0)) {
+      const uint4 o = block_outputs<V>(philox_block<true>(j, p.ctr), p.t);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int64_t i = 4 * (int64_t)j + q - p.r;
+        if (i >= 0 && i < p.nw) out[4 * (int64_t)j + q] = word_of(o, q);
+      }
+    }
+  }
+  const uint32_t step = gridDim.x * (kThreads * U);
+  uint32_t j = jf + blockIdx.x * (kThreads * U) + threadIdx.x;
+  uint32_t* dst = out + 4 * (int64_t)j;
+  for (; j + (U - 1) * kThreads < jl; j += step, dst += 4 * (int64_t)step) {
+    uint4 o[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) o[u] = block_outputs<V>(philox_block<kCross>(j + u * kThreads, p.ctr), p.t);
+#pragma unroll
+    for (int u = 0; u < U; ++u) store_pieces<kOdd>(dst + 4 * u * kThreads, o[u]);
+  }
+  if constexpr (U > 1) {
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+      if (j + u * kThreads < jl)
+        store_pieces<kOdd>(dst + 4 * u * kThreads,
+                           block_outputs<V>(philox_block<kCross>(j + u * kThreads, p.ctr), p.t));
+  }
+}
+
 // The rotation is the same for the whole grid: one loop per rotation, each
 // with it a constant (8-byte elements rotate by one element only).
 template <int V, int U, bool kCross>
 __device__ __forceinline__ void philox_rotate_phases(const RotateParams& p) {
-  if constexpr (VInfo<V>::es == 8) {
-    philox_rotate_body<V, U, kCross, 2>(p);
-  } else {
-    switch (p.s) {
-      case 1: philox_rotate_body<V, U, kCross, 1>(p); break;
-      case 2: philox_rotate_body<V, U, kCross, 2>(p); break;
-      default: philox_rotate_body<V, U, kCross, 3>(p); break;
+  if constexpr (VInfo<V>::weight > 0) {
+    if (VInfo<V>::es == 8 || p.s == 2) {
+      philox_pieces_body<V, U, kCross, false>(p);
+    } else {
+      philox_pieces_body<V, U, kCross, true>(p);
     }
+  } else {
+    static_assert(VInfo<V>::es == 8);
+    philox_rotate_body<V, U, kCross, 2>(p);
   }
 }
 
