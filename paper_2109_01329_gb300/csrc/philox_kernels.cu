@@ -18,12 +18,11 @@
 //     neighbouring lanes by shuffle.  When the output's start splits a
 //     Box-Muller pair, lanes transform pair-aligned groups one element
 //     earlier and exchange the straddling element too (30 groups per warp).
-//   * rotate kernel (one stream of 2- or 4-word units at a word offset
-//     that keeps them inside blocks, the output start at another 16-byte
-//     phase): each lane transforms its own block and rotates its outputs
-//     into the group that lane - 1's block opens, by shuffle; lane 0 and
-//     lane 31 write the groups shared with the neighbouring warps' chunks
-//     with narrower stores, so no unit is transformed twice.
+//   * pieces kernel (one stream of 2- or 4-word units at a word offset that
+//     keeps them inside blocks, the output start at another 16-byte phase):
+//     each lane transforms its own block and stores it in 4- and 8-byte
+//     pieces; the FP64 uniforms, near the write roof, rotate their outputs into
+//     whole groups by shuffle instead (rotate kernel).
 //   * multi-shift kernel: substreams at another phase or alignment, the
 //     shift kernel's exchange applied per stream (a warp works on 30 groups
 //     of one stream).
@@ -327,19 +326,12 @@ __global__ void __launch_bounds__(kThreads, 5) philox_shift_kernel_5(const __gri
   philox_shift_phases<V, U, kCross, kSplit>(p);
 }
 
-// ------------------------------------------------------ single stream, rotated
+// ----------------------------------- single stream, whole units, another phase
 // One stream whose units lie inside counter blocks (the word offset a multiple
 // of the words per unit) while its output start is not at the blocks' 16-byte
 // phase.  Block j's four output words are then output words 4 j - r .. 4 j -
-// r + 3 (r = word offset mod 4): the last kS = (h - r) mod 4 of them open the
-// next 16-byte group (h: output words of out's group before out).  Each lane
-// transforms its own block once and completes its group from the last kS
-// output words of lane - 1 by shuffle; lane 0 writes only its own part of its
-// group and lane 31 the opening words of the next group, with 4- or 8-byte
-// stores at constant offsets from the group's address, so a warp writes 32
-// groups per 32 blocks and no unit is transformed twice (the shift kernel's
-// split form transforms 2 virtual groups in 32 twice).
-struct RotateParams {
+// r + 3 (r = word offset mod 4).
+struct PiecesParams {
   TransformParams t;
   uint4* gbase;       // out's 16-byte group
   char* out;          // element 0
@@ -349,109 +341,18 @@ struct RotateParams {
   int64_t gofs;       // the group lane l completes is out's group + j + gofs (0 or -1)
   int64_t chunks;     // ceil(blocks / 32)
   PhiloxStream ctr;   // block 0: that of the stream's first word
-  uint32_t s;         // the rotation kS, 1..3
 };
-
-// (lane - 1's last kS output words, this lane's first 4 - kS)
-template <int kS>
-__device__ __forceinline__ uint4 rotate_up(uint4 o) {
-  const uint32_t n3 = __shfl_up_sync(0xFFFFFFFFu, o.w, 1);
-  if constexpr (kS == 1) {
-    return make_uint4(n3, o.x, o.y, o.z);
-  } else {
-    const uint32_t n2 = __shfl_up_sync(0xFFFFFFFFu, o.z, 1);
-    if constexpr (kS == 2) {
-      return make_uint4(n2, n3, o.x, o.y);
-    } else {
-      const uint32_t n1 = __shfl_up_sync(0xFFFFFFFFu, o.y, 1);
-      return make_uint4(n1, n2, n3, o.x);
-    }
-  }
-}
 
 __device__ __forceinline__ uint32_t word_of(uint4 v, int q) {
   return q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w;
 }
 
-// Positions [q0, q1) of the 16-byte group at g, position q taking word
-// q + kFrom of v; 8-byte elements go out whole (q0 and q1 even for them).
-template <int V, int q0, int q1, int kFrom>
-__device__ __forceinline__ void store_positions(uint4* g, uint4 v) {
-  if constexpr (VInfo<V>::es == 4) {
-#pragma unroll
-    for (int q = q0; q < q1; ++q) reinterpret_cast<uint32_t*>(g)[q] = word_of(v, q + kFrom);
-  } else {
-#pragma unroll
-    for (int q = q0; q < q1; q += 2)
-      reinterpret_cast<uint2*>(g)[q >> 1] = make_uint2(word_of(v, q + kFrom), word_of(v, q + kFrom + 1));
-  }
-}
-
-// The same with each output word checked against [0, nw) (edge chunks).
-template <int V, int q0, int q1, int kFrom>
-__device__ __forceinline__ void store_positions_checked(const RotateParams& p, int64_t G, uint4 v) {
-  constexpr int kStep = VInfo<V>::es / 4;
-#pragma unroll
-  for (int q = q0; q < q1; q += kStep) {
-    const int64_t i = 4 * G + q - p.h;
-    if (i >= 0 && i < p.nw) {
-      if constexpr (kStep == 1) {
-        reinterpret_cast<uint32_t*>(p.out)[i] = word_of(v, q + kFrom);
-      } else {
-        reinterpret_cast<uint2*>(p.out)[i >> 1] =
-            make_uint2(word_of(v, q + kFrom), word_of(v, q + kFrom + 1));
-      }
-    }
-  }
-}
-
-template <int V, int U, bool kCross, int kS>
-__device__ __forceinline__ void philox_rotate_body(const RotateParams& p) {
-  const int lane = threadIdx.x & 31;
-  const int64_t TW = (int64_t)gridDim.x * (kThreads / 32);
-  const int64_t c0 = ((int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * U;
-  // a warp takes U consecutive chunks; lane l of chunk c holds block j =
-  // 32 c + l, and those of the U chunks lie at constant offsets
-  const int64_t dj = TW * 32;
-  int64_t j = c0 * 32 + lane;
-  uint4* dst = p.gbase + (j + p.gofs);
-  // the loop bound depends only on the warp: every shuffle has all 32 lanes
-  for (int64_t c = c0; c < p.chunks; c += U * TW, j += U * dj, dst += U * dj) {
-    uint4 b[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) b[u] = philox_block<kCross>((uint32_t)j + u * 32, p.ctr);
-    // every output word of this iteration's chunks lies inside the output
-    // (uniform): words 128 c - r .. 128 c' + 127 - r, c' the last chunk
-    const bool interior = c * 128 - p.r >= 0 && (c + U) * 128 - 1 - p.r < p.nw;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint4 o = block_outputs<V>(b[u], p.t);
-      const uint4 g = rotate_up<kS>(o);
-      if (interior) {
-        uint4* gp = dst + u * 32;
-        if (lane > 0) {
-          *gp = g;
-        } else {
-          store_positions<V, kS, 4, 0>(gp, g);
-        }
-        if (lane == 31) store_positions<V, 0, kS, 4 - kS>(gp + 1, o);
-      } else {
-        const int64_t G = j + u * 32 + p.gofs;
-        if (lane > 0) {
-          store_positions_checked<V, 0, 4, 0>(p, G, g);
-        } else {
-          store_positions_checked<V, kS, 4, 0>(p, G, g);
-        }
-        if (lane == 31) store_positions_checked<V, 0, kS, 4 - kS>(p, G + 1, o);
-      }
-    }
-  }
-}
-
-// The transforms longer than a few operations do without the exchange: each
-// lane stores its own block in pieces of 8 (and, kOdd, 4, 8, 4) bytes, back to
+// Each lane stores its own block in pieces of 8 (kOdd: 4, 8, 4) bytes, back to
 // back, and the pieces of a sector meet in L2.  Blocks [jf, jl) lie wholly inside
-// the output; the at most two others are checked word by word.
+// the output; the at most two others are checked word by word.  10^8 FP32
+// gaussians 117 to 119 us at the three phases against 114 aligned, where
+// rotating them into whole groups by shuffle took 131 and 136; FP64 gaussians 574
+// against 660.
 template <bool kOdd>
 __device__ __forceinline__ void store_pieces(uint32_t* d, uint4 o) {
   if constexpr (kOdd) {
@@ -465,7 +366,7 @@ __device__ __forceinline__ void store_pieces(uint32_t* d, uint4 o) {
 }
 
 template <int V, int U, bool kCross, bool kOdd>
-__device__ __forceinline__ void philox_pieces_body(const RotateParams& p) {
+__device__ __forceinline__ void philox_pieces_body(const PiecesParams& p) {
   uint32_t* out = reinterpret_cast<uint32_t*>(p.out) - p.r;  // block j's words at 4 j
   const uint32_t jf = p.r > 0 ? 1u : 0u, jl = (uint32_t)((p.nw + p.r) / 4);
   const uint32_t tid = blockIdx.x * kThreads + threadIdx.x;
@@ -499,30 +400,69 @@ __device__ __forceinline__ void philox_pieces_body(const RotateParams& p) {
   }
 }
 
-// The rotation is the same for the whole grid: one loop per rotation, each
-// with it a constant (8-byte elements rotate by one element only).
 template <int V, int U, bool kCross>
-__device__ __forceinline__ void philox_rotate_phases(const RotateParams& p) {
-  if constexpr (VInfo<V>::weight > 0) {
-    if (VInfo<V>::es == 8 || p.s == 2) {
-      philox_pieces_body<V, U, kCross, false>(p);
-    } else {
-      philox_pieces_body<V, U, kCross, true>(p);
-    }
+__device__ __forceinline__ void philox_pieces_phases(const PiecesParams& p) {
+  if (VInfo<V>::es == 8 || ((p.h - p.r) & 1) == 0) {
+    philox_pieces_body<V, U, kCross, false>(p);
   } else {
-    static_assert(VInfo<V>::es == 8);
-    philox_rotate_body<V, U, kCross, 2>(p);
+    philox_pieces_body<V, U, kCross, true>(p);
   }
 }
 
 template <int V, int U, bool kCross>
-__global__ void __launch_bounds__(kThreads) philox_rotate_kernel(const __grid_constant__ RotateParams p) {
-  philox_rotate_phases<V, U, kCross>(p);
+__global__ void __launch_bounds__(kThreads) philox_pieces_kernel(const __grid_constant__ PiecesParams p) {
+  philox_pieces_phases<V, U, kCross>(p);
 }
 
 template <int V, int U, bool kCross>
-__global__ void __launch_bounds__(kThreads, 5) philox_rotate_kernel_5(const __grid_constant__ RotateParams p) {
-  philox_rotate_phases<V, U, kCross>(p);
+__global__ void __launch_bounds__(kThreads, 5) philox_pieces_kernel_5(const __grid_constant__ PiecesParams p) {
+  philox_pieces_phases<V, U, kCross>(p);
+}
+
+// The FP64 uniforms: a block's second double opens the next 16-byte group, so
+// each lane completes its group from lane - 1's by shuffle; lane 0 stores only
+// its own half of its group and lane 31 the opening half of the next, so a warp
+// writes 32 groups per 32 blocks (10^8 172 us; in 8-byte pieces 188).
+template <int V, int U, bool kCross>
+__global__ void __launch_bounds__(kThreads) philox_rotate_kernel(const __grid_constant__ PiecesParams p) {
+  static_assert(VInfo<V>::es == 8 && VInfo<V>::wpu == 2);
+  const int lane = threadIdx.x & 31;
+  const int64_t TW = (int64_t)gridDim.x * (kThreads / 32);
+  const int64_t c0 = ((int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * U;
+  // a warp takes U consecutive chunks; lane l of chunk c holds block j =
+  // 32 c + l, and those of the U chunks lie at constant offsets
+  const int64_t dj = TW * 32;
+  int64_t j = c0 * 32 + lane;
+  uint4* dst = p.gbase + (j + p.gofs);
+  // the loop bound depends only on the warp: every shuffle has all 32 lanes
+  for (int64_t c = c0; c < p.chunks; c += U * TW, j += U * dj, dst += U * dj) {
+    uint4 b[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) b[u] = philox_block<kCross>((uint32_t)j + u * 32, p.ctr);
+    // every output word of this iteration's chunks lies inside the output
+    // (uniform): words 128 c - r .. 128 (c + U) - 1 - r
+    const bool interior = c * 128 - p.r >= 0 && (c + U) * 128 - 1 - p.r < p.nw;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint4 o = block_outputs<V>(b[u], p.t);
+      const uint32_t n2 = __shfl_up_sync(0xFFFFFFFFu, o.z, 1);
+      const uint32_t n3 = __shfl_up_sync(0xFFFFFFFFu, o.w, 1);
+      if (interior) {
+        uint4* gp = dst + u * 32;
+        if (lane > 0) {
+          *gp = make_uint4(n2, n3, o.x, o.y);
+        } else {
+          reinterpret_cast<uint2*>(gp)[1] = make_uint2(o.x, o.y);
+        }
+        if (lane == 31) *reinterpret_cast<uint2*>(gp + 1) = make_uint2(o.z, o.w);
+      } else {  // each of the block's two doubles checked
+        const int64_t e = (4 * (j + u * 32) - p.r) >> 1;
+        uint2* out = reinterpret_cast<uint2*>(p.out);
+        if (e >= 0 && 2 * e < p.nw) out[e] = make_uint2(o.x, o.y);
+        if (e + 1 >= 0 && 2 * (e + 1) < p.nw) out[e + 1] = make_uint2(o.z, o.w);
+      }
+    }
+  }
 }
 
 // ------------------------------------------------------------ substreams
@@ -829,29 +769,29 @@ void launch_shift(ShiftParams& p, const uint32_t* key, uint64_t a_lo, uint64_t a
   (cross ? k_cross : k_same)<<<(unsigned)grid, kThreads, 0, stream>>>(p);
 }
 
-// Launches the rotate kernel (units inside blocks, output start at another
-// phase); p.t, p.out, p.gbase, p.nw, p.h, p.rk are set by the caller.
+// Launches the pieces or the rotate kernel (units inside blocks, output start at
+// another phase); p.t, p.out, p.gbase, p.nw, p.h are set by the caller.
 template <int V>
-void launch_rotate(RotateParams& p, const uint32_t* key, uint64_t off_lo, uint64_t off_hi, int sms,
+void launch_pieces(PiecesParams& p, const uint32_t* key, uint64_t off_lo, uint64_t off_hi, int sms,
                    int32_t geom, cudaStream_t stream) {
+  constexpr bool kRotate = VInfo<V>::weight == 0;
   constexpr int kU = exchange_blocks_per_thread<V>();
   p.r = (int64_t)(off_lo & 3u);
-  const int64_t d = p.h - p.r;
-  p.s = (uint32_t)((d + 4) & 3);
-  p.gofs = d < 0 ? -1 : 0;
+  p.gofs = p.h - p.r < 0 ? -1 : 0;
   p.ctr = philox_stream(key[0], key[1], (off_lo >> 2) | (off_hi << 62), off_hi >> 2);
   const int64_t blocks = (p.nw - 1 + p.r) / 4 + 1;
   p.chunks = (blocks + 31) / 32;
-  void (*k_same)(const RotateParams);
-  void (*k_cross)(const RotateParams);
-  // the FP64 Box-Muller variants gain from a fifth CTA as in the stream
-  // kernel; the FP32 ones would spill under its register cap here
-  if constexpr (stream_wants_5_ctas<V>() && VInfo<V>::es == 8) {
-    k_same = philox_rotate_kernel_5<V, kU, false>;
-    k_cross = philox_rotate_kernel_5<V, kU, true>;
-  } else {
+  void (*k_same)(const PiecesParams);
+  void (*k_cross)(const PiecesParams);
+  if constexpr (kRotate) {
     k_same = philox_rotate_kernel<V, kU, false>;
     k_cross = philox_rotate_kernel<V, kU, true>;
+  } else if constexpr (stream_wants_5_ctas<V>()) {
+    k_same = philox_pieces_kernel_5<V, kU, false>;
+    k_cross = philox_pieces_kernel_5<V, kU, true>;
+  } else {
+    k_same = philox_pieces_kernel<V, kU, false>;
+    k_cross = philox_pieces_kernel<V, kU, true>;
   }
   static std::atomic<int> occ[2] = {{0}, {0}};
   int o = occ[0].load(std::memory_order_relaxed);
@@ -1005,13 +945,13 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
     // one stream whose units lie inside counter blocks, the output start at
     // another phase (e.g. a Box-Muller pair split by the pointer)
     if constexpr (I::wpu >= 2) {
-      RotateParams p;
+      PiecesParams p;
       p.t = r.t;
       p.out = reinterpret_cast<char*>(r.out);
       p.gbase = reinterpret_cast<uint4*>(addr - phase_w * 4u);
       p.nw = r.n * (I::es / 4);
       p.h = (int64_t)phase_w;
-      launch_rotate<V>(p, r.key, r.off_lo, r.off_hi, sms, geom, stream);
+      launch_pieces<V>(p, r.key, r.off_lo, r.off_hi, sms, geom, stream);
     }
   } else if (r.num_streams == 1 &&
              ((phase_w % (uint32_t)I::wpu) == 0 || (I::epu == 2 && (head & 1) != 0))) {
