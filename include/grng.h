@@ -329,7 +329,8 @@ GRNG_API grng_status grng_batch_create(grng_batch_t* out, const grng_request* re
                                        int32_t ipt, void* dev_workspace, size_t workspace_bytes,
                                        grng_stream_t stream);
 
-/* Enqueues the fill kernel and the offset-advance kernel on `stream`: no host
+/* Enqueues the fill kernel on `stream`, which counts its launches in the
+ * workspace so that the next one continues each sequence: no host
  * synchronisation, no allocation; may be captured into a CUDA graph. */
 GRNG_API grng_status grng_batch_launch(grng_batch_t batch, grng_stream_t stream);
 
@@ -337,7 +338,7 @@ GRNG_API grng_status grng_batch_launch(grng_batch_t batch, grng_stream_t stream)
  * portable native kernels; Sec. 7 shows small batches dominated by per-call
  * overheads).  Times the fill over the launch geometries ipt (16-byte groups
  * per thread per tile: 1, 2, 4, 8, 16, 32) x CTAs per SM (1, 2, 4, 6, 8, 12,
- * 16), without advancing the offsets (the outputs are rewritten
+ * 16, 24, 32), without advancing the offsets (the outputs are rewritten
  * identically), and keeps the fastest.  Only the ipt values whose tile map
  * fits the workspace given to grng_batch_create are tried: a workspace of
  * grng_batch_workspace_bytes(..., ipt = 1, ...) admits every one.  The
