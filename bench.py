@@ -625,7 +625,7 @@ def run_batched(grng, torch, dev, reps):
             "batched_write_gbs": round(out_bytes / med_batch / 1e6, 1),
             "per_request_gsamples_s": round(total / med_loop / 1e6, 2),
             "autotune": {"ipt": ipt, "ctas_per_sm": ctas, "ms": round(tune_ms, 4),
-                         "searched": "ipt {1,2,4,8,16,32} x CTAs/SM {1,2,4,6,8,12,16}"},
+                         "searched": "ipt {1,2,4,8,16,32} x CTAs/SM {1,2,4,6,8,12,16,24,32}"},
             "reps": reps}
 
 
