@@ -145,35 +145,114 @@ __device__ __forceinline__ void tile_blocks_loop(const TransformParams& t, const
 // words, and elements, between neighbouring lanes as in the single-stream
 // shift kernel.  The loop bound depends only on the warp, so every shuffle has
 // all 32 lanes.
-template <int V, bool kCross, bool kSplit>
+//
+// kPh: the word phase as a constant (only the words needed cross lanes), or -1
+// to read it from ph; two chunks per warp at once with a constant phase.  Bits
+// and the uniforms, whose share the exchange is largest of, take it: with
+// tile_halves_loop below the table of 4096 requests 568 -> 541 us a launch, three
+// in four of its requests at another phase.
+template <int V, bool kCross, bool kSplit, int kPh = -1>
 __device__ __forceinline__ void tile_shift_loop(const TransformParams& t, const TileBlocks& q,
                                                 uint32_t ph, const TileOut& out) {
   using I = VInfo<V>;
   constexpr uint32_t kPerWarp = kSplit ? 30 : 31;
+  constexpr uint32_t U = kPh > 0 && I::es == 4 ? 2 : 1;
   const uint32_t lane = threadIdx.x & 31u;
-  for (uint32_t c = (threadIdx.x >> 5) * kPerWarp; c < out.count; c += kPerWarp * (kThreads / 32)) {
+  for (uint32_t c = (threadIdx.x >> 5) * (kPerWarp * U); c < out.count;
+       c += kPerWarp * U * (kThreads / 32)) {
     const uint32_t i = c + lane;
-    const uint4 b = q.at<kCross>(i);
-    uint4 w = b;
-    if ((!kSplit && !kCross) || ph != 0) {
-      const uint32_t n0 = __shfl_down_sync(0xFFFFFFFFu, b.x, 1);
-      const uint32_t n1 = __shfl_down_sync(0xFFFFFFFFu, b.y, 1);
-      const uint32_t n2 = __shfl_down_sync(0xFFFFFFFFu, b.z, 1);
-      if (ph == 1) {
-        w = make_uint4(b.y, b.z, b.w, n0);
-      } else if (ph == 2) {
-        w = make_uint4(b.z, b.w, n0, n1);
-      } else {
-        w = make_uint4(b.w, n0, n1, n2);
+    uint4 b[U];
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) b[u] = q.at<kCross>(i + u * kPerWarp);
+    const bool whole = c >= out.wf && c + kPerWarp * U <= out.wl;  // (uniform)
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      uint4 w = b[u];
+      if constexpr (kPh > 0) {
+        const uint32_t n0 = __shfl_down_sync(0xFFFFFFFFu, b[u].x, 1);
+        if constexpr (kPh == 1) {
+          w = make_uint4(b[u].y, b[u].z, b[u].w, n0);
+        } else {
+          const uint32_t n1 = __shfl_down_sync(0xFFFFFFFFu, b[u].y, 1);
+          if constexpr (kPh == 2) {
+            w = make_uint4(b[u].z, b[u].w, n0, n1);
+          } else {
+            w = make_uint4(b[u].w, n0, n1, __shfl_down_sync(0xFFFFFFFFu, b[u].z, 1));
+          }
+        }
+      } else if ((!kSplit && !kCross) || ph != 0) {
+        const uint32_t n0 = __shfl_down_sync(0xFFFFFFFFu, b[u].x, 1);
+        const uint32_t n1 = __shfl_down_sync(0xFFFFFFFFu, b[u].y, 1);
+        const uint32_t n2 = __shfl_down_sync(0xFFFFFFFFu, b[u].z, 1);
+        if (ph == 1) {
+          w = make_uint4(b[u].y, b[u].z, b[u].w, n0);
+        } else if (ph == 2) {
+          w = make_uint4(b[u].z, b[u].w, n0, n1);
+        } else {
+          w = make_uint4(b[u].w, n0, n1, n2);
+        }
+      }
+      uint4 o = block_outputs<V>(w, t);
+      if constexpr (kSplit) {
+        const uint32_t m0 = __shfl_down_sync(0xFFFFFFFFu, o.x, 1);
+        const uint32_t m1 = __shfl_down_sync(0xFFFFFFFFu, o.y, 1);
+        o = I::es == 4 ? make_uint4(o.y, o.z, o.w, m0) : make_uint4(o.z, o.w, m0, m1);
+      }
+      if (lane < kPerWarp) {
+        const uint32_t g = i + u * kPerWarp;
+        if (whole) {
+          out.dst[g] = o;
+        } else if (g < out.count) {
+          tile_store<V>(out, g, o);
+        }
       }
     }
-    uint4 o = block_outputs<V>(w, t);
-    if constexpr (kSplit) {
-      const uint32_t m0 = __shfl_down_sync(0xFFFFFFFFu, o.x, 1);
-      const uint32_t m1 = __shfl_down_sync(0xFFFFFFFFu, o.y, 1);
-      o = I::es == 4 ? make_uint4(o.y, o.z, o.w, m0) : make_uint4(o.z, o.w, m0, m1);
+  }
+}
+
+// FP32 Box-Muller pairs at word phase 2: block i holds the last pair of group
+// i - 1 and the first of group i, so each lane stores its own block as two
+// 8-byte pieces.  A tile takes the blocks 0 .. count, of the first and the last
+// one only the half that lies in it.
+template <int V>
+__device__ __forceinline__ void tile_halves_loop(const TransformParams& t, const TileBlocks& q,
+                                                 const TileOut& out) {
+  static_assert(VInfo<V>::es == 4 && VInfo<V>::wpu == 2);
+  constexpr uint32_t U = 2;
+  // blocks [wf + 1, wl) lie wholly in whole groups; at most two before them and
+  // two after them, each element checked
+  const uint32_t before = out.wf + 1 < out.count + 1 ? out.wf + 1 : out.count + 1;
+  const uint32_t after = out.wl > before ? out.wl : before;
+  if (threadIdx.x < 4) {
+    const uint32_t i = threadIdx.x < 2 ? threadIdx.x : after + threadIdx.x - 2;
+    if (threadIdx.x < 2 ? i < before : i <= out.count) {
+      const uint4 o = block_outputs<V>(q.at<false>(i), t);
+      const uint32_t ow[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int64_t m = 4 * (int64_t)i - 2 + k, e = out.e0 + m;  // in the tile, in the request
+        if (m >= 0 && m < 4 * (int64_t)out.count && e >= 0 && e < out.n)
+          reinterpret_cast<uint32_t*>(out.base)[e] = ow[k];
+      }
     }
-    if (lane < kPerWarp && i < out.count) tile_store<V>(out, i, o);
+  }
+  uint32_t i = before + threadIdx.x;
+  uint2* dst = reinterpret_cast<uint2*>(out.dst) + 2 * (int64_t)i;
+  for (; i + (U - 1) * kThreads < after; i += U * kThreads, dst += 2 * U * kThreads) {
+    uint4 o[U];
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) o[u] = block_outputs<V>(q.at<false>(i + u * kThreads), t);
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      uint2* d = dst + 2 * u * kThreads;
+      d[-1] = make_uint2(o[u].x, o[u].y);
+      d[0] = make_uint2(o[u].z, o[u].w);
+    }
+  }
+  for (; i < after; i += kThreads, dst += 2 * kThreads) {
+    const uint4 o = block_outputs<V>(q.at<false>(i), t);
+    dst[-1] = make_uint2(o.x, o.y);
+    dst[0] = make_uint2(o.z, o.w);
   }
 }
 
@@ -221,6 +300,18 @@ __device__ __forceinline__ void batch_tile(const BatchReq& r, uint64_t off_lo, u
     tile_shift_loop<V, true, false>(t, q, ph, out);
   } else if (ph == 0) {
     tile_blocks_loop<V>(t, q, out);
+  } else if (I::es == 4 && I::epu == 2 && ph == 2) {
+    if constexpr (I::es == 4 && I::epu == 2) tile_halves_loop<V>(t, q, out);
+  } else if (I::wpu <= 2 && I::weight == 0 && ph == 2) {
+    if constexpr (I::wpu <= 2 && I::weight == 0) tile_shift_loop<V, false, false, 2>(t, q, ph, out);
+  } else if (I::wpu == 1 && I::weight == 0) {
+    if constexpr (I::wpu == 1 && I::weight == 0) {
+      if (ph == 1) {
+        tile_shift_loop<V, false, false, 1>(t, q, ph, out);
+      } else {
+        tile_shift_loop<V, false, false, 3>(t, q, ph, out);
+      }
+    }
   } else {
     tile_shift_loop<V, false, false>(t, q, ph, out);
   }
@@ -231,7 +322,8 @@ __device__ __forceinline__ void batch_tile(const BatchReq& r, uint64_t off_lo, u
 // Bound by issue and the FMA-heavy pipe (bits: 59 instructions per group, 44 in
 // the single-stream kernel; the rest is the set-up per run of tiles and
 // fewer blocks in flight).  The table of 4096 requests at the built-in geometry:
-// 858 -> 603 us a launch (five CTAs per SM, 48 registers and 376 bytes spilled:
+// 858 -> 603 us a launch, 541 with the FP64 add for [-1, 1) and the phases as
+// constants (at 603, five CTAs per SM, 48 registers and 376 bytes spilled:
 // 5 % slower than four).
 template <bool kHeavy>
 __global__ void __launch_bounds__(kThreads, 4) batch_fill_kernel(const BatchReq* __restrict__ reqs,

@@ -260,3 +260,30 @@ def test_launches_continue_across_carries_and_tile_runs(g, heavy):
     b.commit()
     for (e, _, _), (r, _, _, _, _) in zip(reqs, refs):
         assert e.offset == r.offset
+
+
+@pytest.mark.parametrize("kind, dtype", [(0, 0), (1, 1), (1, 2), (2, 1), (3, 1), (4, 1)])
+def test_every_phase_at_the_edges_of_tiles_and_chunks(g, kind, dtype):
+    """Sizes around a group, a warp's one and two chunks of 31 groups and a tile of
+    256 groups, at every word phase and output alignment: equal to the
+    per-request call bit for bit, nothing written outside."""
+    epg = 2 if dtype == 2 else 4  # elements per group
+    sizes = [m * epg + d for m in (0, 1, 2, 30, 31, 61, 62, 63, 256, 257, 258, 512, 1000) for d in (-1, 0, 1, 2)]
+    d = g.Distribution(kind, dtype, 0.0, 1.0 if kind else 0.0)
+    reqs, refs = [], []
+    for i, n in enumerate(n for n in sizes if n > 0):
+        for phase in range(4):
+            lead = (i + phase) % 3 if i % 2 else 0
+            buf = torch.zeros(n + 8, dtype=TDT[dtype], device="cuda")
+            reqs.append((g.Engine(0, i, phase), d, buf[lead:lead + n]))
+            refs.append((g.Engine(0, i, phase), torch.zeros(n, dtype=TDT[dtype], device="cuda"), buf, lead))
+    for ipt in (1, 8):
+        b = g.Batch(reqs, ipt=ipt)
+        b.launch()
+        for e, ref, _, _ in refs:
+            g.generate(d, e.copy(), ref)
+        torch.cuda.synchronize()
+        for (e, ref, buf, lead) in refs:
+            n = ref.numel()
+            assert torch.equal(buf[lead:lead + n].clone().view(torch.uint8), ref.view(torch.uint8)), (n, e.offset, lead)
+            assert not buf[:lead].any() and not buf[lead + n:].any(), (n, e.offset, lead)
