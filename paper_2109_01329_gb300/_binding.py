@@ -229,9 +229,9 @@ class Distribution:
     def _c(self) -> _Dist:
         return _Dist(self.kind, self.dtype, float(self.p0), float(self.p1))
 
-    def __post_init__(self):
-        # the fields are frozen: the C form is made once (read-only to the library)
-        object.__setattr__(self, "_cached", None)
+    # the fields are frozen: the C form is made once, at the first call that
+    # takes it (read-only to the library)
+    _cached = None
 
     def _ref(self) -> _Dist:
         if self._cached is None:
@@ -244,7 +244,6 @@ class Distribution:
     def __setstate__(self, state):
         for k, v in state.items():
             object.__setattr__(self, k, v)
-        object.__setattr__(self, "_cached", None)
 
     @staticmethod
     def bits() -> "Distribution":
