@@ -153,6 +153,7 @@ __device__ __forceinline__ void apply(const uint4* r, uint32_t& x0, uint32_t& x1
 // length and stride, so a launch prepares nothing.
 __device__ __forceinline__ void jump(MrgRegs& s, uint64_t e_lo, uint64_t e_hi) {
   const uint4* row = reinterpret_cast<const uint4*>(d_mrg_digits.row[0]);
+  static_assert(alignof(mrg::DigitTable) >= 16 && mrg::kRowWords % 4 == 0);
   constexpr int kRow16 = mrg::kRowWords / 4;
   while (__any_sync(0xFFFFFFFFu, (e_lo | e_hi) != 0)) {
     const uint32_t k = (uint32_t)e_lo & 31u;

@@ -67,10 +67,11 @@ constexpr PowTable make_pow_table() {
 
 // A^(k 2^(5 d)) for the 26 radix-32 digits d of a 128-bit exponent and
 // k = 0..31 (k = 0 the identity): words 0..8 of a row are A1's power, 12..20
-// A2's, row-major, so that each is a run of 16-byte loads.
+// A2's, row-major, so that each is a run of 16-byte loads, which the type's
+// alignment makes good wherever the linker lays the table.
 constexpr int kDigits = 26;
 constexpr int kRowWords = 24;
-struct DigitTable {
+struct alignas(16) DigitTable {
   uint32_t row[kDigits * 32][kRowWords];
 };
 
