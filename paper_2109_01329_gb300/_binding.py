@@ -540,7 +540,11 @@ def transform_words(dist: Distribution, words, out, n: int | None = None, stream
         raise ValueError("words and out must be contiguous CUDA tensors")
     if not _torch_dtype_ok(out, dist.dtype):
         raise ValueError("out dtype does not match the distribution")
-    n = out.numel() if n is None else n
+    numel = out.numel()
+    if n is None:
+        n = numel
+    elif n > numel:
+        raise ValueError("n exceeds the tensor size")
     if words.numel() * words.element_size() < 4 * words_for(dist, n):
         raise ValueError("not enough words")
     _on_device(out.get_device(), stream, "grng_transform_words", load().grng_transform_words,
