@@ -573,7 +573,10 @@ class Batch:
         dev = None
         for i, r in enumerate(self._reqs):
             engine, dist, out = r[0], r[1], r[2]
-            n = r[3] if len(r) > 3 else out.numel()
+            numel = out.numel()
+            n = r[3] if len(r) > 3 else numel
+            if n > numel:
+                raise ValueError(f"request {i}: n exceeds the tensor size")
             if not out.is_cuda or not _torch_dtype_ok(out, dist.dtype):
                 raise ValueError(f"request {i}: out must be a CUDA tensor of the dtype")
             dev = out.device

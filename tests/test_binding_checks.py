@@ -48,3 +48,10 @@ def test_transform_words_refuses_more_outputs_than_out_holds(g, dtype):
     out = CudaTensor(100, torch.float32 if dtype == 1 else torch.float64)
     with pytest.raises(ValueError, match="n exceeds the tensor size"):
         g.transform_words(d, CudaTensor(1000, torch.int32), out, n=101)
+
+
+def test_batch_refuses_more_outputs_than_out_holds(g):
+    d = g.Distribution.uniform(0.0, 1.0)
+    fits = (g.Engine(g.PHILOX4X32X10, 1), d, CudaTensor(100), 100)
+    with pytest.raises(ValueError, match="request 1: n exceeds the tensor size"):
+        g.Batch([fits, (g.Engine(g.PHILOX4X32X10, 2), d, CudaTensor(100), 101)])
