@@ -579,6 +579,8 @@ class Batch:
                 raise ValueError(f"request {i}: n exceeds the tensor size")
             if not out.is_cuda or not _torch_dtype_ok(out, dist.dtype):
                 raise ValueError(f"request {i}: out must be a CUDA tensor of the dtype")
+            if not out.is_contiguous():
+                raise ValueError(f"request {i}: out must be contiguous")
             dev = out.device
             arr[i].engine = engine.handle
             arr[i].dist = dist._c()

@@ -55,3 +55,10 @@ def test_batch_refuses_more_outputs_than_out_holds(g):
     fits = (g.Engine(g.PHILOX4X32X10, 1), d, CudaTensor(100), 100)
     with pytest.raises(ValueError, match="request 1: n exceeds the tensor size"):
         g.Batch([fits, (g.Engine(g.PHILOX4X32X10, 2), d, CudaTensor(100), 101)])
+
+
+def test_batch_refuses_outputs_with_gaps(g):
+    """A batch writes a request's outputs densely from its tensor's address."""
+    d = g.Distribution.uniform(0.0, 1.0)
+    with pytest.raises(ValueError, match="request 0: out must be contiguous"):
+        g.Batch([(g.Engine(g.PHILOX4X32X10, 1), d, CudaTensor(100, contiguous=False), 100)])
