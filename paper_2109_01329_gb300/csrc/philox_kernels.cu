@@ -727,6 +727,18 @@ int blocks_per_sm(K kernel) {
   return b;
 }
 
+// The same kept in a slot of the kernel's own, 0 until it is known: launches may
+// come from several host threads, and each finds its slot filled or fills it.
+template <typename K>
+int resident_ctas(std::atomic<int>& slot, K kernel) {
+  int o = slot.load(std::memory_order_relaxed);
+  if (o == 0) {
+    o = blocks_per_sm(kernel);
+    slot.store(o, std::memory_order_relaxed);
+  }
+  return o;
+}
+
 // Launches the shift kernel: words of (virtual) group 0 start at word a of
 // the stream (128-bit, a = off - head words, one element earlier for kSplit).
 template <int V, bool kSplit>
@@ -737,36 +749,24 @@ void launch_shift(ShiftParams& p, const uint32_t* key, uint64_t a_lo, uint64_t a
   p.ctr = philox_stream(key[0], key[1], (a_lo >> 2) | (a_hi << 62), a_hi >> 2);
   p.ph = (uint32_t)(a_lo & 3u);
   p.chunks = (p.groups + kPer - 1) / kPer;
-  void (*k_same)(const ShiftParams);
-  void (*k_cross)(const ShiftParams);
+  // a warp's turn starts below chunk `chunks` and takes kU of them: the blocks lie
+  // below (chunks + kU) kPer + 32 past base
+  const uint64_t reach = (uint64_t)(p.chunks + kU) * (uint64_t)kPer + 32u;
+  const bool cross = p.ctr.x0 + reach >= kPhiloxMaxBlocks;
+  void (*kernel)(const ShiftParams);
   if constexpr (stream_wants_5_ctas<V>()) {
-    k_same = philox_shift_kernel_5<V, kU, false, kSplit>;
-    k_cross = philox_shift_kernel_5<V, kU, true, kSplit>;
+    kernel = cross ? philox_shift_kernel_5<V, kU, true, kSplit> : philox_shift_kernel_5<V, kU, false, kSplit>;
   } else {
-    k_same = philox_shift_kernel<V, kU, false, kSplit>;
-    k_cross = philox_shift_kernel<V, kU, true, kSplit>;
+    kernel = cross ? philox_shift_kernel<V, kU, true, kSplit> : philox_shift_kernel<V, kU, false, kSplit>;
   }
   static std::atomic<int> occ[2] = {{0}, {0}};
-  int o = occ[0].load(std::memory_order_relaxed);
-  if (o == 0) {
-    o = blocks_per_sm(k_same);
-    occ[0].store(o, std::memory_order_relaxed);
-    occ[1].store(blocks_per_sm(k_cross), std::memory_order_relaxed);
-  }
+  const int o = resident_ctas(occ[cross ? 1 : 0], kernel);
   const int64_t warps = (p.chunks + kU - 1) / kU;
   int64_t grid = (warps + (kThreads / 32) - 1) / (kThreads / 32);
   if (grid < 1) grid = 1;
   const int64_t cap = (int64_t)sms * ctas_cap(o, geom);
   if (grid > cap) grid = cap;
-  // blocks touched: below (chunks + kU * warps in flight) * kPer + 32 past base
-  const uint64_t reach =
-      (uint64_t)(p.chunks + (int64_t)kU * grid * (kThreads / 32) + 1) * (uint64_t)kPer + 64u;
-  const bool cross = p.ctr.x0 + reach >= kPhiloxMaxBlocks;
-  if (cross) {
-    const int64_t cap2 = (int64_t)sms * ctas_cap(occ[1].load(std::memory_order_relaxed), geom);
-    if (grid > cap2) grid = cap2;
-  }
-  (cross ? k_cross : k_same)<<<(unsigned)grid, kThreads, 0, stream>>>(p);
+  kernel<<<(unsigned)grid, kThreads, 0, stream>>>(p);
 }
 
 // Launches the pieces or the rotate kernel (units inside blocks, output start at
@@ -781,38 +781,25 @@ void launch_pieces(PiecesParams& p, const uint32_t* key, uint64_t off_lo, uint64
   p.ctr = philox_stream(key[0], key[1], (off_lo >> 2) | (off_hi << 62), off_hi >> 2);
   const int64_t blocks = (p.nw - 1 + p.r) / 4 + 1;
   p.chunks = (blocks + 31) / 32;
-  void (*k_same)(const PiecesParams);
-  void (*k_cross)(const PiecesParams);
+  // as in launch_shift
+  const uint64_t reach = (uint64_t)(p.chunks + kU) * 32u + 32u;
+  const bool cross = p.ctr.x0 + reach >= kPhiloxMaxBlocks;
+  void (*kernel)(const PiecesParams);
   if constexpr (kRotate) {
-    k_same = philox_rotate_kernel<V, kU, false>;
-    k_cross = philox_rotate_kernel<V, kU, true>;
+    kernel = cross ? philox_rotate_kernel<V, kU, true> : philox_rotate_kernel<V, kU, false>;
   } else if constexpr (stream_wants_5_ctas<V>()) {
-    k_same = philox_pieces_kernel_5<V, kU, false>;
-    k_cross = philox_pieces_kernel_5<V, kU, true>;
+    kernel = cross ? philox_pieces_kernel_5<V, kU, true> : philox_pieces_kernel_5<V, kU, false>;
   } else {
-    k_same = philox_pieces_kernel<V, kU, false>;
-    k_cross = philox_pieces_kernel<V, kU, true>;
+    kernel = cross ? philox_pieces_kernel<V, kU, true> : philox_pieces_kernel<V, kU, false>;
   }
   static std::atomic<int> occ[2] = {{0}, {0}};
-  int o = occ[0].load(std::memory_order_relaxed);
-  if (o == 0) {
-    o = blocks_per_sm(k_same);
-    occ[0].store(o, std::memory_order_relaxed);
-    occ[1].store(blocks_per_sm(k_cross), std::memory_order_relaxed);
-  }
+  const int o = resident_ctas(occ[cross ? 1 : 0], kernel);
   const int64_t warps = (p.chunks + kU - 1) / kU;
   int64_t grid = (warps + (kThreads / 32) - 1) / (kThreads / 32);
   if (grid < 1) grid = 1;
   const int64_t cap = (int64_t)sms * ctas_cap(o, geom);
   if (grid > cap) grid = cap;
-  // blocks touched: below (chunks + kU * warps in flight) * 32 past base
-  const uint64_t reach = (uint64_t)(p.chunks + (int64_t)kU * grid * (kThreads / 32) + 1) * 32u;
-  const bool cross = p.ctr.x0 + reach >= kPhiloxMaxBlocks;
-  if (cross) {
-    const int64_t cap2 = (int64_t)sms * ctas_cap(occ[1].load(std::memory_order_relaxed), geom);
-    if (grid > cap2) grid = cap2;
-  }
-  (cross ? k_cross : k_same)<<<(unsigned)grid, kThreads, 0, stream>>>(p);
+  kernel<<<(unsigned)grid, kThreads, 0, stream>>>(p);
 }
 
 template <int V>
@@ -868,14 +855,8 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
     } else {
       kernel = cross ? philox_stream_kernel<V, kU, true> : philox_stream_kernel<V, kU, false>;
     }
-    // resident CTAs per SM, found once per kernel (atomic: launches may come
-    // from several host threads)
     static std::atomic<int> occ[2] = {{0}, {0}};
-    int o = occ[cross ? 1 : 0].load(std::memory_order_relaxed);
-    if (o == 0) {
-      o = blocks_per_sm(kernel);
-      occ[cross ? 1 : 0].store(o, std::memory_order_relaxed);
-    }
+    const int o = resident_ctas(occ[cross ? 1 : 0], kernel);
     const int64_t work = (jl - jf + (int64_t)kU - 1) / kU;
     int64_t grid = (work + kThreads - 1) / kThreads;
     if (grid < 1) grid = 1;
@@ -924,11 +905,7 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
     p.sb_hi = r.stride_hi >> 2;
     p.rk = philox_round_keys(r.key[0], r.key[1]);
     static std::atomic<int> occ_cache{0};
-    int occ = occ_cache.load(std::memory_order_relaxed);
-    if (occ == 0) {
-      occ = blocks_per_sm(philox_multi_kernel<V>);
-      occ_cache.store(occ, std::memory_order_relaxed);
-    }
+    const int occ = resident_ctas(occ_cache, philox_multi_kernel<V>);
     int64_t grid = (p.total + kThreads - 1) / kThreads;
     const int64_t cap = (int64_t)sms * ctas_cap(occ, geom);
     if (grid > cap) grid = cap;
@@ -990,11 +967,7 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
     p.stride_hi = r.stride_hi;
     p.rk = philox_round_keys(r.key[0], r.key[1]);
     static std::atomic<int> occ_cache{0};
-    int occ = occ_cache.load(std::memory_order_relaxed);
-    if (occ == 0) {
-      occ = blocks_per_sm(philox_multishift_kernel<V, true>);
-      occ_cache.store(occ, std::memory_order_relaxed);
-    }
+    const int occ = resident_ctas(occ_cache, philox_multishift_kernel<V, true>);
     int64_t grid = (p.total + (kThreads / 32) - 1) / (kThreads / 32);
     const int64_t cap = (int64_t)sms * ctas_cap(occ, geom);
     if (grid > cap) grid = cap;
