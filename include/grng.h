@@ -251,14 +251,14 @@ GRNG_API grng_status grng_generate_host(const grng_distribution* dist, grng_engi
                                grng_stream_t stream);
 
 /* ---------------------------------------------------------- fill geometry
- * Launch geometry of grng_generate / grng_generate_substreams (aligned Philox
- * substreams of 256 groups or more choose their own tiles), one integer
+ * Launch geometry of grng_generate / grng_generate_substreams, one integer
  * per (engine kind, distribution variant, size bucket = bit length of the
  * element count): Philox4x32-10, the CTAs per SM of its grid-stride kernels
  * (1..16: a cap on the resident CTAs; 17..64: value - 16 waves of resident
  * CTAs); MRG32k3a, the threads per SM of the chunk plan in units of 256 (sets
  * the chunk length); 0 = the built-in choice (Philox: 8 waves of resident
- * CTAs; MRG32k3a: 2048 threads per SM, 3072 for long fills).  Tuning is
+ * CTAs, one CTA per tile for aligned substreams of 256 16-byte groups or more;
+ * MRG32k3a: 2048 threads per SM, 3072 for long fills).  Tuning is
  * what the paper expects of kernels written for the hardware (Sec. 8; Sec. 7
  * shows the launch configuration mattering).  Outputs never depend on the
  * geometry.  The table starts from the file named by the environment

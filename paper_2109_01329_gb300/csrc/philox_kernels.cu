@@ -519,14 +519,15 @@ struct MultiTileParams {
   uint32_t groups;    // groups per stream
   uint32_t tile;      // groups per tile
   uint32_t tps;       // tiles per stream
+  uint32_t tiles;     // of all streams
   uint64_t base_lo, base_hi;
   uint64_t sb_lo, sb_hi;  // block-counter stride between streams
   PhiloxRoundKeys rk;
 };
 
 template <int V, int U>
-__device__ __forceinline__ void philox_multi_tile_body(const MultiTileParams& p) {
-  const uint32_t s = blockIdx.x / p.tps, first = (blockIdx.x - s * p.tps) * p.tile;
+__device__ __forceinline__ void philox_multi_tile(const MultiTileParams& p, uint32_t tile) {
+  const uint32_t s = tile / p.tps, first = (tile - s * p.tps) * p.tile;
   uint64_t lo = p.base_lo, hi = p.base_hi;  // block counter of group 0 of stream s
   add128(lo, hi, (uint64_t)s * p.sb_lo, __umul64hi((uint64_t)s, p.sb_lo) + (uint64_t)s * p.sb_hi);
   const uint32_t x0 = (uint32_t)lo;
@@ -556,6 +557,12 @@ __device__ __forceinline__ void philox_multi_tile_body(const MultiTileParams& p)
   if constexpr (U > 1)
     for (; j < end; j += kThreads, dst += kThreads)
       *dst = block_outputs<V>(philox_block(x0 + j, up, p.rk), p.t);
+}
+
+// One tile a CTA, or, with a tuned geometry, fewer CTAs that walk the tiles.
+template <int V, int U>
+__device__ __forceinline__ void philox_multi_tile_body(const MultiTileParams& p) {
+  for (uint32_t tile = blockIdx.x; tile < p.tiles; tile += gridDim.x) philox_multi_tile<V, U>(p, tile);
 }
 
 template <int V, int U>
@@ -887,12 +894,20 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
     p.tile = (uint32_t)tile;
     const int64_t tps = (groups + tile - 1) / tile;
     p.tps = (uint32_t)tps;
-    const int64_t grid = tps * r.num_streams;
+    int64_t grid = tps * r.num_streams;
+    p.tiles = (uint32_t)grid;
+    void (*kernel)(const MultiTileParams);
     if constexpr (stream_wants_5_ctas<V>()) {
-      philox_multi_tile_kernel_5<V, kU><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+      kernel = philox_multi_tile_kernel_5<V, kU>;
     } else {
-      philox_multi_tile_kernel<V, kU><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+      kernel = philox_multi_tile_kernel<V, kU>;
     }
+    if (geom != 0) {
+      static std::atomic<int> occ_cache{0};
+      const int64_t cap = (int64_t)sms * ctas_cap(resident_ctas(occ_cache, kernel), geom);
+      if (grid > cap) grid = cap;
+    }
+    kernel<<<(unsigned)grid, kThreads, 0, stream>>>(p);
   } else if (fast && head == 0 && (stream_bytes % 16u) == 0) {
     MultiParams p;
     p.t = r.t;

@@ -568,3 +568,28 @@ def test_philox_multi_shift_long_runs_across_a_carry(g):
         for s in (0, 1, 31, 63):
             got = out[s * n:(s + 1) * n].cpu().numpy().view(np.uint32)
             assert np.array_equal(got, oracle.generate(0, 77, o + s * stride, 0, 0, 0.0, 0.0, n)), (o, s)
+
+
+@pytest.mark.parametrize("var", [VARIANTS[0], VARIANTS[4], VARIANTS[7], VARIANTS[10]], ids=lambda v: v[0])
+def test_tuned_geometry_of_long_substreams_keeps_outputs(g, var):
+    """Fewer CTAs than tiles, each walking several tiles of several streams, one of
+    which carries out of its low block counter word: the built-in geometry's
+    outputs, bit for bit."""
+    _, kind, dtype, p0, p1 = var
+    d = g.Distribution(kind, dtype, p0, p1)
+    n, S, off = 8192 * (2 if dtype == 2 else 4), 500, (1 << 34) - 4096 * 4
+
+    def fill(geometry):
+        g.fill_geometry(0, d, n * S, geometry)
+        out = torch.zeros(S * n, dtype=_torch_dtype(dtype), device="cuda")
+        g.generate_substreams(d, g.Engine(0, 77, off), out, n, S, 1 << 40)
+        torch.cuda.synchronize()
+        return out.view(torch.uint8)
+
+    g.tune_reset()
+    try:
+        want = fill(0)
+        for geometry in (1, 2, 17, 64):
+            assert torch.equal(fill(geometry), want), geometry
+    finally:
+        g.tune_reset()

@@ -78,3 +78,24 @@ def test_first_fills_from_two_threads(lib, name):
     [t.join() for t in threads]
     assert status == {"inside": 0, "crossing": 0}
     assert len(_launches(lib)) == 2
+
+
+@pytest.mark.parametrize("n", [1024, 1024 * 2 + 4, 1 << 18])
+@pytest.mark.parametrize("kind, dtype", [(0, 0), (2, 1), (2, 2)])
+def test_tuned_geometry_reaches_long_aligned_substreams(lib, kind, dtype, n):
+    """Substreams long enough for a CTA per tile of a stream: a tuned geometry still
+    caps the CTAs (the recording runtime has 152 SMs of 4 resident CTAs)."""
+    d, e, streams = _dist(kind, dtype), _engine(lib, 0, 0), 16384
+
+    def grid():
+        first = lib.fake_launches()
+        assert lib.grng_generate_substreams(ctypes.byref(d), e, n, streams, 1 << 40, 0, OUT, None) == 0
+        (name, g), = _launches(lib, first)
+        return name, g
+
+    name, built_in = grid()
+    for geometry, ctas in ((1, 152), (3, 3 * 152), (16, 4 * 152), (18, 8 * 152)):
+        assert lib.grng_fill_set_geometry(0, ctypes.byref(d), n * streams, geometry) == 0
+        assert grid() == (name, ctas)
+    assert lib.grng_fill_set_geometry(0, ctypes.byref(d), n * streams, 0) == 0
+    assert grid() == (name, built_in)
