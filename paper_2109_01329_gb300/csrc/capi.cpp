@@ -326,6 +326,7 @@ grng_status fill(const grng_distribution* dist, grng_engine* e, int64_t n, int64
   r.engine_kind = e->kind;
   r.n = n;
   r.num_streams = num_streams;
+  r.asked = n * num_streams;
   r.off_lo = e->off_lo;
   r.off_hi = e->off_hi;
   r.stride_lo = stride_lo;

@@ -91,6 +91,7 @@ struct FillRequest {
   int engine_kind;
   int64_t n;
   int64_t num_streams;
+  int64_t asked;       // elements of the whole call, whose size picks the geometry
   uint64_t off_lo, off_hi;
   uint64_t stride_lo, stride_hi;
   void* out;

@@ -360,7 +360,7 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
   // for long fills (several waves, so that an SM refills as its CTAs finish:
   // 10^9 FP64 gaussians 6.67 ms, with 2048 6.78), 1536 for middling ones of the
   // shorter transforms (10^8 bits 96 us, with 2048 99), 2048 below.
-  const int32_t geom = fill_geometry(GRNG_MRG32K3A, V, r.n * r.num_streams);
+  const int32_t geom = fill_geometry(GRNG_MRG32K3A, V, r.asked);
   const int64_t span = p.units + p.head_units;
   const int64_t words = span * I::wpu * r.num_streams;
   const int64_t per_sm = geom > 0                                              ? 256 * (int64_t)geom

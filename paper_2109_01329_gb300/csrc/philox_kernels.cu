@@ -815,7 +815,7 @@ grng_status launch_variant(const FillRequest& r, cudaStream_t stream) {
   constexpr int kEpg = 16 / I::es;
   int dev = 0;
   const int sms = current_device_sms(&dev);
-  const int32_t geom = fill_geometry(GRNG_PHILOX4X32X10, V, r.n * r.num_streams);
+  const int32_t geom = fill_geometry(GRNG_PHILOX4X32X10, V, r.asked);
   const uintptr_t addr = (uintptr_t)r.out;
   const uint32_t phase_w = (uint32_t)((addr & 15u) / 4u);  // output words before out in group 0
   const uint64_t stream_bytes = (uint64_t)r.n * I::es;
@@ -1023,7 +1023,7 @@ grng_status launch_by_variant(const FillRequest& r, cudaStream_t stream) {
 
 // A single-stream fill counts its blocks in 32 bits: a longer one is launched
 // in pieces of 2^32 elements (at most 2^31 blocks), each a fill of its own at
-// its own word offset.
+// its own word offset, with the geometry of the whole.
 grng_status launch_philox(const FillRequest& r, CUstream_st* stream) {
   constexpr int64_t kPiece = int64_t(1) << 32;
   if (r.num_streams != 1 || r.n <= kPiece) return launch_by_variant(r, stream);

@@ -99,3 +99,14 @@ def test_tuned_geometry_reaches_long_aligned_substreams(lib, kind, dtype, n):
         assert grid() == (name, ctas)
     assert lib.grng_fill_set_geometry(0, ctypes.byref(d), n * streams, 0) == 0
     assert grid() == (name, built_in)
+
+
+@pytest.mark.parametrize("phase", [0, 1, 2])
+def test_pieces_of_a_long_fill_take_its_geometry(lib, phase):
+    """A fill launched in pieces of 2^32 elements has one geometry, that of its own
+    size: the aligned, the shift and the pieces kernel."""
+    d, n = _dist(2, 1), (1 << 33) + (1 << 30)
+    assert lib.grng_fill_set_geometry(0, ctypes.byref(d), n, 1) == 0
+    assert lib.grng_generate(ctypes.byref(d), _engine(lib, 0, phase), n, OUT, None) == 0
+    launches = _launches(lib)
+    assert len(launches) == 3 and [g for _, g in launches] == [152] * 3
