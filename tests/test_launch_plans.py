@@ -23,8 +23,9 @@ def lib(tmp_path):
     if not all(os.path.exists(o) for o in objs):
         build.build(force=True)
     path = str(tmp_path / "libgrng_fake.so")
-    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-pthread", os.path.join(HERE, "fake_cudart.cpp"),
-                    *objs, "-o", path], check=True, timeout=300)
+    # bound to itself: the runtime that torch loads has the same names
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-pthread",
+                    os.path.join(HERE, "fake_cudart.cpp"), *objs, "-o", path], check=True, timeout=300)
     L = ctypes.CDLL(path)
     for name in ("grng_generate", "grng_generate_substreams", "grng_engine_create", "grng_fill_set_geometry"):
         f, g = getattr(L, name), getattr(_binding.load(), name)
