@@ -331,7 +331,10 @@ GRNG_API grng_status grng_batch_create(grng_batch_t* out, const grng_request* re
 
 /* Enqueues the fill kernel on `stream`, which counts its launches in the
  * workspace so that the next one continues each sequence: no host
- * synchronisation, no allocation; may be captured into a CUDA graph. */
+ * synchronisation, no allocation; may be captured into a CUDA graph.
+ * A batch's launches belong in one order (one stream, or streams ordered by
+ * events).  Launches that overlap all the same write each other's outputs, of
+ * either place in the sequences; those after them continue past all of them. */
 GRNG_API grng_status grng_batch_launch(grng_batch_t batch, grng_stream_t stream);
 
 /* The autotuner of the batched fill (Sec. 8 names tuning as the cost of

@@ -8,8 +8,8 @@
 // advances per launch.  The tables live in a caller-provided device
 // workspace.  grng_batch_launch then enqueues one kernel: CTAs walk the tiles (a
 // tile is kThreads * ipt 16-byte groups of one request) with a static grid
-// stride, up to eight at a time, and the last CTA to finish counts the launch in the
-// workspace.  A request's offset is its start plus that count times its
+// stride, up to eight at a time, and count the launch in the workspace as they
+// finish.  A request's offset is its start plus the launches so far times its
 // advance, so launching again (or replaying a CUDA graph of the launch)
 // continues every generator's sequence with no host work.  grng_batch_commit
 // reads the count and moves the engines.
@@ -39,14 +39,8 @@ using namespace dev;
 constexpr int kThreads = 256;
 
 // Workspace layout (each part 256-byte aligned):
-//   BatchReq reqs[count] | uint64_t off[count][2] | BatchCount | int32_t tile_req[tiles]
+//   BatchReq reqs[count] | uint64_t off[count][2] | uint64_t arrivals | int32_t tile_req[tiles]
 size_t align256(size_t x) { return (x + 255u) & ~(size_t)255u; }
-
-// Launches of a batch so far, and the CTAs of the running one that are done.
-struct BatchCount {
-  uint64_t launches;
-  uint32_t done;
-};
 
 // Stores the elements of group (first element e0) that lie in [0, n).
 template <int V>
@@ -330,8 +324,12 @@ __global__ void __launch_bounds__(kThreads, 4) batch_fill_kernel(const BatchReq*
                                                               const uint64_t* __restrict__ off,
                                                               const int32_t* __restrict__ tile_req,
                                                               int64_t tiles, int ipt, int run,
-                                                              BatchCount* count, bool advance) {
-  const uint64_t launches = count != nullptr ? count->launches : 0;
+                                                              uint64_t* arrivals, bool advance) {
+  uint64_t launches = 0;
+  if (arrivals != nullptr) {
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(launches) : "l"(arrivals) : "memory");
+    launches >>= kArrivalBits;
+  }
   // a CTA takes `run` consecutive tiles at a time; those of one request are
   // one longer tile, so that a request's set-up is shared
   for (int64_t t0 = (int64_t)blockIdx.x * run; t0 < tiles; t0 += (int64_t)gridDim.x * run) {
@@ -376,15 +374,12 @@ __global__ void __launch_bounds__(kThreads, 4) batch_fill_kernel(const BatchReq*
       }
     }
   }
-  // every thread of the grid has read the launch count by the time the last
-  // CTA arrives: it counts this launch (a kernel of its own for the offsets took
-  // 2.5 us a launch)
-  if (count != nullptr && advance) {
+  // every thread of this CTA has read the launch count: it arrives (a kernel of
+  // its own for the offsets took 2.5 us a launch)
+  if (arrivals != nullptr && advance) {
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&count->done, 1u) == gridDim.x - 1) {
-      count->done = 0;
-      count->launches = launches + 1;
-    }
+    if (threadIdx.x == 0)
+      atomicAdd((unsigned long long*)arrivals, (unsigned long long)batch_arrival(blockIdx.x, gridDim.x));
   }
 }
 
@@ -400,13 +395,14 @@ static int run_of(int64_t tiles) {
 }
 
 static void launch_tiles(const BatchReq* reqs, const uint64_t* offs, const int32_t* tile_req,
-                         int64_t tiles, int ipt, bool heavy, int64_t grid, BatchCount* count,
+                         int64_t tiles, int ipt, bool heavy, int64_t grid, uint64_t* arrivals,
                          bool advance, cudaStream_t stream) {
   const int run = run_of(tiles);
   if (grid > (tiles + run - 1) / run) grid = (tiles + run - 1) / run;
   if (grid < 1) grid = 1;
+  if (grid > (int64_t(1) << kArrivalBits)) grid = int64_t(1) << kArrivalBits;
   (heavy ? batch_fill_kernel<true> : batch_fill_kernel<false>)<<<(unsigned)grid, kThreads, 0, stream>>>(
-      reqs, offs, tile_req, tiles, ipt, run, count, advance);
+      reqs, offs, tile_req, tiles, ipt, run, arrivals, advance);
 }
 
 int64_t plan_parts(const PartDesc* parts, int32_t count, int ipt, BatchReq* reqs_out,
@@ -539,7 +535,7 @@ grng_status grng_batch_workspace_bytes(const grng_request* reqs, int32_t count, 
   grng_status st = plan_sizes(reqs, count, ipt, &tiles, &groups, &heads, &variants, &tps);
   if (st != GRNG_OK) return st;
   *bytes = align256(sizeof(BatchReq) * (size_t)count) + align256(16u * (size_t)count) +
-           align256(sizeof(BatchCount)) + align256(4u * (size_t)(tiles > 0 ? tiles : 1));
+           align256(sizeof(uint64_t)) + align256(4u * (size_t)(tiles > 0 ? tiles : 1));
   return GRNG_OK;
 }
 
@@ -581,7 +577,7 @@ grng_status grng_batch_create(grng_batch_t* out, const grng_request* reqs, int32
   b->reqs_off = 0;
   b->offs_off = align256(sizeof(BatchReq) * (size_t)count);
   b->count_off = b->offs_off + align256(16u * (size_t)count);
-  b->tiles_off = b->count_off + align256(sizeof(BatchCount));
+  b->tiles_off = b->count_off + align256(sizeof(uint64_t));
   b->groups_total = 0;
 
   // Requests of one engine follow each other in its sequence, in table order.
@@ -662,7 +658,7 @@ grng_status grng_batch_create(grng_batch_t* out, const grng_request* reqs, int32
     err = cudaMemcpyAsync(ws + b->offs_off, offs.data(), 16u * (size_t)count,
                           cudaMemcpyHostToDevice, (cudaStream_t)stream);
   if (err == cudaSuccess)
-    err = cudaMemsetAsync(ws + b->count_off, 0, sizeof(BatchCount), (cudaStream_t)stream);
+    err = cudaMemsetAsync(ws + b->count_off, 0, sizeof(uint64_t), (cudaStream_t)stream);
   if (err == cudaSuccess && tiles > 0)
     err = cudaMemcpyAsync(ws + b->tiles_off, tile_req.data(), 4u * (size_t)tiles,
                           cudaMemcpyHostToDevice, (cudaStream_t)stream);
@@ -757,7 +753,7 @@ static grng_status batch_enqueue(grng_batch_t b, cudaStream_t stream, bool advan
   const int32_t* tile_req = reinterpret_cast<const int32_t*>(ws + b->tiles_off);
   if (b->tiles > 0)
     launch_tiles(reqs, offs, tile_req, b->tiles, b->ipt, b->heavy, (int64_t)b->sms * b->ctas_per_sm,
-                 reinterpret_cast<BatchCount*>(ws + b->count_off), advance, stream);
+                 reinterpret_cast<uint64_t*>(ws + b->count_off), advance, stream);
   const cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) {
     set_error("batch launch failed: %s", cudaGetErrorString(err));
@@ -835,9 +831,9 @@ grng_status grng_batch_commit(grng_batch_t b, grng_stream_t stream) {
     set_error("batch is NULL");
     return GRNG_ERR_INVALID_ARG;
   }
-  BatchCount done;
+  uint64_t arrivals = 0;
   const char* ws = reinterpret_cast<const char*>(b->workspace);
-  cudaError_t err = cudaMemcpyAsync(&done, ws + b->count_off, sizeof(done), cudaMemcpyDeviceToHost,
+  cudaError_t err = cudaMemcpyAsync(&arrivals, ws + b->count_off, sizeof(arrivals), cudaMemcpyDeviceToHost,
                                     (cudaStream_t)stream);
   if (err == cudaSuccess) err = cudaStreamSynchronize((cudaStream_t)stream);
   if (err != cudaSuccess) {
@@ -854,7 +850,7 @@ grng_status grng_batch_commit(grng_batch_t b, grng_stream_t stream) {
     const BatchReq& r = b->host_reqs[i];
     const unsigned __int128 at =
         (((unsigned __int128)b->start_hi[i] << 64) | b->start_lo[i]) +
-        (((unsigned __int128)r.adv_hi << 64) | r.adv_lo) * done.launches;
+        (((unsigned __int128)r.adv_hi << 64) | r.adv_lo) * (arrivals >> kArrivalBits);
     const unsigned __int128 skip = at - (((unsigned __int128)es.offset_hi << 64) | es.offset_lo);
     const uint64_t d_lo = (uint64_t)skip, d_hi = (uint64_t)(skip >> 64);
     grng_engine_skip_ahead(b->engines[i], d_lo, d_hi);

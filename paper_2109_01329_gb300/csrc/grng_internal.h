@@ -113,6 +113,19 @@ struct BatchReq {
   int32_t head;        // elements of group 0 before out
 };
 
+// A batch's launches so far in one 64-bit counter: each CTA of a launch adds its
+// arrival when it is done, and the arrivals of a launch add up to 2^20 whatever its
+// grid, below that until the last.  So the counter's upper bits are the launches
+// that are over, the same for every CTA of a launch that runs alone, and launches
+// of one batch that overlap leave it at their number once they are all over.
+constexpr int kArrivalBits = 20;  // CTAs of a launch: at most 2^20
+#if defined(__CUDACC__)
+__host__ __device__
+#endif
+inline uint64_t batch_arrival(uint32_t cta, uint32_t ctas) {
+  return cta == 0 ? (uint64_t(1) << kArrivalBits) - (ctas - 1) : 1u;
+}
+
 // A Philox fill described for plan_parts: key, starting word offset,
 // distribution (variant + parameters), size and device output address.
 struct PartDesc {

@@ -287,3 +287,39 @@ def test_every_phase_at_the_edges_of_tiles_and_chunks(g, kind, dtype):
             n = ref.numel()
             assert torch.equal(buf[lead:lead + n].clone().view(torch.uint8), ref.view(torch.uint8)), (n, e.offset, lead)
             assert not buf[:lead].any() and not buf[lead + n:].any(), (n, e.offset, lead)
+
+
+def test_launches_after_overlapping_ones_continue_past_all(g):
+    """Launches of one batch left to overlap on two streams, with unequal grids
+    between: those after them still give the per-request calls' outputs at the
+    launches' number of advances, and commit moves the engines by all of them."""
+    dists = [(0, 0), (1, 1), (2, 1), (1, 2)]
+    reqs, refs = [], []
+    for i, (kind, dtype) in enumerate(dists * 6):
+        n = (1003, 70_001, 1 << 18)[i % 3]
+        d = g.Distribution(kind, dtype, 0.0, 1.0 if kind else 0.0)
+        reqs.append((g.Engine(0, i, 5 * i), d, torch.empty(n, dtype=TDT[dtype], device="cuda")))
+        refs.append(g.Engine(0, i, 5 * i))
+    b = g.Batch(reqs)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    total = 0
+    for ctas in (32, 1, 4):
+        b.set_config(8, ctas)
+        torch.cuda.synchronize()
+        for _ in range(20):
+            for s in streams:
+                b.launch(stream=s)
+                total += 1
+        torch.cuda.synchronize()
+        b.launch()
+        total += 1
+        torch.cuda.synchronize()
+        for i, ((_, d, out), start) in enumerate(zip(reqs, refs)):
+            e = start.copy()
+            e.skip_ahead((total - 1) * g.words_for(d, out.numel()))
+            want = torch.empty_like(out)
+            g.generate(d, e, want)
+            assert torch.equal(out.view(torch.uint8), want.view(torch.uint8)), (ctas, i)
+    b.commit()
+    for (e, d, out), start in zip(reqs, refs):
+        assert e.offset == start.offset + total * g.words_for(d, out.numel())
