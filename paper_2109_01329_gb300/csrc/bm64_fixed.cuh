@@ -49,20 +49,20 @@
 namespace grng {
 namespace bm64 {
 
-// (sin, cos) and (ln c_i, c_i) are interleaved so that each lookup is one
-// 16-byte load.
+// (sin, cos), (ln c_i, c_i) and the two parts of e ln 2 are interleaved so that
+// each lookup is one 16-byte load.
 struct U64Pair {
   uint64_t a, b;
 };
 #if defined(__CUDACC__)
 __device__ const ulonglong2 d_sc[GRNG_BM64_SINT_LEN] = GRNG_BM64_SC;
 __device__ const ulonglong2 d_lt[GRNG_BM64_LOGT_LEN] = GRNG_BM64_LT;
-__device__ const uint64_t d_e57[GRNG_BM64_E57_LEN] = GRNG_BM64_E57;
+__device__ const ulonglong2 d_ln2[GRNG_BM64_LN2_LEN] = GRNG_BM64_LN2;
 __device__ const uint64_t d_exp2t[GRNG_BM64_EXP2T_LEN] = GRNG_BM64_EXP2T;
 #endif
 static const U64Pair h_sc[GRNG_BM64_SINT_LEN] = GRNG_BM64_SC;
 static const U64Pair h_lt[GRNG_BM64_LOGT_LEN] = GRNG_BM64_LT;
-static const uint64_t h_e57[GRNG_BM64_E57_LEN] = GRNG_BM64_E57;
+static const U64Pair h_ln2[GRNG_BM64_LN2_LEN] = GRNG_BM64_LN2;
 static const uint64_t h_exp2t[GRNG_BM64_EXP2T_LEN] = GRNG_BM64_EXP2T;
 
 #if defined(__CUDA_ARCH__)
@@ -70,7 +70,6 @@ static const uint64_t h_exp2t[GRNG_BM64_EXP2T_LEN] = GRNG_BM64_EXP2T;
 #else
 #define GRNG_BM_TABLE(d, h, i) h[i]
 #endif
-GRNG_BM_HD uint64_t e57(uint32_t e) { return GRNG_BM_TABLE(d_e57, h_e57, e); }
 GRNG_BM_HD uint64_t exp2t(uint32_t j) { return GRNG_BM_TABLE(d_exp2t, h_exp2t, j); }
 #undef GRNG_BM_TABLE
 // sin and cos of 2 pi j / 8192 (2^63 scale)
@@ -84,7 +83,7 @@ GRNG_BM_HD void sincos_tab(uint32_t j, uint64_t& s, uint64_t& c) {
   c = h_sc[j].b;
 #endif
 }
-// ln c_i 2^63 and c_i 2^24
+// ln c_i 2^64 and c_i 2^24
 GRNG_BM_HD void log_tab(uint32_t i, uint64_t& t, uint32_t& c) {
 #if defined(__CUDA_ARCH__)
   const ulonglong2 v = __ldg(&d_lt[i]);
@@ -93,6 +92,18 @@ GRNG_BM_HD void log_tab(uint32_t i, uint64_t& t, uint32_t& c) {
 #else
   t = h_lt[i].a;
   c = (uint32_t)h_lt[i].b;
+#endif
+}
+
+// e ln 2 in units of 2^-57 and the next 32 bits
+GRNG_BM_HD void ln2_tab(uint32_t e, uint64_t& t, uint32_t& f) {
+#if defined(__CUDA_ARCH__)
+  const ulonglong2 v = __ldg(&d_ln2[e]);
+  t = v.x;
+  f = (uint32_t)v.y;
+#else
+  t = h_ln2[e].a;
+  f = (uint32_t)h_ln2[e].b;
 #endif
 }
 
@@ -189,6 +200,23 @@ GRNG_BM_HD uint32_t shr_lo(uint32_t lo, uint32_t hi, uint32_t s) {
 #endif
 }
 
+// (a2:a1:a0) + (t:f) as (r2:r1:r0).
+GRNG_BM_HD void add96(uint32_t a2, uint32_t a1, uint32_t a0, uint64_t t, uint32_t f, uint32_t& r2,
+                      uint32_t& r1, uint32_t& r0) {
+  const uint32_t th = (uint32_t)(t >> 32), tl = (uint32_t)t;
+#if defined(__CUDA_ARCH__)
+  asm("add.cc.u32 %0, %3, %6; addc.cc.u32 %1, %4, %7; addc.u32 %2, %5, %8;"
+      : "=&r"(r0), "=&r"(r1), "=r"(r2)
+      : "r"(a0), "r"(a1), "r"(a2), "r"(f), "r"(tl), "r"(th));
+#else
+  const uint64_t s0 = (uint64_t)a0 + f;
+  const uint64_t s1 = (uint64_t)a1 + tl + (s0 >> 32);
+  r0 = (uint32_t)s0;
+  r1 = (uint32_t)s1;
+  r2 = a2 + th + (uint32_t)(s1 >> 32);
+#endif
+}
+
 GRNG_BM_HD uint64_t join(uint32_t hi, uint32_t lo) { return ((uint64_t)hi << 32) | lo; }
 
 GRNG_BM_HD float fma32(float a, float b, float c) {
@@ -250,42 +278,46 @@ GRNG_BM_HD void neg2_log(uint32_t m0h, uint32_t m0l, uint64_t& X, int& E) {
     M = join(shl_hi(m0l, m0h, e), m0l << e);
   }
   const uint32_t i = (uint32_t)((0ull - M) >> 54);  // delta 2^10, 0..512
-  uint64_t Ti;                              // ln c_i 2^63
+  uint64_t Ti;                              // ln c_i 2^64
   uint32_t C;                               // c_i 2^24
   log_tab(i, Ti, C);
-  // r 2^63 = 2^63 - M C 2^-25 (truncating M C 2^-25 leaves r >= 0); the
-  // 96-bit product M C is exact, and M C 2^-25 = (hi << 7) | (lo32 >> 25)
+  // r 2^64 = 2^64 - M C 2^-24 (truncating M C 2^-24 leaves r >= 0); the
+  // 96-bit product M C is exact, and M C 2^-24 = (hi << 8) | (lo32 >> 24)
   uint64_t mc_hi;
   uint32_t mc_lo;
   mul64x32(M, C, mc_hi, mc_lo);
-  const uint64_t R = (1ull << 63) - ((mc_hi << 7) | (uint64_t)(mc_lo >> 25));  // < 2^54
-  // -ln(1 - r) 2^63 = R + R^2/2 + T3 + T4 + T5 + T6 (r^7/7 < 2^-65.8), R^2/2
-  // being the high word of R^2.  With r32 = r 2^41, r^3 comes from 32-bit high
-  // products: q = r^2 2^50, t = r^3 2^59.
-  const uint32_t r32 = (uint32_t)(R >> 22);
+  const uint64_t R = 0ull - ((mc_hi << 8) | (uint64_t)(mc_lo >> 24));  // < 2^55
+  // -ln(1 - r) 2^64 = R + R^2/2 + T3 + T4 + T5 + T6 (r^7/7 < 2^-65.8).
+  // With r32 = r 2^41, r^3 comes from 32-bit high products: q = r^2 2^50,
+  // t = r^3 2^59.
+  const uint32_t r32 = (uint32_t)(R >> 23);
   const uint32_t q = mulh(r32, r32);
   const uint32_t t = mulh(q, r32);
-  const uint64_t T3 = mulw(t, 0xAAAAAAABu) >> 29;              // t 2^4 / 3
-  // r^4/4 + r^5/5 + r^6/6 stay below 2^25 units of 2^-63, so FP32 is exact
-  // enough (error about 2 units) and keeps them off the integer multiplier,
-  // the busiest pipe: with x = r 2^9 < 1, 2^63 (r^4/4 + r^5/5 + r^6/6) =
-  // x^4 (2^25 + x (2^18/5 + x 2^9/6))
+  const uint64_t T3 = mulw(t, 0xAAAAAAABu) >> 28;              // t 2^5 / 3
+  // r^4/4 + r^5/5 + r^6/6 stay below 2^26 units of 2^-64, so FP32 is exact
+  // enough (error about 4 units) and keeps them off the integer multiplier,
+  // the busiest pipe: with x = r 2^9 < 1, 2^64 (r^4/4 + r^5/5 + r^6/6) =
+  // x^4 (2^26 + x (2^19/5 + x 2^10/6))
   const float x = u32_to_f32(r32) * 0x1p-32f;
   const float x2 = x * x;
   const uint32_t T456 =
-      f32_to_u32_rn(x2 * x2 * fma32(x, fma32(x, 85.333333f, 52428.8f), 33554432.0f));
-  // -ln(1 - delta) 2^63 = ln c_i 2^63 + S < ln 2 2^63 + 2^54; with e >= 1 the
-  // sum e ln 2 + ... is kept in units of 2^-57 (below 37 2^57 < 2^63)
-  const uint64_t S = Ti + R + sqr_hi(R) + T3 + T456;
-  const uint32_t sh = e != 0 ? 6u : 0u;
+      f32_to_u32_rn(x2 * x2 * fma32(x, fma32(x, 170.66667f, 104857.6f), 67108864.0f));
+  // -ln(1 - delta) 2^64 = S < ln 2 2^64 + 2^55.  -ln u1, all of S's bits kept, as
+  // a 96-bit A: in units of 2^-95 for e = 0, of 2^-89 with e ln 2 added else
+  // (below 37 2^89 < 2^95)
+  const uint64_t S = Ti + R + (sqr_hi(R) >> 1) + T3 + T456;
+  const uint32_t sh = e != 0 ? 7u : 1u;
   const uint32_t Sh = (uint32_t)(S >> 32), Sl = (uint32_t)S;
-  const uint64_t Lf = e57(e) + join(Sh >> sh, shr_lo(Sl, Sh, sh));
-  // Lf >= 2^53 (-ln u1 >= ln c_1 > 2^-10 here), so its high word is not 0;
-  // an even shift leaves its top bit at bit 63 or 62 and E even
-  const uint32_t Lh = (uint32_t)(Lf >> 32), Ll = (uint32_t)Lf;
-  const uint32_t n = clz32(Lh) & 30u;       // 0..10 (Lh >= 2^21)
-  X = join(shl_hi(Ll, Lh, n), Ll << n);
-  E = (int)sh - 62 - (int)n;
+  uint64_t Lt;
+  uint32_t Lf;
+  ln2_tab(e, Lt, Lf);
+  uint32_t A2, A1, A0;
+  add96(Sh >> sh, shr_lo(Sl, Sh, sh), shr_lo(0u, Sl, sh), Lt, Lf, A2, A1, A0);
+  // -ln u1 >= ln c_1 > 2^-10 here, so A2 >= 2^21; an even shift leaves the top bit
+  // at bit 63 or 62 and E even
+  const uint32_t n = clz32(A2) & 30u;       // 0..10
+  X = join(shl_hi(A1, A2, n), shl_hi(A0, A1, n));
+  E = (int)sh - 63 - (int)n;
 }
 
 // sqrt(X 2^E), E even and X in [2^62, 2^64), as sq 2^se, sq in [2^61, 2^62].
@@ -333,7 +365,6 @@ GRNG_BM_HD void sincos_turns(uint32_t wa, uint32_t wb, uint64_t& c_abs, uint32_t
   const uint32_t j = (uint32_t)(t >> 51);           // 0..1024
   // phi 2^64 = 2 pi h 2^11 < 2^53.7, h the low 40 bits of t
   const uint64_t P = umulhi_apx((t & ((1ull << 51) - 1)) << 3, k2Pi61);
-  // phi 2^64 = 2 pi h 2^11 < 2^53.7
   const uint64_t P2 = sqr_hi(P);                    // phi^2 2^64 < 2^43.4
   const uint32_t a = (uint32_t)(P2 >> 12);          // phi^2 2^52
   const uint32_t b = (uint32_t)(P >> 22);           // phi 2^42

@@ -1,9 +1,11 @@
 """The parts of the CUDA path's headers that compile for the host too, built with
 g++ and checked without a GPU."""
 
+import ctypes
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -68,3 +70,51 @@ int main() {
 """)
     r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout
+
+
+@pytest.fixture(scope="module")
+def bm64(tmp_path_factory):
+    """neg2_log and the square root after it, of the FP64 fixed-point transforms."""
+    lib = ctypes.CDLL(_build(tmp_path_factory.mktemp("bm64"), """
+#include "bm64_fixed.cuh"
+using namespace grng::bm64;
+// for u1 = m 2^-53: -2 ln u1 = X 2^E and its root s 2^k
+extern "C" void rho(int n, const uint64_t* m, uint64_t* X, int* E, uint64_t* s, int* k) {
+  for (int i = 0; i < n; ++i) {
+    neg2_log((uint32_t)(m[i] >> 21), (uint32_t)(m[i] << 11), X[i], E[i]);
+    sqrt_fixed(X[i], E[i], s[i], k[i]);
+  }
+}
+""", "-shared", "-fPIC"))
+
+    def rho(m):
+        m = np.ascontiguousarray(m, dtype=np.uint64)
+        X, s = np.empty_like(m), np.empty_like(m)
+        E, k = np.empty(m.size, np.int32), np.empty(m.size, np.int32)
+        lib.rho(m.size, *(a.ctypes.data_as(ctypes.c_void_p) for a in (m, X, E, s, k)))
+        return X, E, s, k
+
+    return rho
+
+
+def test_fp64_logarithm_keeps_64_bit_units(bm64):
+    """-ln u1 for u1 in [1/2, 1) in units of 2^-64, and below 1/2 within 58 of them and
+    what the result holds: the sum's terms truncate by at most that (r^3/3: 5 units
+    of 2^-59 times 32/3; the others 5 more), and e ln 2 adds nothing of its size."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.prec = 160
+    r = np.random.Generator(np.random.PCG64(64))
+    top = 1 << 53
+    band = r.integers(top - (top >> 9), top - (top >> 10), 2000)  # u1 in (1 - 2^-9, 1 - 2^-10)
+    X, E, _, _ = bm64(band)
+    # 2 L in units of 2^-63: odd half of the time
+    odd = [(int(x) << (int(e) + 63) if e >= -63 else int(x) >> (-63 - int(e))) & 1 for x, e in zip(X, E)]
+    assert 800 < sum(odd) < 1200
+    worst = 0
+    for e in range(1, 21):
+        m = r.integers(top >> (e + 1), top >> e, 500)
+        X, E, _, _ = bm64(m)
+        for mi, x, ex in zip(m.tolist(), X.tolist(), E.tolist()):
+            worst = max(worst, abs(mp.ldexp(x, ex - 1) + mp.log(mp.ldexp(mi, -53))))
+    # X holds -2 ln u1 < 32 to 2^-58, -ln u1 to half of that
+    assert worst < mp.ldexp(58, -64) + mp.ldexp(1, -59)
