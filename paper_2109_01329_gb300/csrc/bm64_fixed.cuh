@@ -347,7 +347,10 @@ GRNG_BM_HD void sqrt_fixed(uint64_t X, int E, uint64_t& sq, int& se) {
   // (x - s0^2) 2^60 y1 / 2 in 2^-62 units is d (y1 2^30) 2^-29
   const uint64_t s0 = umulhi_apx(X, Y1);
   const int32_t d = (int32_t)((uint32_t)(X >> 4) - (uint32_t)sqr_hi(s0));
-  const int32_t y30 = (int32_t)(uint32_t)(Y1 >> 32);
+  // (y1 rounds to 2 where x is within about 2^-42 above 1/4: y1 2^30 = 2^31 would
+  // change its sign, and one less is as good)
+  const uint32_t yh = (uint32_t)(Y1 >> 32);
+  const int32_t y30 = (int32_t)(yh < 0x7FFFFFFFu ? yh : 0x7FFFFFFFu);
   sq = s0 + (uint64_t)(((int64_t)d * (int64_t)y30) >> 29);
   // sqrt(X 2^E) = sqrt(x) 2^32 2^(E/2) = sq 2^(E/2 - 30)
   se = E / 2 - 30;

@@ -317,3 +317,27 @@ def test_exact_affine_f64_both_forms(g, a, b):
     got = _gpu(g, 1, 2, a, b, words, 2 * len(xs))
     ref = oracle.transform_words(1, 2, a, b, 2 * len(xs), words)
     assert np.array_equal(got.view(np.uint64), ref.view(np.uint64))
+
+
+@pytest.mark.parametrize("kind, sd, tol", [(2, 1.0, 2.0**-50 + 2.0**-52), (4, 1.0, 2.0**-50 + 2.0**-52),
+                                           (3, 0.25, 2.0**-49), (5, 0.25, 2.0**-49)])
+def test_f64_transforms_where_the_root_meets_a_power_of_two(g, kind, sd, tol):
+    """u1 (or the tail probability) on both sides of -2 ln u1 = 4^k, where the fixed-point
+    root's reciprocal rounds to 2: within the stated 2^-50 of max(1, |z|) and the
+    oracle's rounding; the lognormals of a quarter of z < 5 within twice that."""
+    words = []
+    for k in range(-3, 3):
+        u = np.exp(-np.longdouble(4.0) ** k / 2)
+        for d in range(-1500, 1500):
+            m = int(np.floor(u * 2.0**53)) + d
+            if kind in (2, 3):  # u1 = m 2^-53, u2 = 0
+                x = [m - 1, 0]
+                words += [w for v in x for w in ((v << 11) >> 32, (v << 11) & 0xFFFFFFFF)]
+            elif m < 1 << 52:   # p = (2 x + 1) 2^-53 from the 52-bit x
+                words += [((m >> 1) << 12) >> 32, ((m >> 1) << 12) & 0xFFFFFFFF]
+    w = np.array(words, dtype=np.uint32)
+    n = w.size // 2
+    got = _gpu(g, kind, 2, 0.0, sd, w, n)
+    ref = oracle.transform_words(kind, 2, 0.0, sd, n, w)
+    err = np.abs(got - ref) / np.maximum(1.0, np.abs(ref))
+    assert err.max() < tol, (int(np.argmax(err)), float(err.max()))

@@ -118,3 +118,18 @@ def test_fp64_logarithm_keeps_64_bit_units(bm64):
             worst = max(worst, abs(mp.ldexp(x, ex - 1) + mp.log(mp.ldexp(mi, -53))))
     # X holds -2 ln u1 < 32 to 2^-58, -ln u1 to half of that
     assert worst < mp.ldexp(58, -64) + mp.ldexp(1, -59)
+
+
+@pytest.mark.parametrize("k", [-3, -2, -1, 0, 1, 2])
+def test_fp64_root_where_its_reciprocal_rounds_to_two(bm64, k):
+    """rho = sqrt(-2 ln u1) on both sides of -2 ln u1 = 4^k, where x in [1/4, 1) is
+    just above 1/4 and just below 1: within 2^-51, as stated (relative, or absolute
+    below 1)."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.prec = 160
+    m0 = int(mp.floor(mp.ldexp(mp.exp(-mp.ldexp(1, 2 * k) / 2), 53)))
+    m = np.arange(max(1, m0 - 1500), m0 + 1500)
+    _, _, s, e = bm64(m)
+    rho = [mp.sqrt(-2 * mp.log(mp.ldexp(v, -53))) for v in m.tolist()]
+    worst = max(abs(mp.ldexp(int(a), int(b)) - r) / max(1, r) for a, b, r in zip(s, e, rho))
+    assert worst < mp.ldexp(1, -51)
