@@ -389,7 +389,7 @@ GRNG_BM_HD void sincos_turns(uint32_t wa, uint32_t wb, uint64_t& c_abs, uint32_t
   const uint64_t k3 = umulhi_apx(Sj, sphi - eps);
   const uint64_t cs = Cj - k1 - k3;                 // cos(alpha + phi) 2^63 >= 2^62.5
   // sin(alpha + phi) 2^63: the products truncate by at most 2, the table's
-  // sine is 2 up
+  // sine is 2 up at 0 and 8 elsewhere
   const uint64_t sn = Sj + k2 - k1;
   // in Gray code the octant's bits are the swap (octants 1, 2, 5, 6), the
   // cosine's sign (2..5) and the sine's (4..7)
@@ -474,7 +474,11 @@ GRNG_BM_HD FixedPair box_muller_fixed(uint32_t w0, uint32_t w1, uint32_t w2, uin
   int E, se;
   neg2_log((uint32_t)(m0 >> 32), (uint32_t)m0, X, E);
   sqrt_fixed(X, E, sq, se);
-  // z = sq 2^se * c 2^-63 = umulhi(sq, c) 2^(se + 1)
+  // z = sq 2^se * c 2^-63 = umulhi(sq, c) 2^(se + 1).  The root and these products
+  // truncate, by 2.4 units of p on average, and the rounding to even that
+  // follows rounds half of the ties the wrong way for it (rms error at u1 in
+  // 1 - [2^-9, 2^-8] 5.489e-18, with ties away from 0 5.472e-18): so the tables of sine
+  // and cosine stand 8 and 4 units up, 5.460e-18
   r.p0 = umulhi_apx(sq, c_abs);
   r.p1 = umulhi_apx(sq, s_abs);
   r.k = se + 1;

@@ -7,8 +7,9 @@ Tables (emitted as initializer macros: the device and host copies are declared w
   LT[i], i = 0..512:     (ln(c_i) * 2^64, c_i * 2^24) with c_i = floor(2^24 / (1 - i/1024))
                          / 2^24, the reduction factor for -ln(1 - delta) with delta in
                          [i/1024, (i+1)/1024)
-  SC[j], j = 0..1024:    (sin + 2, cos)(2 pi j / 8192) * 2^63, the sine 2 units up so
-                         that the truncating rotation never leaves it below 0
+  SC[j], j = 0..1024:    (sin, cos)(2 pi j / 8192) * 2^63, a few units up: the products
+                         by rho that follow truncate, and the truncating rotation must
+                         not leave a sine below 0
   LN2[e], e = 0..52:     e ln 2 * 2^89, its upper 64 bits and its lowest 32
   kExp2T[j], j = 0..256: 2^(j / 256) * 2^62
 Scalars
@@ -44,8 +45,9 @@ def main():
         logt.append(rnd(mp.log(mp.mpf(c) / two24) * two64))
     assert logc[0] == 1 << 24 and logc[512] == 1 << 25
     assert all(t < 1 << 64 for t in logt)
-    sint = [rnd(mp.sin(2 * mp.pi * j / 8192) * two63) + 2 for j in range(1025)]
-    cost = [rnd(mp.cos(2 * mp.pi * j / 8192) * two63) for j in range(1025)]
+    # sin 0 at most 3 up, so that an exact 0 stays one (rho 2^62 by 3 2^-64 is below 1)
+    sint = [rnd(mp.sin(2 * mp.pi * j / 8192) * two63) + (8 if j else 2) for j in range(1025)]
+    cost = [rnd(mp.cos(2 * mp.pi * j / 8192) * two63) + 4 for j in range(1025)]
     ln2 = [rnd(e * mp.log(2) * mp.mpf(2) ** 89) for e in range(53)]
     assert all(v < 1 << 95 for v in ln2)
     exp2t = [rnd(mp.mpf(2) ** (mp.mpf(j) / 256) * mp.mpf(2) ** 62) for j in range(257)]

@@ -78,6 +78,15 @@ def bm64(tmp_path_factory):
     lib = ctypes.CDLL(_build(tmp_path_factory.mktemp("bm64"), """
 #include "bm64_fixed.cuh"
 using namespace grng::bm64;
+// words of pairs -> |z0|, |z1| = p 2^k
+extern "C" void pairs(int n, const uint32_t* w, uint64_t* p, int* k) {
+  for (int i = 0; i < n; ++i) {
+    const FixedPair f = box_muller_fixed(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+    p[2 * i] = f.p0;
+    p[2 * i + 1] = f.p1;
+    k[i] = f.k;
+  }
+}
 // for u1 = m 2^-53: -2 ln u1 = X 2^E and its root s 2^k
 extern "C" void rho(int n, const uint64_t* m, uint64_t* X, int* E, uint64_t* s, int* k) {
   for (int i = 0; i < n; ++i) {
@@ -87,6 +96,11 @@ extern "C" void rho(int n, const uint64_t* m, uint64_t* X, int* E, uint64_t* s, 
 }
 """, "-shared", "-fPIC"))
 
+    def pairs(w):
+        p, k = np.empty(w.size // 2, np.uint64), np.empty(w.size // 4, np.int32)
+        lib.pairs(w.size // 4, *(a.ctypes.data_as(ctypes.c_void_p) for a in (w, p, k)))
+        return p.reshape(-1, 2), k
+
     def rho(m):
         m = np.ascontiguousarray(m, dtype=np.uint64)
         X, s = np.empty_like(m), np.empty_like(m)
@@ -94,6 +108,7 @@ extern "C" void rho(int n, const uint64_t* m, uint64_t* X, int* E, uint64_t* s, 
         lib.rho(m.size, *(a.ctypes.data_as(ctypes.c_void_p) for a in (m, X, E, s, k)))
         return X, E, s, k
 
+    rho.pairs = pairs
     return rho
 
 
@@ -133,3 +148,18 @@ def test_fp64_root_where_its_reciprocal_rounds_to_two(bm64, k):
     rho = [mp.sqrt(-2 * mp.log(mp.ldexp(v, -53))) for v in m.tolist()]
     worst = max(abs(mp.ldexp(int(a), int(b)) - r) / max(1, r) for a, b, r in zip(s, e, rho))
     assert worst < mp.ldexp(1, -51)
+
+
+def test_fp64_pairs_before_rounding_are_near_the_middle(bm64):
+    """The fixed-point pair ahead of its rounding to even: low by less than 2 of its
+    units on average (a result of rho's own size has 2^8 or more in its last place)."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.prec = 130
+    w = np.random.Generator(np.random.PCG64(65)).integers(0, 1 << 32, 4 * 4000, dtype=np.uint32)
+    p, k = bm64.pairs(w)
+    total = mp.mpf(0)
+    for (a, b, c, d), q, e in zip(w.reshape(-1, 4).tolist(), p.tolist(), k.tolist()):
+        rho = mp.sqrt(-2 * mp.log(mp.ldexp((((a << 32) | b) >> 11) + 1, -53)))
+        turn = mp.ldexp(((c << 32) | d) >> 11, -52)
+        total += q[0] - mp.ldexp(rho * abs(mp.cospi(turn)), -e) + q[1] - mp.ldexp(rho * abs(mp.sinpi(turn)), -e)
+    assert -2 < total / (2 * k.size) < 2
