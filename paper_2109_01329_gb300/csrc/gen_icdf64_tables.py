@@ -9,13 +9,16 @@ segments: width 1/16 for D < 3/4 (12), 1/8 for D < 5/2 (14), 1/4 beyond
 (20).  On each segment t = c0 + c1 s + ... + c8 s^8, s in [0, 1) the
 position inside it; the coefficients are least-squares fits on Chebyshev
 nodes against mpmath at 200 bits (t = sqrt(2) erfinv(1 - 2p)), rounded to
-integers in units of 2^-59.  The fits stay below 1e-17 of max(1, t).
+integers in units of 2^-59.  The fits stay below 1e-17 of max(1, t).  The root
+and Horner's steps that use them truncate, by 3.9 units on average, so c0 stands
+2 units up (rms error of t over p in (0, 1/2): 7.3e-18, 4.9e-18 so).
 """
 
 import mpmath as mp
 
 mp.mp.prec = 200
 DEG = 8
+C0_UP = 2
 W0 = mp.sqrt(2 * mp.log(2))
 WMAX = mp.sqrt(106 * mp.log(2))
 REGIONS = [(mp.mpf(0), mp.mpf("0.75"), mp.mpf(1) / 16),
@@ -46,7 +49,9 @@ def fit(a, h):
         t = t_of_w(a + h * s)
         v = sum(coef[c] * s ** c for c in range(DEG + 1))
         err = max(err, abs(v - t) / max(1, t))
-    return [int(mp.nint(c * mp.mpf(2) ** 59)) for c in coef], err
+    row = [int(mp.nint(c * mp.mpf(2) ** 59)) for c in coef]
+    row[0] += C0_UP
+    return row, err
 
 
 def main():

@@ -163,3 +163,23 @@ def test_fp64_pairs_before_rounding_are_near_the_middle(bm64):
         turn = mp.ldexp(((c << 32) | d) >> 11, -52)
         total += q[0] - mp.ldexp(rho * abs(mp.cospi(turn)), -e) + q[1] - mp.ldexp(rho * abs(mp.sinpi(turn)), -e)
     assert -2 < total / (2 * k.size) < 2
+
+
+def test_fp64_inverse_cdf_before_rounding_is_near_the_middle(tmp_path):
+    """t = -Phi^-1(p) in its units of 2^-59: off by less than 3 on average (the fits
+    stay below 6 of them)."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.prec = 130
+    lib = ctypes.CDLL(_build(tmp_path, """
+#include "icdf64_fixed.cuh"
+extern "C" uint64_t t59(uint64_t m) { return grng::icdf64::neg_icdf(m); }
+""", "-shared", "-fPIC"))
+    lib.t59.argtypes, lib.t59.restype = [ctypes.c_uint64], ctypes.c_uint64
+    total, n = mp.mpf(0), 600
+    for m in np.random.Generator(np.random.PCG64(66)).integers(1, 1 << 51, n).tolist():
+        m = 2 * m + 1
+        t = mp.ldexp(lib.t59(m), -59)
+        # one Newton step from t, which is right to 2^-50: then to 2^-99
+        density = mp.exp(-t * t / 2) / mp.sqrt(2 * mp.pi)
+        total += mp.ldexp((mp.ldexp(m, -53) - mp.erfc(t / mp.sqrt(2)) / 2) / density, 59)
+    assert -3 < total / n < 3
