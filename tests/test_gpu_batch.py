@@ -323,3 +323,40 @@ def test_launches_after_overlapping_ones_continue_past_all(g):
     b.commit()
     for (e, d, out), start in zip(reqs, refs):
         assert e.offset == start.offset + total * g.words_for(d, out.numel())
+
+
+@pytest.mark.parametrize("run", [2, 8])
+@pytest.mark.parametrize("heavy", [False, True])
+def test_merged_tiles_with_carries_splits_and_ragged_ends(g, heavy, run):
+    """Batches of enough tiles that a CTA takes two or eight at a time, those of one
+    request as one: requests that end inside a run, start misaligned, at every word
+    phase, with a Box-Muller pair split by the output's start, and before and
+    across a carry out of the low block counter word equal the per-request calls bit
+    for bit."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    dists = [(0, 0), (1, 1), (2, 1), (3, 1)] + ([(2, 2), (3, 2), (4, 2)] if heavy else [(1, 2), (4, 1)])
+    # tiles of 256 groups: this many of them over the requests below
+    per = (16 * sms * run + 16 * sms // 2) // (2 * len(dists)) + 3
+    reqs, refs, tiles = [], [], 0
+    for i, (kind, dtype) in enumerate(dists * 2):
+        epg = 2 if dtype == 2 else 4
+        n = (per * 256 + 37 * i) * epg + i % 3
+        words = oracle.words_for(kind, dtype, n)
+        off = ((1 << 34) - words // 3 + i, i, (1 << 34) - 2 * words - i)[i % 3] & ~(1 if dtype == 2 and i % 2 else 0)
+        lead = i % 4 if dtype != 2 else i % 2
+        d = g.Distribution(kind, dtype, 0.0, 1.0 if kind else 0.0)
+        buf = torch.zeros(n + 8, dtype=TDT[dtype], device="cuda")
+        reqs.append((g.Engine(0, 100 + i, off), d, buf[lead:lead + n]))
+        refs.append((g.Engine(0, 100 + i, off), buf, lead))
+        tiles += -(-(lead + n) // (256 * epg))
+    assert min(8, tiles // (16 * sms)) == run
+    b = g.Batch(reqs)
+    b.set_config(1, 32)
+    for _ in range(2):
+        b.launch()
+        for (_, d, out), (e, buf, lead) in zip(reqs, refs):
+            want = torch.empty_like(out)
+            g.generate(d, e, want)
+            torch.cuda.synchronize()
+            assert torch.equal(out.clone().view(torch.uint8), want.view(torch.uint8)), (d, lead, out.numel())
+            assert not buf[:lead].any() and not buf[lead + out.numel():].any(), (d, lead)

@@ -593,3 +593,21 @@ def test_tuned_geometry_of_long_substreams_keeps_outputs(g, var):
             assert torch.equal(fill(geometry), want), geometry
     finally:
         g.tune_reset()
+
+
+@pytest.mark.parametrize("var", [VARIANTS[4], VARIANTS[7], VARIANTS[10], VARIANTS[14]], ids=lambda v: v[0])
+def test_pieces_of_a_long_fill_meet(g, var):
+    """The seam of a fill of more than 2^32 outputs, launched in pieces, for two words
+    an output, pairs, pairs of two words each and the inverse CDF: windows across
+    the seam and at the end equal the oracle's, and the engine advances by the whole."""
+    _, kind, dtype, p0, p1 = var
+    n, off = (1 << 32) + 1003, 6
+    words = oracle.words_for(kind, dtype, 2) // 2  # per output
+    out = torch.empty(n, dtype=_torch_dtype(dtype), device="cuda")
+    e = g.Engine(0, 2021, off)
+    g.generate(g.Distribution(kind, dtype, p0, p1), e, out)
+    torch.cuda.synchronize()
+    assert e.offset == off + oracle.words_for(kind, dtype, n)
+    for at, m in (((1 << 32) - 516, 1001), (n - 401, 401)):
+        ref = oracle.generate(0, 2021, off + at * words, kind, dtype, p0, p1, m)
+        assert_parity(kind, dtype, out[at:at + m].cpu().numpy(), ref, f"{var[0]} at {at}")
