@@ -169,13 +169,12 @@ __device__ __forceinline__ void jump(MrgRegs& s, uint64_t e_lo, uint64_t e_hi) {
 
 // Generates one unit's words and writes its kWpu output words to o.
 template <int V>
-__device__ __forceinline__ void gen_unit(MrgRegs& st, uint32_t* o, const MrgParams& p,
-                                         bool odd = false) {
+__device__ __forceinline__ void gen_unit(MrgRegs& st, uint32_t* o, const MrgParams& p) {
   constexpr int kWpu = VInfo<V>::wpu;
   uint32_t w[kWpu];
 #pragma unroll
   for (int i = 0; i < kWpu; ++i) w[i] = mrg_next(st, p);
-  unit_outputs<V>(w, o, p.t, odd);
+  unit_outputs<V>(w, o, p.t);
 }
 
 // The 16-byte group from 4 new output words: as they are, or (carry
