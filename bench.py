@@ -199,12 +199,13 @@ def oracle_rate(seconds_per_case: float, cores: int, n_cap: int):
 
 
 # 32x32 products per output sample, counted from the algorithms as
-# implemented: Philox4x32-10 is 20 products per 4-word block; an MRG32k3a word
-# is 7 (per component two multiplier products, then the folds of 2^32 = c
-# mod m: one 32-bit product for m1, one wide and one 32-bit product for m2);
-# the fixed-point FP64 Box-Muller pair is 35 products (log: 7, square root:
-# 6, sine and cosine: 16, the two final products: 6) on top of the products
-# of its 4 words.
+# implemented: Philox4x32-10 is 18 products per 4-word block of one stream (20,
+# less the two that the fixed upper counter words make once per launch); an
+# MRG32k3a word is 7 (per component two multiplier products, then the folds of
+# 2^32 = c mod m: one 32-bit product for m1, one wide and one 32-bit product
+# for m2); the fixed-point FP64 Box-Muller pair is 35 products (log: 7, square
+# root: 6, sine and cosine: 16, the two final products: 6) on top of the
+# products of its 4 words.
 BM64_PRODUCTS_PER_PAIR = 35
 
 # DRAM bytes (read + write) per launch at n = 10^9 from ncu captures of the
@@ -212,10 +213,10 @@ BM64_PRODUCTS_PER_PAIR = 35
 # a kernel whose code changed after its capture is left out (no number
 # rather than a stale one).
 NCU_TRAFFIC_PER_1E9 = {
-    "mrg32k3a/gaussian_f64": (2.083313e9 + 0.118e6) / 0.268,
-    "philox4x32_10/gaussian_f64": (2.082409e9 + 0.304e6) / 0.268,
-    "philox4x32_10/uniform_f32": (1.010023e9 + 0.042e6) / 0.268,
-    "philox4x32_10/uniform_f64": (2.081978e9 + 0.056e6) / 0.268,
+    "mrg32k3a/gaussian_f64": (2.089137e9 + 0.334e6) / 0.268,
+    "philox4x32_10/gaussian_f64": (2.082362e9 + 0.345e6) / 0.268,
+    "philox4x32_10/uniform_f32": (1.009950e9 + 0.043e6) / 0.268,
+    "philox4x32_10/uniform_f64": (2.082375e9 + 0.330e6) / 0.268,
 }
 
 # The method's own 32x32 -> 64-bit products per sample, independent of how
@@ -250,10 +251,10 @@ def transcendental_ceiling(name: str, ops: dict):
             "CUDA normcdfinvf + expf per sample"
     return None
 PRODUCTS_PER_SAMPLE = {
-    "philox4x32_10/bits_u32": 5, "philox4x32_10/uniform_f32": 5,
-    "philox4x32_10/uniform_f64": 10, "philox4x32_10/gaussian_f32": 5,
-    "philox4x32_10/gaussian_f64": (20 + BM64_PRODUCTS_PER_PAIR) / 2,
-    "philox4x32_10/lognormal_f32": 5,
+    "philox4x32_10/bits_u32": 4.5, "philox4x32_10/uniform_f32": 4.5,
+    "philox4x32_10/uniform_f64": 9, "philox4x32_10/gaussian_f32": 4.5,
+    "philox4x32_10/gaussian_f64": (18 + BM64_PRODUCTS_PER_PAIR) / 2,
+    "philox4x32_10/lognormal_f32": 4.5,
     "mrg32k3a/bits_u32": 7, "mrg32k3a/uniform_f32": 7, "mrg32k3a/uniform_f64": 14,
     "mrg32k3a/gaussian_f32": 7, "mrg32k3a/gaussian_f64": (28 + BM64_PRODUCTS_PER_PAIR) / 2,
     "mrg32k3a/lognormal_f32": 7,
