@@ -199,7 +199,9 @@ def _on_device(index: int, stream, where: str, fn, *args) -> None:
     """fn(*args, stream) with device `index` current, on `stream` or that
     device's current one.  Where the device is current already, as it nearly
     always is, the call goes straight through: the guard and the Stream object of
-    the general way cost 5 us a call, more than the launch."""
+    the general way cost 5 us a call, more than the launch.  (The two torch calls
+    that read the current device and stream without them are not public; 2.9 and
+    2.11 both have them.)"""
     torch = _t()
     if torch._C._cuda_getDevice() == index:
         raw = torch._C._cuda_getCurrentRawStream(index) if stream is None \
@@ -230,7 +232,8 @@ class Distribution:
         return _Dist(self.kind, self.dtype, float(self.p0), float(self.p1))
 
     # the fields are frozen: the C form is made once, at the first call that
-    # takes it (read-only to the library)
+    # takes it (read-only to the library).  A fill of 10^3 takes 4.1 us with a
+    # distribution that is kept, 5.4 with one made for the call
     _cached = None
 
     def _ref(self) -> _Dist:

@@ -319,6 +319,10 @@ __device__ __forceinline__ void batch_tile(const BatchReq& r, uint64_t off_lo, u
 // 858 -> 603 us a launch, 541 with the FP64 add for [-1, 1) and the phases as
 // constants (at 603, five CTAs per SM, 48 registers and 376 bytes spilled:
 // 5 % slower than four).
+// With those transforms (a fifth each FP64 gaussians, lognormals, inverse CDFs, FP32
+// uniforms and gaussians): 4096 requests 3.96 -> 2.90 ms (3.29 at the best geometry
+// before), 1024 of up to 2^18 305 -> 225 us, 16 of up to 2^14 22.7 -> 19.3.  Both kernels
+// stand at the cap of 64 registers.
 template <bool kHeavy>
 __global__ void __launch_bounds__(kThreads, 4) batch_fill_kernel(const BatchReq* __restrict__ reqs,
                                                               const uint64_t* __restrict__ off,

@@ -259,7 +259,8 @@ __device__ __forceinline__ double u01_f64_dadd(uint32_t wa, uint32_t wb) {
   const uint32_t h = wa >> 11;                      // x >> 32: 21 bits
   const uint32_t l = __funnelshift_r(wb, wa, 11);   // low 32 bits of x
   const double B = __hiloint2double((int)((h & 0xFFFFFu) | 0x3FE00000u), (int)l);
-  // 0 or -1/2 by a mask of the top bit (selecting it: 10^9 1.409 ms, 1.383 so)
+  // 0 or -1/2 by a mask of the top bit (selected instead: 10^9 in 1.419 ms both on
+  // Philox, 2.145 ms against 2.156 on MRG32k3a)
   const uint32_t c = ~(uint32_t)((int32_t)wa >> 31) & 0xBFE00000u;
   return __dadd_rn(B, __hiloint2double((int)c, 0));
 }

@@ -79,9 +79,9 @@ __device__ __forceinline__ void store_partial(char* stream_base, int64_t e0, int
 // with 18 products, each one wide multiply, a bits block costs 44 instructions
 // of 55 before, and the contiguous tiles keep a CTA's stores together (grid-
 // strided: bits 0.541 ms).  10^9 outputs, before -> now: bits 0.602 -> 0.531 ms
-// (7.53 TB/s), FP32 uniforms 0.665 -> 0.594, FP64 uniforms 1.650 -> 1.405, FP32
-// gaussians 1.351 -> 1.095 (1.22 with the f32x2 polynomials alone), FP64
-// gaussians 6.26 -> 6.10.
+// (7.53 TB/s), FP32 uniforms 0.665 -> 0.594, FP64 uniforms 1.650 -> 1.41, FP32
+// gaussians 1.351 -> 1.10 (1.22 with the f32x2 polynomials alone), FP64
+// gaussians 6.26 -> 6.10 (5.69 with the pair reworked after it).
 struct StreamParams {
   TransformParams t;
   uint4* gbase;       // 16-byte aligned address of group 0 (may precede out)
@@ -290,13 +290,13 @@ __device__ __forceinline__ void philox_shift_body(const ShiftParams& p) {
 }
 
 // The phase is the same for the whole grid.  Raw bits take one loop per
-// phase, each with the phase a constant (n = 10^9 at phases 1, 2, 3: 0.764,
-// 0.771, 0.796 ms against 0.852, 0.851, 0.915 with the phase a variable).  The
-// FP32 uniforms take the constant form for phases 2 and 3 only: with a
-// constant phase 1 they ran 10 % slower (ncu: 207 against 186 million
-// instructions, the words moved into place one by one where the variable form
-// selects each into place), while phases 2 and 3 gained 4-8 %.  The other
-// variants keep the variable phase.
+// phase, each with the phase a constant (n = 10^9 at phases 1, 2, 3: 0.638,
+// 0.630, 0.640 ms against 0.682, 0.677, 0.746 with the phase a variable).  The
+// FP32 uniforms take the constant form for phases 2 and 3 (0.706, 0.715 ms
+// against 0.761, 0.814).  Their phase 1 keeps the variable form, from loops with
+// 64-bit counters, where the constant one was 10 % slower; in the present ones it
+// would be the faster (0.706 ms against 0.743).  The other variants keep the
+// variable phase.
 template <int V, int U, bool kCross, bool kSplit>
 __device__ __forceinline__ void philox_shift_phases(const ShiftParams& p) {
   if constexpr (V == V_BITS && !kSplit) {
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(kThreads) philox_multi_kernel(const __grid_con
 // in the single-stream kernel (one group at a time with 128-bit counters took
 // 90 instructions a block against 64 there).  16384 x 16384: FP32 uniforms
 // 258 -> 169 us (159 in one stream), bits 230 -> 147, FP64 uniforms 540 -> 402,
-// FP32 gaussians 428 -> 311, FP64 gaussians 1791 -> 1656.
+// FP32 gaussians 428 -> 311, FP64 gaussians 1791 -> 1656 (1560 with the pair reworked).
 struct MultiTileParams {
   TransformParams t;
   uint4* out;
